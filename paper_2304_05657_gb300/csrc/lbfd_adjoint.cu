@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(256) to_rev_kernel(long long n, const S* __res
 // Record: thread t of the launch takes cell c0 + u, u = t % chunk, of the
 // step from the state of slot t / chunk (several steps' tapes are recorded
 // in one launch), and leaves its node count in count[t].
-template <int DIM, typename V>
+template <int DIM, typename V, bool HI1>
 __global__ void __launch_bounds__(REV_BLOCK, 8)
     adjoint_record_kernel(StepParams<RevT<V>> P, const RevStoreT<V>* __restrict__ rin, RevStoreT<V>* __restrict__ rout,
                           const uint8_t* __restrict__ solid, long long c0, long long n, long long chunk,
@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(REV_BLOCK, 8)
         const long long r = c / P.nx;
         p[1] = (int)(r % P.ny);
         p[2] = (int)(r / P.ny);
-        cell_step_general<DIM, RevStoreT<V>, RevT<V>>(P, p, c, in, out, in + (long long)Q * N, out + (long long)Q * N,
+        cell_step_general<DIM, RevStoreT<V>, RevT<V>, true, HI1>(P, p, c, in, out, in + (long long)Q * N, out + (long long)Q * N,
                                               in + (long long)(Q + 1) * N, out + (long long)(Q + 1) * N, solid);
     }
     count[t] = rev_count_dyn[threadIdx.x];
@@ -208,7 +208,6 @@ static StepParams<RevT<V>> rev_params(const StepParams<double>& D)
     for (int k = 0; k < NSP; ++k) {
         P.inv_Wk[k] = Rv(D.inv_Wk[k]);
         P.yield[k] = Rv(D.yield[k]);
-        P.a_diff[k] = Rv(D.a_diff[k]);
         P.a12[k] = Rv(D.a12[k]);
         P.Y_in[k] = Rv(D.Y_in[k]);
     }
@@ -223,13 +222,14 @@ static StepParams<RevT<V>> rev_params(const StepParams<double>& D)
     P.omega_s = Rv(D.omega_s);
     P.omega_b = Rv(D.omega_b);
     P.omega_hi = Rv(D.omega_hi);
-    P.alpha = Rv(D.alpha);
     P.alpha12 = Rv(D.alpha12);
     P.lam_yield = Rv(D.lam_yield);
     P.u_in = Rv(D.u_in, 3);
     P.T_in = Rv(D.T_in);
     P.invW_in = Rv(D.invW_in);
     P.rho_in = Rv(D.rho_in);
+    P.rho_c = Rv(D.rho_c);
+    P.inv_rho_c = Rv(D.inv_rho_c);
     P.T_solid = D.solid_isothermal ? Rv(D.T_solid, 2) : Rv(D.T_solid);
     P.solid_isothermal = D.solid_isothermal;
     P.poiseuille = D.poiseuille;
@@ -278,7 +278,8 @@ static cudaError_t record_steps(const StepParams<double>& Pd, int planes, const 
     // slot (idle ones return at once) so that the interleaved layout has a
     // fixed stride
     const unsigned blocks = (unsigned)((w.slots * w.chunk + REV_BLOCK - 1) / REV_BLOCK);
-    adjoint_record_kernel<2, V><<<blocks, REV_BLOCK, REV_BLOCK * sizeof(int), stream>>>(
+    auto kern = Pd.omega_hi == 1.0 ? adjoint_record_kernel<2, V, true> : adjoint_record_kernel<2, V, false>;
+    kern<<<blocks, REV_BLOCK, REV_BLOCK * sizeof(int), stream>>>(
         P, rin, (RevStoreT<V>*)w.rout, solid, c0, n, w.chunk, nel, w.count);
     return cudaGetLastError();
 }

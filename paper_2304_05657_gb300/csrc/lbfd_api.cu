@@ -151,7 +151,6 @@ void fill_params(const lbfd_handle* h, StepParams<R>& P)
     for (int k = 0; k < lbfd::NSP; ++k) {
         P.inv_Wk[k] = (R)(1.0 / M.W[k]);
         P.yield[k] = (R)(M.nu_stoich[k] * M.W[k] / yF);
-        P.a_diff[k] = (R)(alpha / M.Le[k] * M.W[k]);
         P.a12[k] = (R)(alpha / M.Le[k] / 12.0);
         P.Y_in[k] = (R)p.Y_in[k];
     }
@@ -167,7 +166,6 @@ void fill_params(const lbfd_handle* h, StepParams<R>& P)
     P.omega_s = (R)omega_s;
     P.omega_b = (R)(p.omega_bulk > 0.0 ? p.omega_bulk : omega_s);
     P.omega_hi = (R)p.omega_hi;
-    P.alpha = (R)alpha;
     P.alpha12 = (R)(alpha / 12.0);
     {
         double ly = 0.0;
@@ -177,6 +175,8 @@ void fill_params(const lbfd_handle* h, StepParams<R>& P)
     P.u_in = (R)p.u_in;
     P.T_in = (R)p.T_in;
     P.invW_in = (R)invW_in;
+    P.rho_c = (R)(p.T_in * invW_in);
+    P.inv_rho_c = (R)(1.0 / (p.T_in * invW_in));
     P.rho_in = (R)1.0;  // EOS reference state (T_in, Y_in)
     P.T_solid = (R)p.T_solid;
     P.solid_isothermal = p.solid_isothermal;
@@ -186,8 +186,11 @@ void fill_params(const lbfd_handle* h, StepParams<R>& P)
         P.face_solid[f] = (b == LBFD_BC_WALL_ISOTHERMAL && p.solid_isothermal && G.T_wall[f] == p.T_solid) ||
                           (b == LBFD_BC_WALL_ADIABATIC && !p.solid_isothermal);
     }
-    P.epsY = (R)p.weno_eps;
-    P.epsT = (R)(p.weno_eps * p.T_in * p.T_in);
+    // the WENO3 weights hold eps^2 (FP32) and eps^4 (FP64): kept in range (the
+    // limits lie far below the squared resolution of any field)
+    const double eps_lo = sizeof(R) % 8 ? 1e-18 : 1e-75;
+    P.epsY = (R)std::max(p.weno_eps, eps_lo);
+    P.epsT = (R)std::max(p.weno_eps * p.T_in * p.T_in, eps_lo);
     P.cs = (R)sqrt(cs2);
 }
 

@@ -70,12 +70,6 @@ __device__ __forceinline__ F2& F2::operator*=(const F2& b) { return *this = F2(*
 __device__ __forceinline__ F2& F2::operator+=(const F2M& b) { return *this = *this + b; }
 __device__ __forceinline__ F2& F2::operator-=(const F2M& b) { return *this = *this - b; }
 
-// per-lane fast division (hardware reciprocal), as fdiv(float, float)
-__device__ __forceinline__ F2 fdiv(const F2& a, const F2& b)
-{
-    return F2(__fdividef(a.v.x, b.v.x), __fdividef(a.v.y, b.v.y));
-}
-
 // per-lane select
 __device__ __forceinline__ F2 f2sel(bool p0, bool p1, const F2& a, const F2& b)
 {
@@ -94,22 +88,12 @@ struct ScalarOf<F2> {
 template <typename R>
 using scalar_t = typename ScalarOf<R>::type;
 
-// WENO3 derivative of two cells (the per-lane form of weno3_deriv_fast)
-__device__ __forceinline__ F2 weno3_deriv_fast(const F2* v, const F2& u, const F2& eps)
-{
-    const bool n0 = u.v.x < 0.f, n1 = u.v.y < 0.f;
-    const F2 a = f2sel(n0, n1, v[4], v[0]);
-    const F2 b = f2sel(n0, n1, v[3], v[1]);
-    const F2 c = v[2];
-    const F2 d = f2sel(n0, n1, v[1], v[3]);
-    const F2 dab = b - a, dbc = c - b, dcd = d - c;
-    const F2 e_ab = eps + dab * dab, e_bc = eps + dbc * dbc, e_cd = eps + dcd * dcd;
-    const F2 w0p = e_cd * e_cd, w1p = F2(2.f) * e_bc * e_bc;
-    const F2 fp = c + F2(0.5f) * fdiv(w0p * dbc + w1p * dcd, w0p + w1p);
-    const F2 w0m = e_bc * e_bc, w1m = F2(2.f) * e_ab * e_ab;
-    const F2 fm = b + F2(0.5f) * fdiv(w0m * dab + w1m * dbc, w0m + w1m);
-    const F2 r = fp - fm;
-    return f2sel(n0, n1, -r, r);
-}
+// upwind side per lane (the forms of upwind_neg, _abs and _sel for a pair)
+struct Neg2 {
+    bool x, y;
+};
+__device__ __forceinline__ Neg2 upwind_neg(const F2& u) { return Neg2{u.v.x < 0.f, u.v.y < 0.f}; }
+__device__ __forceinline__ F2 upwind_abs(const F2& u, Neg2) { return F2(fabsf(u.v.x), fabsf(u.v.y)); }
+__device__ __forceinline__ F2 upwind_sel(Neg2 n, const F2& a, const F2& b) { return f2sel(n.x, n.y, a, b); }
 
 }  // namespace lbfd

@@ -26,8 +26,7 @@ struct StepParams {
     R T_wall[6];
     R inv_Wk[NSP];   // 1/W_k
     R yield[NSP];    // nu_k W_k / (-nu_F W_F)
-    R a_diff[NSP];   // D_k W_k, D_k = alpha / Le_k
-    R a12[NSP];      // a_diff / (12 W_k): the tiles' diffusion on Y_k W with 12x stencils
+    R a12[NSP];      // D_k / 12, D_k = alpha / Le_k: the diffusion on Y_k W with 12x stencils
     R alpha12;       // alpha / 12
     R lam_yield;     // sum_k yield_k / W_k (the reaction's share of Lambda's species sum)
     int fuel, oxid;
@@ -37,8 +36,8 @@ struct StepParams {
     double A_lat_d, Ta_d;  // FP64 copies for the mixed-precision Arrhenius
     R T_fp64;
     R omega_s, omega_b, omega_hi;
-    R alpha;
     R u_in, T_in, Y_in[NSP], invW_in, rho_in;
+    R rho_c, inv_rho_c;  // EOS: rho = rho_c / (T invW), rho_c = T_in invW_in
     R T_solid;
     int solid_isothermal;
     int poiseuille;

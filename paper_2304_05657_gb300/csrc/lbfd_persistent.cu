@@ -87,7 +87,7 @@ __device__ bool grid_wait(PersistentWait* w, unsigned nblocks, long long limit_n
 }
 
 // FP32: four blocks per SM (128 registers); FP64: two
-template <typename S, typename R>
+template <typename S, typename R, bool HI1>
 __global__ void __launch_bounds__(PT_THREADS, sizeof(R) == 4 ? 4 : 2)
     step_kernel_persistent2d(StepParams<R> P, StateView a, StateView b, int n, const uint8_t* solid,
                              const uint8_t* interior, const int* wall_tiles, int nwall_tiles,
@@ -118,15 +118,15 @@ __global__ void __launch_bounds__(PT_THREADS, sizeof(R) == 4 ? 4 : 2)
                 if (i < ncells) {
                     const long long c = cells[i];
                     const int p[3] = {(int)(c % P.nx), (int)(c / P.nx), 0};
-                    cell_step_general<2, S, R, true>(P, p, c, g_in, g_out, T_in, T_out, Y_in, Y_out, solid);
+                    cell_step_general<2, S, R, true, HI1>(P, p, c, g_in, g_out, T_in, T_out, Y_in, Y_out, solid);
                 }
             } else if (it < nchunk + (unsigned)nwall_tiles) {
                 const int wt = wall_tiles[it - nchunk];
-                tiled2d_body<S, R, WALL_TX, WALL_TY, true>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, solid, nullptr,
+                tiled2d_body<S, R, WALL_TX, WALL_TY, true, HI1>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, solid, nullptr,
                                                            tid % WALL_TX, tid / WALL_TX, wt % wgx, wt / wgx);
             } else {
                 const int t = (int)(it - nchunk - (unsigned)nwall_tiles);
-                tiled2d_body<S, R, PT_TX, PT_TY, false>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, nullptr, interior,
+                tiled2d_body<S, R, PT_TX, PT_TY, false, HI1>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, nullptr, interior,
                                                         tid % PT_TX, tid / PT_TX, t % gx, t / gx);
             }
             __syncthreads();  // the next tile restages the shared memory
@@ -140,7 +140,7 @@ cudaError_t launch_pers(const StepParams<R>& P, StateView a, StateView b, int n,
                         const BoundaryLists& bl, PersistentWait* w, long long limit_ns, cudaStream_t stream,
                         int* blocks)
 {
-    auto kern = step_kernel_persistent2d<S, R>;
+    auto kern = P.omega_hi == R(1) ? step_kernel_persistent2d<S, R, true> : step_kernel_persistent2d<S, R, false>;
     const size_t smem = tile_smem_bytes<R, PT_TX, PT_TY>() > tile_smem_bytes<R, WALL_TX, WALL_TY>()
                             ? tile_smem_bytes<R, PT_TX, PT_TY>()
                             : tile_smem_bytes<R, WALL_TX, WALL_TY>();

@@ -15,7 +15,7 @@
 
 namespace lbfd {
 
-template <int DIM, typename S, typename R>
+template <int DIM, typename S, typename R, bool HI1>
 __global__ void __launch_bounds__(256) step_kernel_general(StepParams<R> P, const S* __restrict__ g_in,
                                                            S* __restrict__ g_out, const S* __restrict__ T_in,
                                                            S* __restrict__ T_out, const S* __restrict__ Y_in,
@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(256) step_kernel_general(StepParams<R> P, cons
     const long long r = c / P.nx;
     p[1] = (int)(r % P.ny);
     p[2] = (int)(r / P.ny);
-    cell_step_general<DIM, S, R>(P, p, c, g_in, g_out, T_in, T_out, Y_in, Y_out, solid);
+    cell_step_general<DIM, S, R, true, HI1>(P, p, c, g_in, g_out, T_in, T_out, Y_in, Y_out, solid);
 }
 
 template <int DIM, typename S, typename R>
@@ -38,23 +38,24 @@ static cudaError_t launch_general(const StepParams<R>& P, StateView in, StateVie
 {
     const int threads = 256;
     const long long blocks = (P.ncell + threads - 1) / threads;
-    step_kernel_general<DIM, S, R><<<(unsigned)blocks, threads, 0, stream>>>(
+    auto kern = P.omega_hi == R(1) ? step_kernel_general<DIM, S, R, true> : step_kernel_general<DIM, S, R, false>;
+    kern<<<(unsigned)blocks, threads, 0, stream>>>(
         P, (const S*)in.g, (S*)out.g, (const S*)in.T, (S*)out.T, (const S*)in.Y, (S*)out.Y, solid);
     return cudaGetLastError();
 }
 
 // PAIR: the interior tiles compute two cells per thread in packed FP32
 // (FP32 storage only; the FP64 form keeps one cell per thread)
-template <typename S, typename R, int TX, int TY, bool WALLS, bool PAIR = false, int MINB = 1>
+template <bool HI1, typename S, typename R, int TX, int TY, bool WALLS, bool PAIR = false, int MINB = 1>
 static cudaError_t launch_tiled(const StepParams<R>& P, StateView in, StateView out, const uint8_t* solid,
                                 const BoundaryLists& b, const SideStream& side, cudaStream_t stream)
 {
     constexpr bool pair = PAIR && std::is_same<S, float>::value && std::is_same<R, float>::value;
     constexpr size_t smem = tile_smem_bytes<R, TX, TY>();
-    auto kern = step_kernel_tiled2d<S, R, TX, TY>;
+    auto kern = step_kernel_tiled2d<S, R, TX, TY, HI1>;
     const dim3 block(pair ? TX / 2 : TX, TY);
     constexpr size_t wsmem = tile_smem_bytes<R, WALL_TX, WALL_TY>();
-    auto wkern = step_kernel_tiled2d_walls<S, R, WALL_TX, WALL_TY>;
+    auto wkern = step_kernel_tiled2d_walls<S, R, WALL_TX, WALL_TY, HI1>;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -77,7 +78,7 @@ static cudaError_t launch_tiled(const StepParams<R>& P, StateView in, StateView 
     const int prio = fork ? side.priority : 0;
     if (nb > 0) {  // the longest-latency blocks first
         const unsigned nbk = (unsigned)((nb + 127) / 128);
-        e = launch_prio(step_kernel_boundary<2, S, R>, dim3(nbk), dim3(128), 0, bs, prio, P, (const S*)in.g,
+        e = launch_prio(step_kernel_boundary<2, S, R, true, HI1>, dim3(nbk), dim3(128), 0, bs, prio, P, (const S*)in.g,
                         (S*)out.g, (const S*)in.T, (S*)out.T, (const S*)in.Y, (S*)out.Y, solid, bl, nb);
         if (e != cudaSuccess) return e;
     }
@@ -91,7 +92,7 @@ static cudaError_t launch_tiled(const StepParams<R>& P, StateView in, StateView 
         if (e != cudaSuccess) return e;
     }
     if constexpr (pair) {
-        auto pk = step_kernel_pair2d<TX / 2, TY, MINB>;
+        auto pk = step_kernel_pair2d<TX / 2, TY, MINB, HI1>;
         constexpr size_t psmem = pair_smem_bytes<TX, TY>();
         if (psmem > 48 * 1024 &&
             (e = cudaFuncSetAttribute(pk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem)) != cudaSuccess)
@@ -110,7 +111,8 @@ static cudaError_t launch_tiled(const StepParams<R>& P, StateView in, StateView 
     return cudaSuccess;
 }
 
-template <typename S, typename R>
+// HI1: omega_hi = 1 (the collision from the moments of orders 0-2)
+template <bool HI1, typename S, typename R>
 static cudaError_t launch_2d(int variant, const StepParams<R>& P, StateView in, StateView out, const uint8_t* solid,
                              const BoundaryLists& b, const SideStream& side, cudaStream_t stream)
 {
@@ -119,21 +121,21 @@ static cudaError_t launch_2d(int variant, const StepParams<R>& P, StateView in, 
     // go through the general form
     switch (variant) {
     case 0: return launch_general<2, S, R>(P, in, out, solid, stream);
-    case 1: return launch_tiled<S, R, 32, 8, false>(P, in, out, solid, b, side, stream);
-    case 2: return launch_tiled<S, R, 32, 4, false>(P, in, out, solid, b, side, stream);
-    case 3: return launch_tiled<S, R, 64, 4, false>(P, in, out, solid, b, side, stream);
-    case 4: return launch_tiled<S, R, 32, 16, false>(P, in, out, solid, b, side, stream);
-    case 5: return launch_tiled<S, R, 32, 8, true>(P, in, out, solid, b, side, stream);
-    case 6: return launch_tiled<S, R, 32, 4, true>(P, in, out, solid, b, side, stream);
-    case 7: return launch_tiled<S, R, 64, 4, true>(P, in, out, solid, b, side, stream);
-    case 8: return launch_tiled<S, R, 32, 16, true>(P, in, out, solid, b, side, stream);
+    case 1: return launch_tiled<HI1, S, R, 32, 8, false>(P, in, out, solid, b, side, stream);
+    case 2: return launch_tiled<HI1, S, R, 32, 4, false>(P, in, out, solid, b, side, stream);
+    case 3: return launch_tiled<HI1, S, R, 64, 4, false>(P, in, out, solid, b, side, stream);
+    case 4: return launch_tiled<HI1, S, R, 32, 16, false>(P, in, out, solid, b, side, stream);
+    case 5: return launch_tiled<HI1, S, R, 32, 8, true>(P, in, out, solid, b, side, stream);
+    case 6: return launch_tiled<HI1, S, R, 32, 4, true>(P, in, out, solid, b, side, stream);
+    case 7: return launch_tiled<HI1, S, R, 64, 4, true>(P, in, out, solid, b, side, stream);
+    case 8: return launch_tiled<HI1, S, R, 32, 16, true>(P, in, out, solid, b, side, stream);
     // variants 9-12: as 5-8 with two cells per thread in packed FP32, at
     // 128 registers (9, 10) or 96 (11, 12, five 128-thread blocks per SM;
     // six blocks at 80 registers spill and are slower)
-    case 9: return launch_tiled<S, R, 32, 8, true, true, 4>(P, in, out, solid, b, side, stream);
-    case 10: return launch_tiled<S, R, 64, 8, true, true, 2>(P, in, out, solid, b, side, stream);
-    case 11: return launch_tiled<S, R, 32, 8, true, true, 5>(P, in, out, solid, b, side, stream);
-    case 12: return launch_tiled<S, R, 64, 4, true, true, 5>(P, in, out, solid, b, side, stream);
+    case 9: return launch_tiled<HI1, S, R, 32, 8, true, true, 4>(P, in, out, solid, b, side, stream);
+    case 10: return launch_tiled<HI1, S, R, 64, 8, true, true, 2>(P, in, out, solid, b, side, stream);
+    case 11: return launch_tiled<HI1, S, R, 32, 8, true, true, 5>(P, in, out, solid, b, side, stream);
+    case 12: return launch_tiled<HI1, S, R, 64, 4, true, true, 5>(P, in, out, solid, b, side, stream);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -167,10 +169,16 @@ cudaError_t launch_step(int dim, int precision, int variant, const StepParams<do
     if (dim == 3 && variant > 0)
         return launch_step3d_tiled(precision, variant, Pd, Pf, in, out, solid, b, side, stream);
     if (precision == 0) {
-        if (dim == 2) return launch_2d<double, double>(variant, Pd, in, out, solid, b, side, stream);
+        if (dim == 2) {
+            if (Pd.omega_hi == 1.0) return launch_2d<true, double, double>(variant, Pd, in, out, solid, b, side, stream);
+            return launch_2d<false, double, double>(variant, Pd, in, out, solid, b, side, stream);
+        }
         return launch_general<3, double, double>(Pd, in, out, solid, stream);
     }
-    if (dim == 2) return launch_2d<float, float>(variant, Pf, in, out, solid, b, side, stream);
+    if (dim == 2) {
+        if (Pf.omega_hi == 1.f) return launch_2d<true, float, float>(variant, Pf, in, out, solid, b, side, stream);
+        return launch_2d<false, float, float>(variant, Pf, in, out, solid, b, side, stream);
+    }
     return launch_general<3, float, float>(Pf, in, out, solid, stream);
 }
 

@@ -11,7 +11,7 @@ namespace lbfd {
 // solids (b.wall) go through their coded neighbourhoods (or, with curved
 // walls, the general form with the face rules compiled out).
 // the tile kernel instance: MINB > 0 caps its registers for MINB blocks per SM
-template <typename S, typename R, int TX, int TY, int ZC, int MINB, bool HI1 = false>
+template <typename S, typename R, int TX, int TY, int ZC, int MINB, bool HI1>
 static auto tile3_kernel()
 {
     if constexpr (MINB > 0) return step_kernel_tiled3d_capped<S, R, TX, TY, ZC, MINB, HI1>;
@@ -22,20 +22,16 @@ static auto tile3_kernel()
 // smaller kernels instead of one; Lambda and grad rho pass through aux)
 // WALLS: the wall-aware tile kernel also updates the cells next to
 // in-domain solids, so the wall list runs only with curved walls
-template <typename S, typename R, int TX, int TY, int ZC, int MINB = 0, bool SPLIT = false, bool WALLS = false>
+template <bool HI1, typename S, typename R, int TX, int TY, int ZC, int MINB = 0, bool SPLIT = false, bool WALLS = false>
 static cudaError_t launch_t3(const StepParams<R>& P, StateView in, StateView out, const uint8_t* solid,
                              const BoundaryLists& bin, const SideStream& side, cudaStream_t stream)
 {
     constexpr size_t smem = tile3_smem_bytes<R, TX, TY>();
-    // FP32 with omega_hi = 1 (the usual setting): the tile and coded kernels
-    // that skip the pre-collision cumulants of order >= 3
-    constexpr bool F32 = sizeof(R) == 4;
-    const bool hi1 = F32 && P.omega_hi == R(1);
-    auto kern = hi1 ? tile3_kernel<S, R, TX, TY, ZC, MINB, F32>() : tile3_kernel<S, R, TX, TY, ZC, MINB>();
+    auto kern = tile3_kernel<S, R, TX, TY, ZC, MINB, HI1>();
     auto fkern = step_kernel_fd3d<S, R, TX, TY, ZC>;
-    auto wkern = step_kernel_tiled3d_walls<S, R, TX, TY, ZC>;
-    auto fcode = hi1 ? step_kernel_wallcode<3, S, R, true, F32> : step_kernel_wallcode<3, S, R, true>;
-    auto wcode = hi1 ? step_kernel_wallcode<3, S, R, false, F32> : step_kernel_wallcode<3, S, R, false>;
+    auto wkern = step_kernel_tiled3d_walls<S, R, TX, TY, ZC, HI1>;
+    auto fcode = step_kernel_wallcode<3, S, R, true, HI1>;
+    auto wcode = step_kernel_wallcode<3, S, R, false, HI1>;
     cudaError_t e = SPLIT   ? cudaFuncSetAttribute(fkern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
                     : WALLS ? cudaFuncSetAttribute(wkern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
                             : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -52,7 +48,7 @@ static cudaError_t launch_t3(const StepParams<R>& P, StateView in, StateView out
     const int prio = fork ? side.priority : 0;
     if (b.nface > 0) {
         const unsigned nb = (unsigned)((b.nface + 127) / 128);
-        e = launch_prio(step_kernel_boundary<3, S, R, true>, dim3(nb), dim3(128), 0, bs, prio, P, (const S*)in.g,
+        e = launch_prio(step_kernel_boundary<3, S, R, true, HI1>, dim3(nb), dim3(128), 0, bs, prio, P, (const S*)in.g,
                         (S*)out.g, (const S*)in.T, (S*)out.T, (const S*)in.Y, (S*)out.Y, solid, b.face, b.nface);
         if (e != cudaSuccess) return e;
     }
@@ -70,7 +66,7 @@ static cudaError_t launch_t3(const StepParams<R>& P, StateView in, StateView out
                             (S*)out.g, (const S*)in.T, (S*)out.T, (const S*)in.Y, (S*)out.Y, b.wall, b.wall_code,
                             b.nwall);
         else
-            e = launch_prio(step_kernel_boundary<3, S, R, false>, dim3(nb), dim3(128), 0, bs, prio, P,
+            e = launch_prio(step_kernel_boundary<3, S, R, false, HI1>, dim3(nb), dim3(128), 0, bs, prio, P,
                             (const S*)in.g, (S*)out.g, (const S*)in.T, (S*)out.T, (const S*)in.Y, (S*)out.Y, solid,
                             b.wall, b.nwall);
         if (e != cudaSuccess) return e;
@@ -80,7 +76,7 @@ static cudaError_t launch_t3(const StepParams<R>& P, StateView in, StateView out
         fkern<<<grid, dim3(TX, TY), smem, stream>>>(P, (const S*)in.g, (const S*)in.T, (S*)out.T, (const S*)in.Y,
                                                     (S*)out.Y, b.interior, (R*)b.aux);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        step_kernel_collide3d<S, R><<<dim3((P.nx + 127) / 128, P.ny, P.nz), 128, 0, stream>>>(
+        step_kernel_collide3d<S, R, HI1><<<dim3((P.nx + 127) / 128, P.ny, P.nz), 128, 0, stream>>>(
             P, (const S*)in.g, (S*)out.g, (const S*)in.T, (const S*)in.Y, b.interior, (const R*)b.aux);
     } else if constexpr (WALLS) {
         wkern<<<grid, dim3(TX, TY), smem, stream>>>(P, (const S*)in.g, (S*)out.g, (const S*)in.T, (S*)out.T,
@@ -97,23 +93,24 @@ static cudaError_t launch_t3(const StepParams<R>& P, StateView in, StateView out
     return cudaSuccess;
 }
 
-template <typename S, typename R>
+// HI1: omega_hi = 1 (the collision from the moments of orders 0-2)
+template <bool HI1, typename S, typename R>
 static cudaError_t launch_3d_tiles(int variant, const StepParams<R>& P, StateView in, StateView out,
                                    const uint8_t* solid, const BoundaryLists& b, const SideStream& side,
                                    cudaStream_t stream)
 {
     switch (variant) {
-    case 1: return launch_t3<S, R, 32, 4, 16>(P, in, out, solid, b, side, stream);
-    case 2: return launch_t3<S, R, 32, 4, 32>(P, in, out, solid, b, side, stream);
+    case 1: return launch_t3<HI1, S, R, 32, 4, 16>(P, in, out, solid, b, side, stream);
+    case 2: return launch_t3<HI1, S, R, 32, 4, 32>(P, in, out, solid, b, side, stream);
     // variant 3: as 1 with the registers capped for four blocks per SM (FP32)
-    case 3: return launch_t3<S, R, 32, 4, 16, sizeof(R) == 4 ? 4 : 0>(P, in, out, solid, b, side, stream);
+    case 3: return launch_t3<HI1, S, R, 32, 4, 16, sizeof(R) == 4 ? 4 : 0>(P, in, out, solid, b, side, stream);
     // variants 4, 5: as 1, 2 split into an FD tile kernel and a collision kernel
-    case 4: return launch_t3<S, R, 32, 4, 16, 0, true>(P, in, out, solid, b, side, stream);
-    case 5: return launch_t3<S, R, 32, 4, 32, 0, true>(P, in, out, solid, b, side, stream);
+    case 4: return launch_t3<HI1, S, R, 32, 4, 16, 0, true>(P, in, out, solid, b, side, stream);
+    case 5: return launch_t3<HI1, S, R, 32, 4, 32, 0, true>(P, in, out, solid, b, side, stream);
     // variants 6, 7: as 1, 2 with the cells next to in-domain solids in the
     // tile kernel (wall-aware), no wall list
-    case 6: return launch_t3<S, R, 32, 4, 16, 0, false, true>(P, in, out, solid, b, side, stream);
-    case 7: return launch_t3<S, R, 32, 4, 32, 0, false, true>(P, in, out, solid, b, side, stream);
+    case 6: return launch_t3<HI1, S, R, 32, 4, 16, 0, false, true>(P, in, out, solid, b, side, stream);
+    case 7: return launch_t3<HI1, S, R, 32, 4, 32, 0, false, true>(P, in, out, solid, b, side, stream);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -122,8 +119,12 @@ cudaError_t launch_step3d_tiled(int precision, int variant, const StepParams<dou
                                 StateView in, StateView out, const uint8_t* solid, const BoundaryLists& b,
                                 const SideStream& side, cudaStream_t stream)
 {
-    if (precision == 0) return launch_3d_tiles<double, double>(variant, Pd, in, out, solid, b, side, stream);
-    return launch_3d_tiles<float, float>(variant, Pf, in, out, solid, b, side, stream);
+    if (precision == 0) {
+        if (Pd.omega_hi == 1.0) return launch_3d_tiles<true, double, double>(variant, Pd, in, out, solid, b, side, stream);
+        return launch_3d_tiles<false, double, double>(variant, Pd, in, out, solid, b, side, stream);
+    }
+    if (Pf.omega_hi == 1.f) return launch_3d_tiles<true, float, float>(variant, Pf, in, out, solid, b, side, stream);
+    return launch_3d_tiles<false, float, float>(variant, Pf, in, out, solid, b, side, stream);
 }
 
 }  // namespace lbfd

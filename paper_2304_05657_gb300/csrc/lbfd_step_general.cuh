@@ -250,12 +250,12 @@ __device__ __forceinline__ void build_line(const StepParams<R>& P, const int p[3
     }
 }
 
-// values of one line point: T, Y_k, 1/W, rho (ghost rules of Eq. 34; the
+// values of one line point: T, Y_k, 1/W, W, rho (ghost rules of Eq. 34; the
 // density of a ghost is reconstructed directly, with rho_B = EOS(T_B, Y))
 template <typename S, typename R>
 __device__ __forceinline__ void line_point(const StepParams<R>& P, const LineDesc<R>& L, int j,
                                            const S* LBFD_RESTRICT T, const S* LBFD_RESTRICT Y, R& Tj, R* Yj,
-                                           R& invWj, R& rhoj)
+                                           R& invWj, R& Wj, R& rhoj)
 {
     const long long s = L.src[j];
     if (L.mode[j] == G_CURVED) {  // precomputed image-point ghost of this step
@@ -264,6 +264,7 @@ __device__ __forceinline__ void line_point(const StepParams<R>& P, const LineDes
 #pragma unroll
         for (int k = 0; k < NSP; ++k) Yj[k] = gv[1 + k];
         invWj = gv[1 + NSP];
+        Wj = frcp(invWj);
         rhoj = gv[2 + 2 * NSP];
         return;
     }
@@ -272,80 +273,66 @@ __device__ __forceinline__ void line_point(const StepParams<R>& P, const LineDes
 #pragma unroll
     for (int k = 0; k < NSP; ++k) Ym[k] = R(Y[(long long)k * P.N + s]);
     const R invWm = inv_molar_mass(P, Ym);
-    const R rhom = eos(P, Tm, invWm);
+    R rhom, Wm;
+    eos_w(P, Tm, invWm, rhom, Wm);
     const int mode = L.mode[j];
     if (mode == G_DIRECT || mode == G_NEUMANN) {
         Tj = Tm;
 #pragma unroll
         for (int k = 0; k < NSP; ++k) Yj[k] = Ym[k];
         invWj = invWm;
+        Wj = Wm;
         rhoj = rhom;
     } else if (mode == G_DIRICHLET_T) {
         Tj = R(2) * L.TB[j] - Tm;
 #pragma unroll
         for (int k = 0; k < NSP; ++k) Yj[k] = Ym[k];
         invWj = invWm;
+        Wj = Wm;
         rhoj = R(2) * eos(P, L.TB[j], invWm) - rhom;
     } else {  // inlet: Dirichlet T_in and Y_in
         Tj = R(2) * P.T_in - Tm;
 #pragma unroll
         for (int k = 0; k < NSP; ++k) Yj[k] = R(2) * P.Y_in[k] - Ym[k];
         invWj = inv_molar_mass(P, Yj);
+        Wj = frcp(invWj);
         rhoj = R(2) * P.rho_in - rhom;
     }
 }
 
-// ---------------------------------------------------------------------------
-// FD right-hand side along one axis, accumulated into the cell's terms.
-// ---------------------------------------------------------------------------
+// one axis of a cell's FD terms from gathered line points
 template <typename R>
-struct FDAccum {
-    R conv_T, diff_T;
-    R conv_Y[NSP], diff_Y[NSP];
-    R grad_rho[3];
-};
-
-template <typename R>
-__device__ __forceinline__ void fd_axis(const StepParams<R>& P, int a, int near, const R* Tl, const R (*Yl)[5],
-                                        const R* invWl, const R* rhol, R u_a, R T0, const R* Y0, R invW0, R rho0,
-                                        FDAccum<R>& acc)
+__device__ __forceinline__ void fd_axis_points(const StepParams<R>& P, R u_a, int near, const R* Tl, const R (*Yl)[5],
+                                               const R* invWl, const R* Wl, const R* rhol, R invW0, R inv_rho0,
+                                               R* gam_a, FDAccum<R>& acc)
 {
-    const R drho = fd_d1(rhol);
-    acc.grad_rho[a] = drho;
-    const R drho_r = fdiv(drho, rho0);
-    // temperature: convection without correction, diffusion (Eq. 7)
-    acc.conv_T += u_a * (near ? fd_c2(Tl) : weno3_deriv_fast(Tl, u_a, P.epsT));
-    acc.diff_T += P.alpha * (fd_d2(Tl) + drho_r * fd_d1(Tl));
-    // species convection with the correction of Eq. 26
-    R Lk[NSP], sumL = R(0);
+    auto copy = [](const R* f, R* v) {
 #pragma unroll
-    for (int k = 0; k < NSP; ++k) {
-        Lk[k] = near ? fd_c2(Yl[k]) : weno3_deriv_fast(Yl[k], u_a, P.epsY);
-        sumL += Lk[k];
-    }
+        for (int j = 0; j < 5; ++j) v[j] = f[j];
+    };
+    fd_axis<true, R>(
+        P, u_a, invW0, inv_rho0, near != 0, [&](R* v) { copy(rhol, v); }, [&](R* v) { copy(Tl, v); },
+        [&](R* v) { copy(invWl, v); },
+        [&](int k, R* v) {
 #pragma unroll
-    for (int k = 0; k < NSP; ++k) acc.conv_Y[k] += u_a * (Lk[k] - Y0[k] * sumL);
-    // species diffusion with the correction velocity (Eq. 1-2), expanded
-    const R dinvW = fd_d1(invWl);
-    R Wl[5];
-#pragma unroll
-    for (int j = 0; j < 5; ++j) Wl[j] = fdiv(R(1), invWl[j]);
-    R m[NSP], dm[NSP], dY[NSP], M = R(0), dM = R(0);
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) {
-        R Xl[5];
-#pragma unroll
-        for (int j = 0; j < 5; ++j) Xl[j] = Yl[k][j] * P.inv_Wk[k] * Wl[j];
-        const R dX = fd_d1(Xl), d2X = fd_d2(Xl);
-        m[k] = P.a_diff[k] * invW0 * dX;
-        dm[k] = P.a_diff[k] * (invW0 * d2X + dinvW * dX);
-        dY[k] = fd_d1(Yl[k]);
-        M += m[k];
-        dM += dm[k];
-    }
+            for (int j = 0; j < 5; ++j) v[j] = Yl[k][j] * Wl[j];
+        },
+        [&](int k, R* v) { copy(Yl[k], v); }, gam_a, acc);
+}
+
+// a6-a7 of a cell: the reaction, the Euler update of T and Y_k (Eq. 1, 7)
+// and Lambda from the non-convective rates (Eq. 6)
+template <typename S, typename R>
+__device__ __forceinline__ R update_scalars(const StepParams<R>& P, long long c, R T0, const R* Y0, R inv_T0, R W0,
+                                            const FDAccum<R>& acc, S* LBFD_RESTRICT T_out, S* LBFD_RESTRICT Y_out)
+{
+    const R q = arrhenius(P, T0, pick_species(Y0, P.fuel), pick_species(Y0, P.oxid));
+    const R DT = acc.diff_T + P.Q_cp * q;
+    T_out[c] = S(T0 + (DT - acc.conv_T));
 #pragma unroll
     for (int k = 0; k < NSP; ++k)
-        acc.diff_Y[k] += dm[k] - dY[k] * M - Y0[k] * dM + (m[k] - Y0[k] * M) * drho_r;
+        Y_out[(long long)k * P.N + c] = S(Y0[k] + ((acc.rhs_Y[k] + Y0[k] * acc.along) + P.yield[k] * q));
+    return DT * inv_T0 + (acc.lamY + P.lam_yield * q) * W0;
 }
 
 // ---------------------------------------------------------------------------
@@ -353,7 +340,7 @@ __device__ __forceinline__ void fd_axis(const StepParams<R>& P, int a, int near,
 // false: a cell whose stencils reach no non-periodic domain face (the face
 // rules are compiled out).
 // ---------------------------------------------------------------------------
-template <int DIM, typename S, typename R, bool FACES = true>
+template <int DIM, typename S, typename R, bool FACES = true, bool HI1 = false>
 __device__ __forceinline__ void cell_step_general(const StepParams<R>& P, const int p[3], long long c,
                                                   const S* LBFD_RESTRICT g_in, S* LBFD_RESTRICT g_out,
                                                   const S* LBFD_RESTRICT T_in, S* LBFD_RESTRICT T_out,
@@ -368,7 +355,9 @@ __device__ __forceinline__ void cell_step_general(const StepParams<R>& P, const 
 #pragma unroll
     for (int k = 0; k < NSP; ++k) Y0[k] = R(Y_in[(long long)k * N + c]);
     const R invW0 = inv_molar_mass(P, Y0);
-    const R rho0 = eos(P, T0, invW0);
+    R rho0, W0;
+    eos_w(P, T0, invW0, rho0, W0);
+    const R inv_rho0 = T0 * invW0 * P.inv_rho_c, inv_T0 = rho0 * invW0 * P.inv_rho_c;
     // a1: a rolled loop (one copy of the boundary rules keeps this kernel
     // small enough for the instruction cache; the pulled values pass
     // through a local array)
@@ -388,57 +377,33 @@ __device__ __forceinline__ void cell_step_general(const StepParams<R>& P, const 
         for (int i = 0; i < Q; ++i) g[i] = gl[i];
     }
     // a2: velocity, Eq. 13b
+    LowMoments<DIM, R> lm;
+    low_moments<DIM>(g, lm);
     R u[3] = {R(0), R(0), R(0)};
-    {
-        const R inv = fdiv(R(3), rho0);
 #pragma unroll
-        for (int a = 0; a < DIM; ++a) {
-            R m = R(0);
-#pragma unroll
-            for (int i = 0; i < Q; ++i) {
-                const int ci = ccomp<DIM>(i, a);
-                if (ci) m += R(ci) * g[i];
-            }
-            u[a] = m * inv;
-        }
-    }
+    for (int a = 0; a < DIM; ++a) u[a] = lm.m1[a] * (R(3) * inv_rho0);
     // a3-a5
     FDAccum<R> acc;
-    acc.conv_T = acc.diff_T = R(0);
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) acc.conv_Y[k] = acc.diff_Y[k] = R(0);
-    acc.grad_rho[0] = acc.grad_rho[1] = acc.grad_rho[2] = R(0);
+    acc.clear();
 #pragma unroll 1
     for (int a = 0; a < DIM; ++a) {
         LineDesc<R> L;
         build_line<DIM, R, FACES>(P, p, c, a, solid, L);
-        R Tl[5], Yl[NSP][5], invWl[5], rhol[5];
+        R Tl[5], Yl[NSP][5], invWl[5], Wl[5], rhol[5];
 #pragma unroll 1
         for (int j = 0; j < 5; ++j) {
             R Yj[NSP];
-            line_point<S, R>(P, L, j, T_in, Y_in, Tl[j], Yj, invWl[j], rhol[j]);
+            line_point<S, R>(P, L, j, T_in, Y_in, Tl[j], Yj, invWl[j], Wl[j], rhol[j]);
 #pragma unroll
             for (int k = 0; k < NSP; ++k) Yl[k][j] = Yj[k];
         }
-        fd_axis<R>(P, a, L.near, Tl, Yl, invWl, rhol, u[a], T0, Y0, invW0, rho0, acc);
+        fd_axis_points<R>(P, u[a], L.near, Tl, Yl, invWl, Wl, rhol, invW0, inv_rho0, &acc.gam[a], acc);
     }
-    // a6: reaction
-    const R q = arrhenius(P, T0, pick_species(Y0, P.fuel), pick_species(Y0, P.oxid));
-    const R reac_T = P.Q_cp * q;
-    // a7: Euler update and Lambda from the non-convective rates (Eq. 6)
-    const R DT = acc.diff_T + reac_T;
-    T_out[c] = S(T0 + (DT - acc.conv_T));
-    R lam_Y = R(0);
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) {
-        const R DY = acc.diff_Y[k] + P.yield[k] * q;
-        Y_out[(long long)k * N + c] = S(Y0[k] + (DY - acc.conv_Y[k]));
-        lam_Y += P.inv_Wk[k] * DY;
-    }
-    const R Lam = fdiv(DT, T0) + fdiv(lam_Y, invW0);
-    // a8-a9
-    collide<DIM, R>(P, g, rho0, u, acc.grad_rho, Lam);
-    // a10
+    // a6-a7
+    const R Lam = update_scalars<S, R>(P, c, T0, Y0, inv_T0, W0, acc, T_out, Y_out);
+    // a8-a10
+    if constexpr (HI1) collide_hi1<DIM, R>(P, lm, rho0, inv_rho0, u, acc.gam, Lam, g);
+    else collide<DIM, R>(P, g, rho0, inv_rho0, u, acc.gam, Lam);
 #pragma unroll
     for (int i = 0; i < Q; ++i) g_out[(long long)i * N + c] = S(g[i]);
 }
@@ -521,7 +486,9 @@ __device__ __forceinline__ void cell_step_coded(const StepParams<R>& P, const in
 #pragma unroll
     for (int k = 0; k < NSP; ++k) Y0[k] = R(Y_in[(long long)k * N + c]);
     const R invW0 = inv_molar_mass(P, Y0);
-    const R rho0 = eos(P, T0, invW0);
+    R rho0, W0;
+    eos_w(P, T0, invW0, rho0, W0);
+    const R inv_rho0 = T0 * invW0 * P.inv_rho_c, inv_T0 = rho0 * invW0 * P.inv_rho_c;
     // a1: pull, half-way bounce-back (Eq. 28) where the code says solid
     R g[Q];
     {
@@ -613,53 +580,33 @@ __device__ __forceinline__ void cell_step_coded(const StepParams<R>& P, const in
             g[i] = R(g_in[bb ? (long long)opposite<DIM>(i) * N + c : (long long)i * N + s]);
         }
     }
+    LowMoments<DIM, R> lm;
+    low_moments<DIM>(g, lm);
     R u[3] = {R(0), R(0), R(0)};
-    {
-        const R inv = fdiv(R(3), rho0);
 #pragma unroll
-        for (int a = 0; a < DIM; ++a) {
-            R m = R(0);
-#pragma unroll
-            for (int i = 0; i < Q; ++i) {
-                const int ci = ccomp<DIM>(i, a);
-                if (ci) m += R(ci) * g[i];
-            }
-            u[a] = m * inv;
-        }
-    }
+    for (int a = 0; a < DIM; ++a) u[a] = lm.m1[a] * (R(3) * inv_rho0);
     FDAccum<R> acc;
-    acc.conv_T = acc.diff_T = R(0);
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) acc.conv_Y[k] = acc.diff_Y[k] = R(0);
-    acc.grad_rho[0] = acc.grad_rho[1] = acc.grad_rho[2] = R(0);
+    acc.clear();
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
         LineDesc<R> L;
         coded_line<DIM, R>(P, p, c, a, (unsigned)(code >> (32 + 6 * a)) & 63u,
                            FACES ? (unsigned)(code >> (50 + 2 * a)) & 3u : 0u, L);
-        R Tl[5], Yl[NSP][5], invWl[5], rhol[5];
+        R Tl[5], Yl[NSP][5], invWl[5], Wl[5], rhol[5];
 #pragma unroll
         for (int j = 0; j < 5; ++j) {  // every point's loads at once
             R Yj[NSP];
-            line_point<S, R>(P, L, j, T_in, Y_in, Tl[j], Yj, invWl[j], rhol[j]);
+            line_point<S, R>(P, L, j, T_in, Y_in, Tl[j], Yj, invWl[j], Wl[j], rhol[j]);
 #pragma unroll
             for (int k = 0; k < NSP; ++k) Yl[k][j] = Yj[k];
         }
-        fd_axis<R>(P, a, L.near, Tl, Yl, invWl, rhol, u[a], T0, Y0, invW0, rho0, acc);
+        fd_axis_points<R>(P, u[a], L.near, Tl, Yl, invWl, Wl, rhol, invW0, inv_rho0, &acc.gam[a], acc);
     }
-    const R q = arrhenius(P, T0, pick_species(Y0, P.fuel), pick_species(Y0, P.oxid));
-    const R reac_T = P.Q_cp * q;
-    const R DT = acc.diff_T + reac_T;
-    T_out[c] = S(T0 + (DT - acc.conv_T));
-    R lam_Y = R(0);
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) {
-        const R DY = acc.diff_Y[k] + P.yield[k] * q;
-        Y_out[(long long)k * N + c] = S(Y0[k] + (DY - acc.conv_Y[k]));
-        lam_Y += P.inv_Wk[k] * DY;
-    }
-    const R Lam = fdiv(DT, T0) + fdiv(lam_Y, invW0);
-    collide<DIM, R, R, HI1>(P, g, rho0, u, acc.grad_rho, Lam);
+    // a6-a7
+    const R Lam = update_scalars<S, R>(P, c, T0, Y0, inv_T0, W0, acc, T_out, Y_out);
+    // a8-a10
+    if constexpr (HI1) collide_hi1<DIM, R>(P, lm, rho0, inv_rho0, u, acc.gam, Lam, g);
+    else collide<DIM, R>(P, g, rho0, inv_rho0, u, acc.gam, Lam);
 #pragma unroll
     for (int i = 0; i < Q; ++i) g_out[(long long)i * N + c] = S(g[i]);
 }

@@ -122,7 +122,8 @@ __device__ __forceinline__ void stage_tile2d_pairs(const StepParams<float>& P, c
         F2 invW = F2(0.f);
 #pragma unroll
         for (int k = 0; k < NSP; ++k) invW += Y[it][k] * F2(P.inv_Wk[k]);
-        const F2 W = fdiv(F2(1.f), invW);
+        F2 W, rho;
+        eos_w(P, T[it], invW, rho, W);
         auto put = [&](float* f, const F2& v) { *reinterpret_cast<float2*>(f + pt) = v.v; };
         put(sm.T, T[it]);
 #pragma unroll
@@ -131,13 +132,13 @@ __device__ __forceinline__ void stage_tile2d_pairs(const StepParams<float>& P, c
             put(sm.X + k * NPT, Y[it][k] * W);  // X_k W_k (1/W_k folded into a12)
         }
         put(sm.invW, invW);
-        put(sm.rho, fdiv(F2(P.T_in * P.invW_in) * W, T[it]));
+        put(sm.rho, rho);
     }
 }
 
 // TXP x TY threads, a tile of 2 TXP x TY cells, at least MINB blocks per
 // SM (which caps the registers); FP32 storage and arithmetic
-template <int TXP, int TY, int MINB>
+template <int TXP, int TY, int MINB, bool HI1>
 __global__ void __launch_bounds__(TXP * TY, MINB)
     step_kernel_pair2d(StepParams<float> P, const float* LBFD_RESTRICT g_in, float* LBFD_RESTRICT g_out,
                        const float* LBFD_RESTRICT T_in, float* LBFD_RESTRICT T_out, const float* LBFD_RESTRICT Y_in,
@@ -211,52 +212,48 @@ __global__ void __launch_bounds__(TXP * TY, MINB)
 
     // a2
     const F2 T0 = pair_at(sm.T, p0), invW0 = pair_at(sm.invW, p0), rho0 = pair_at(sm.rho, p0);
-    F2 Y0[NSP];
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) Y0[k] = pair_at(sm.Y + k * NPT, p0);
-    F2 u[3];
-    {
-        const F2 inv = fdiv(F2(3.f), rho0);
-        u[0] = ((g[2] + g[5] + g[8]) - (g[0] + g[3] + g[6])) * inv;
-        u[1] = ((g[6] + g[7] + g[8]) - (g[0] + g[1] + g[2])) * inv;
-        u[2] = F2(0.f);
-    }
+    const F2 inv_rho0 = T0 * invW0 * F2(P.inv_rho_c);
+    LowMoments<2, F2> lm;
+    low_moments<2>(g, lm);
+    const F2 inv3 = F2(3.f) * inv_rho0;
+    const F2 u[3] = {lm.m1[0] * inv3, lm.m1[1] * inv3, F2(0.f)};
     // a3-a5
-    TileAccum<F2> acc;
+    FDAccum<F2> acc;
     acc.clear();
     {
         auto line_x = [&](const float* f, F2* v) { pair_line<true, SX>(f, p0, v); };
         auto line_y = [&](const float* f, F2* v) { pair_line<false, SX>(f, p0, v); };
-        fd_axis_core<F2>(P, sm, NPT, line_x, 0, u[0], Y0, invW0, rho0, acc);
-        // the point values are read again from shared memory for each use
-        // (the compiler barrier keeps them out of registers in between)
-        asm volatile("" ::: "memory");
-#pragma unroll
-        for (int k = 0; k < NSP; ++k) Y0[k] = pair_at(sm.Y + k * NPT, p0);
-        fd_axis_core<F2>(P, sm, NPT, line_y, 1, u[1], Y0, invW0, rho0, acc);
+        fd_axis_tile<F2>(P, sm, NPT, line_x, 0, u[0], invW0, inv_rho0, acc);
+        fd_axis_tile<F2>(P, sm, NPT, line_y, 1, u[1], invW0, inv_rho0, acc);
     }
-    asm volatile("" ::: "memory");
+    F2 Y0[NSP];
 #pragma unroll
     for (int k = 0; k < NSP; ++k) Y0[k] = pair_at(sm.Y + k * NPT, p0);
     // a6: per lane (the mixed form switches to FP64 above T_fp64)
     const F2 yf = pick_species(Y0, P.fuel), yo = pick_species(Y0, P.oxid);
     const F2 q(arrhenius(P, T0.v.x, yf.v.x, yo.v.x), arrhenius(P, T0.v.y, yf.v.y, yo.v.y));
-    const F2 reac_T = F2(P.Q_cp) * q;
     // a7
-    const F2 DT = acc.diff_T + reac_T;
+    const F2 DT = acc.diff_T + F2(P.Q_cp) * q;
     const bool vec = ok0 && ok1 && (c & 1) == 0;
     pair_store(T_out + c, T0 + (DT - acc.conv_T), ok0, ok1, vec);
 #pragma unroll
     for (int k = 0; k < NSP; ++k)
-        pair_store(Y_out + (long long)k * N + c, Y0[k] + (acc.rhs_Y[k] + F2(P.yield[k]) * q), ok0, ok1, vec);
+        pair_store(Y_out + (long long)k * N + c,
+                   Y0[k] + ((acc.rhs_Y[k] + Y0[k] * acc.along) + F2(P.yield[k]) * q), ok0, ok1, vec);
+    const F2 rc = rho0 * F2(P.inv_rho_c);
     const F2 lam_Y = acc.lamY + F2(P.lam_yield) * q;
-    const F2 Lam = fdiv(DT, T0) + fdiv(lam_Y, invW0);
-    // a8-a10, on the populations read again from shared memory (the compiler
-    // barrier keeps them out of registers during the FD part)
-    asm volatile("" ::: "memory");
+    const F2 Lam = DT * F2(rc * invW0) + lam_Y * F2(rc * T0);
+    // a8-a10; with omega_hi != 1 on the populations read again from shared
+    // memory (the compiler barrier keeps them out of registers during the FD
+    // part)
+    if constexpr (HI1) {
+        collide_hi1<2, F2>(P, lm, rho0, inv_rho0, u, acc.gam, Lam, g);
+    } else {
+        asm volatile("" ::: "memory");
 #pragma unroll
-    for (int i = 0; i < 9; ++i) g[i] = F2(*reinterpret_cast<const float2*>(gs + i * 2 * NT));
-    collide<2, F2>(P, g, rho0, u, acc.grad_rho, Lam);
+        for (int i = 0; i < 9; ++i) g[i] = F2(*reinterpret_cast<const float2*>(gs + i * 2 * NT));
+        collide<2, F2>(P, g, rho0, inv_rho0, u, acc.gam, Lam);
+    }
 #pragma unroll
     for (int i = 0; i < 9; ++i) pair_store(g_out + (long long)i * N + c, g[i], ok0, ok1, vec);
 }

@@ -41,88 +41,31 @@ __host__ __device__ constexpr size_t tile_smem_bytes()
     return sizeof(R) * (size_t)TileGeom<TX, TY>::NPT * (3 + 2 * NSP) + (size_t)TileGeom<TX, TY>::NPT;
 }
 
-// FD sums of the tile kernels: T's convective and non-convective parts,
-// and for the species the net rate rhs_Y = sum over axes of (diffusion -
-// convection) plus lamY = sum_k (diffusion of Y_k) / W_k, the FD part of
-// Lambda's species sum (Eq. 6), which is all that Lambda needs of them
-template <typename R>
-struct TileAccum {
-    R conv_T, diff_T;
-    R rhs_Y[NSP];
-    R lamY;
-    R grad_rho[3];
-    __device__ __forceinline__ void clear()
-    {
-        conv_T = diff_T = lamY = R(0);
-#pragma unroll
-        for (int k = 0; k < NSP; ++k) rhs_Y[k] = R(0);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) grad_rho[a] = R(0);
-    }
-};
-
-// FD terms along one axis of an interior cell (Eq. 25-27): `line(f, v)`
-// gathers the five points of the staged field f along the axis into v.
-// R is the compute type (float, double, or F2 for a pair of cells), PR the
-// parameters' type.
+// FD terms along one axis of an interior cell from the staged tile:
+// `line(f, v)` gathers the five points of the staged field f along the axis
+// into v.  R is the compute type (float, double, or F2 for a pair of
+// cells), PR the parameters' type.
 template <typename R, typename PR, typename SR, typename Line>
-__device__ __forceinline__ void fd_axis_core(const StepParams<PR>& P, const TileSmem<SR>& sm, int npt, Line line,
-                                             int a, R u_a, const R* Y0, R invW0, R rho0, TileAccum<R>& acc)
+__device__ __forceinline__ void fd_axis_tile(const StepParams<PR>& P, const TileSmem<SR>& sm, int npt, Line line,
+                                             int a, R u_a, R invW0, R inv_rho0, FDAccum<R>& acc)
 {
-    R v[5], w[5];
-    line(sm.rho, v);
-    const R drho = fd_d1(v);
-    acc.grad_rho[a] = drho;
-    const R drho_r = fdiv(drho, rho0);
-    line(sm.T, v);
-    acc.conv_T += u_a * weno3_deriv_fast(v, u_a, R(P.epsT));
-    acc.diff_T += R(P.alpha12) * (fd_D2(v) + drho_r * fd_D1(v));  // 12x stencils, alpha / 12
-    line(sm.invW, w);
-    const R dinvW = fd_d1(w);
-    // diffusion fluxes from the staged Y_k W lines first (X_k = Y_k W / W_k;
-    // 1/W_k and 1/12 are folded into a12): their sums M, dM enter every
-    // species' correction term
-    R m[NSP], dm[NSP];
-    R M = R(0), dM = R(0);
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) {
-        line(sm.X + k * npt, v);
-        const R dX = fd_D1(v), d2X = fd_D2(v);
-        const R ak = R(P.a12[k]);
-        m[k] = ak * invW0 * dX;
-        dm[k] = ak * (invW0 * d2X + dinvW * dX);
-        M += m[k];
-        dM += dm[k];
-    }
-    // then the Y_k lines; the convective correction -Y_k u_a sum_j L_j is
-    // added once the sum is known
-    R sumL = R(0);
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) {
-        line(sm.Y + k * npt, v);
-        const R Lk = weno3_deriv_fast(v, u_a, R(P.epsY));
-        sumL += Lk;
-        const R dY = fd_d1(v);
-        const R dk = dm[k] - dY * M - Y0[k] * dM + (m[k] - Y0[k] * M) * drho_r;
-        acc.rhs_Y[k] += dk - u_a * Lk;
-        acc.lamY += R(P.inv_Wk[k]) * dk;
-    }
-    const R us = u_a * sumL;
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) acc.rhs_Y[k] += Y0[k] * us;
+    fd_axis<false, R>(
+        P, u_a, invW0, inv_rho0, false, [&](R* v) { line(sm.rho, v); }, [&](R* v) { line(sm.T, v); },
+        [&](R* v) { line(sm.invW, v); }, [&](int k, R* v) { line(sm.X + k * npt, v); },
+        [&](int k, R* v) { line(sm.Y + k * npt, v); }, &acc.gam[a], acc);
 }
 
-// fast-path FD terms along one axis from shared memory; `st` is the point
-// stride of the axis (1 for x, SX for y) and p0 the centre point
+// the same with the axis' point stride `st` (1 for x, SX for y) and the
+// centre point p0
 template <typename R>
 __device__ __forceinline__ void fd_axis_smem(const StepParams<R>& P, const TileSmem<R>& sm, int npt, int p0, int st,
-                                             int a, R u_a, R T0, const R* Y0, R invW0, R rho0, TileAccum<R>& acc)
+                                             int a, R u_a, R invW0, R inv_rho0, FDAccum<R>& acc)
 {
     auto line = [&](const R* f, R* v) {
 #pragma unroll
         for (int j = 0; j < 5; ++j) v[j] = f[p0 + (j - 2) * st];
     };
-    fd_axis_core<R>(P, sm, npt, line, a, u_a, Y0, invW0, rho0, acc);
+    fd_axis_tile<R>(P, sm, npt, line, a, u_a, invW0, inv_rho0, acc);
 }
 
 // FD terms along one axis for a cell next to in-domain solid cells (staircase
@@ -131,53 +74,33 @@ __device__ __forceinline__ void fd_axis_smem(const StepParams<R>& P, const TileS
 // take the Dirichlet form when the solid is isothermal (Y, X, 1/W mirror).
 template <typename R>
 __device__ __forceinline__ void fd_axis_smem_walls(const StepParams<R>& P, const TileSmem<R>& sm, int npt,
-                                                   const int* pts, int ghost, int a, R u_a, const R* Y0, R invW0,
-                                                   R rho0, TileAccum<R>& acc)
+                                                   const int* pts, int ghost, int a, R u_a, R invW0, R inv_rho0,
+                                                   FDAccum<R>& acc)
 {
     const bool iso = P.solid_isothermal;
     const R TB = P.T_solid;
-    R v[5], w[5];
+    auto line = [&](const R* f, R* v) {
 #pragma unroll
-    for (int j = 0; j < 5; ++j) {
-        w[j] = sm.invW[pts[j]];
-        v[j] = sm.rho[pts[j]];
-        if (iso && ((ghost >> j) & 1)) v[j] = R(2) * eos(P, TB, w[j]) - v[j];
-    }
-    const R drho = fd_d1(v);
-    acc.grad_rho[a] = drho;
-    const R drho_r = fdiv(drho, rho0);
-    const R dinvW = fd_d1(w);
+        for (int j = 0; j < 5; ++j) v[j] = f[pts[j]];
+    };
+    auto line_rho = [&](R* v) {
 #pragma unroll
-    for (int j = 0; j < 5; ++j) {
-        v[j] = sm.T[pts[j]];
-        if (iso && ((ghost >> j) & 1)) v[j] = R(2) * TB - v[j];
-    }
-    const bool near = ghost != 0;
-    acc.conv_T += u_a * (near ? fd_c2(v) : weno3_deriv_fast(v, u_a, P.epsT));
-    acc.diff_T += P.alpha * (fd_d2(v) + drho_r * fd_d1(v));
-    R Lk[NSP], m[NSP], dm[NSP], dY[NSP];
-    R sumL = R(0), M = R(0), dM = R(0);
+        for (int j = 0; j < 5; ++j) {
+            v[j] = sm.rho[pts[j]];
+            if (iso && ((ghost >> j) & 1)) v[j] = R(2) * eos(P, TB, sm.invW[pts[j]]) - v[j];
+        }
+    };
+    auto line_T = [&](R* v) {
 #pragma unroll
-    for (int k = 0; k < NSP; ++k) {
-#pragma unroll
-        for (int j = 0; j < 5; ++j) v[j] = sm.Y[k * npt + pts[j]];
-        Lk[k] = near ? fd_c2(v) : weno3_deriv_fast(v, u_a, P.epsY);
-        sumL += Lk[k];
-        dY[k] = fd_d1(v);
-#pragma unroll
-        for (int j = 0; j < 5; ++j) v[j] = sm.X[k * npt + pts[j]];  // Y_k W
-        const R dX = fd_D1(v), d2X = fd_D2(v);
-        m[k] = P.a12[k] * invW0 * dX;
-        dm[k] = P.a12[k] * (invW0 * d2X + dinvW * dX);
-        M += m[k];
-        dM += dm[k];
-    }
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) {
-        const R dk = dm[k] - dY[k] * M - Y0[k] * dM + (m[k] - Y0[k] * M) * drho_r;
-        acc.rhs_Y[k] += dk - u_a * (Lk[k] - Y0[k] * sumL);
-        acc.lamY += P.inv_Wk[k] * dk;
-    }
+        for (int j = 0; j < 5; ++j) {
+            v[j] = sm.T[pts[j]];
+            if (iso && ((ghost >> j) & 1)) v[j] = R(2) * TB - v[j];
+        }
+    };
+    fd_axis<true, R>(
+        P, u_a, invW0, inv_rho0, ghost != 0, line_rho, line_T, [&](R* v) { line(sm.invW, v); },
+        [&](int k, R* v) { line(sm.X + k * npt, v); }, [&](int k, R* v) { line(sm.Y + k * npt, v); }, &acc.gam[a],
+        acc);
 }
 
 // the five points of an axis line after the mirror rule of Eq. 34 for
@@ -290,7 +213,8 @@ __device__ __forceinline__ void stage_tile2d(const StepParams<R>& P, const TileS
             if (s[it]) continue;
         }
         const R invW = inv_molar_mass(P, Y[it]);
-        const R W = fdiv(R(1), invW);
+        R W, rho;
+        eos_w(P, T[it], invW, rho, W);
         sm.T[pt] = T[it];
 #pragma unroll
         for (int k = 0; k < NSP; ++k) {
@@ -298,7 +222,7 @@ __device__ __forceinline__ void stage_tile2d(const StepParams<R>& P, const TileS
             sm.X[k * NPT + pt] = Y[it][k] * W;  // X_k W_k (1/W_k folded into a12)
         }
         sm.invW[pt] = invW;
-        sm.rho[pt] = fdiv(P.T_in * P.invW_in * W, T[it]);
+        sm.rho[pt] = rho;
     }
 }
 
@@ -318,7 +242,7 @@ __device__ __forceinline__ bool interior_point(const uint8_t* mask, int p0)
 // WALLS == true: only the cells next to in-domain solid cells (or walls that
 // act like them).  Every thread of the block calls it (it synchronises the
 // block once, after the staging).
-template <typename S, typename R, int TX, int TY, bool WALLS>
+template <typename S, typename R, int TX, int TY, bool WALLS, bool HI1>
 __device__ __forceinline__ void tiled2d_body(const StepParams<R>& P, const S* LBFD_RESTRICT g_in, S* LBFD_RESTRICT g_out,
                                              const S* LBFD_RESTRICT T_in, S* LBFD_RESTRICT T_out,
                                              const S* LBFD_RESTRICT Y_in, S* LBFD_RESTRICT Y_out,
@@ -393,58 +317,49 @@ __device__ __forceinline__ void tiled2d_body(const StepParams<R>& P, const S* LB
     }
     // a2
     const R T0 = sm.T[p0], invW0 = sm.invW[p0], rho0 = sm.rho[p0];
-    R Y0[NSP];
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) Y0[k] = sm.Y[k * NPT + p0];
-    R u[3];
-    {
-        const R inv = fdiv(R(3), rho0);
-        u[0] = ((g[2] + g[5] + g[8]) - (g[0] + g[3] + g[6])) * inv;
-        u[1] = ((g[6] + g[7] + g[8]) - (g[0] + g[1] + g[2])) * inv;
-        u[2] = R(0);
-    }
+    const R inv_rho0 = T0 * invW0 * P.inv_rho_c;
+    LowMoments<2, R> lm;
+    low_moments<2>(g, lm);
+    const R u[3] = {lm.m1[0] * (R(3) * inv_rho0), lm.m1[1] * (R(3) * inv_rho0), R(0)};
     // a3-a5
-    TileAccum<R> acc;
+    FDAccum<R> acc;
     acc.clear();
     if constexpr (WALLS) {
         int pts[5];
         int gh = wall_line(sm.mask, p0, 1, pts);
-        fd_axis_smem_walls<R>(P, sm, NPT, pts, gh, 0, u[0], Y0, invW0, rho0, acc);
+        fd_axis_smem_walls<R>(P, sm, NPT, pts, gh, 0, u[0], invW0, inv_rho0, acc);
         gh = wall_line(sm.mask, p0, SX, pts);
-        fd_axis_smem_walls<R>(P, sm, NPT, pts, gh, 1, u[1], Y0, invW0, rho0, acc);
+        fd_axis_smem_walls<R>(P, sm, NPT, pts, gh, 1, u[1], invW0, inv_rho0, acc);
     } else {
-        fd_axis_smem<R>(P, sm, NPT, p0, 1, 0, u[0], T0, Y0, invW0, rho0, acc);
-        fd_axis_smem<R>(P, sm, NPT, p0, SX, 1, u[1], T0, Y0, invW0, rho0, acc);
+        fd_axis_smem<R>(P, sm, NPT, p0, 1, 0, u[0], invW0, inv_rho0, acc);
+        fd_axis_smem<R>(P, sm, NPT, p0, SX, 1, u[1], invW0, inv_rho0, acc);
     }
-    // a6
-    const R q = arrhenius(P, T0, pick_species(Y0, P.fuel), pick_species(Y0, P.oxid));
-    const R reac_T = P.Q_cp * q;
-    // a7
-    const R DT = acc.diff_T + reac_T;
-    T_out[c] = S(T0 + (DT - acc.conv_T));
+    // a6-a7
+    R Y0[NSP];
 #pragma unroll
-    for (int k = 0; k < NSP; ++k) Y_out[(long long)k * N + c] = S(Y0[k] + (acc.rhs_Y[k] + P.yield[k] * q));
-    const R lam_Y = acc.lamY + P.lam_yield * q;
-    const R Lam = fdiv(DT, T0) + fdiv(lam_Y, invW0);
+    for (int k = 0; k < NSP; ++k) Y0[k] = sm.Y[k * NPT + p0];
+    const R rc = rho0 * P.inv_rho_c;
+    const R Lam = update_scalars<S, R>(P, c, T0, Y0, rc * invW0, rc * T0, acc, T_out, Y_out);
     // a8-a10
-    collide<2, R>(P, g, rho0, u, acc.grad_rho, Lam);
+    if constexpr (HI1) collide_hi1<2, R>(P, lm, rho0, inv_rho0, u, acc.gam, Lam, g);
+    else collide<2, R>(P, g, rho0, inv_rho0, u, acc.gam, Lam);
 #pragma unroll
     for (int i = 0; i < 9; ++i) g_out[(long long)i * N + c] = S(g[i]);
 }
 
 // FP32: four 256-thread blocks (1024 threads) per SM, i.e. <= 64 registers
-template <typename S, typename R, int TX, int TY>
+template <typename S, typename R, int TX, int TY, bool HI1>
 __global__ void __launch_bounds__(TX * TY, sizeof(R) == 4 ? 1024 / (TX * TY) : 1)
     step_kernel_tiled2d(StepParams<R> P, const S* LBFD_RESTRICT g_in, S* LBFD_RESTRICT g_out,
                         const S* LBFD_RESTRICT T_in, S* LBFD_RESTRICT T_out, const S* LBFD_RESTRICT Y_in,
                         S* LBFD_RESTRICT Y_out, const uint8_t* LBFD_RESTRICT interior)
 {
-    tiled2d_body<S, R, TX, TY, false>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, nullptr, interior, threadIdx.x,
+    tiled2d_body<S, R, TX, TY, false, HI1>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, nullptr, interior, threadIdx.x,
                                       threadIdx.y, blockIdx.x, blockIdx.y);
 }
 
 // the cells next to in-domain solid cells, over the tiles that contain any
-template <typename S, typename R, int TX, int TY>
+template <typename S, typename R, int TX, int TY, bool HI1>
 __global__ void __launch_bounds__(TX * TY)
     step_kernel_tiled2d_walls(StepParams<R> P, const S* LBFD_RESTRICT g_in, S* LBFD_RESTRICT g_out,
                               const S* LBFD_RESTRICT T_in, S* LBFD_RESTRICT T_out, const S* LBFD_RESTRICT Y_in,
@@ -452,7 +367,7 @@ __global__ void __launch_bounds__(TX * TY)
 {
     const int t = tiles[blockIdx.x];
     const int gxn = (P.nx + TX - 1) / TX;
-    tiled2d_body<S, R, TX, TY, true>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, solid, nullptr, threadIdx.x,
+    tiled2d_body<S, R, TX, TY, true, HI1>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, solid, nullptr, threadIdx.x,
                                      threadIdx.y, t % gxn, t / gxn);
 }
 
@@ -481,7 +396,7 @@ __global__ void __launch_bounds__(128) step_kernel_wallcode(StepParams<R> P, con
 
 // The cells the tiled kernel leaves out: general form over a cell list
 // (FACES == false: cells whose stencils reach no non-periodic face).
-template <int DIM, typename S, typename R, bool FACES = true>
+template <int DIM, typename S, typename R, bool FACES, bool HI1>
 __global__ void __launch_bounds__(128) step_kernel_boundary(StepParams<R> P, const S* LBFD_RESTRICT g_in,
                                                             S* LBFD_RESTRICT g_out, const S* LBFD_RESTRICT T_in,
                                                             S* LBFD_RESTRICT T_out, const S* LBFD_RESTRICT Y_in,
@@ -496,7 +411,7 @@ __global__ void __launch_bounds__(128) step_kernel_boundary(StepParams<R> P, con
     const long long r = c / P.nx;
     p[1] = (int)(r % P.ny);
     p[2] = (int)(r / P.ny);
-    cell_step_general<DIM, S, R, FACES>(P, p, c, g_in, g_out, T_in, T_out, Y_in, Y_out, solid);
+    cell_step_general<DIM, S, R, FACES, HI1>(P, p, c, g_in, g_out, T_in, T_out, Y_in, Y_out, solid);
 }
 
 }  // namespace lbfd

@@ -33,71 +33,46 @@ __host__ __device__ constexpr size_t tile3_smem_bytes()
     return sizeof(R) * (size_t)Tile3Geom<TX, TY>::NPT * (4 + NSP) + (size_t)Tile3Geom<TX, TY>::NPT;
 }
 
-// FD terms along one axis from five explicit shared-memory points (the
-// X_k lines first, as in fd_axis_core); returns d rho / d x_a.  `ghost`
+// FD terms along one axis from five explicit shared-memory points.  `ghost`
 // flags (bit j) the points that are ghosts of an in-domain solid (pts then
 // holds their mirror points): T and rho take the Dirichlet form at
 // isothermal solids, Y_k and W mirror, and the convection of the axis is
-// centred (Sec. II.D, next to a boundary).  ghost == 0 for interior cells.
-template <typename R>
-__device__ __forceinline__ R fd_axis_pts(const StepParams<R>& P, const TileSmem<R>& sm, int npt, const int* pts,
-                                         int ghost, R u_a, const R* Y0, R invW0, R rho0, TileAccum<R>& acc)
+// centred (Sec. II.D, next to a boundary).  WALLS == false: no ghosts.
+template <bool WALLS, typename R>
+__device__ __forceinline__ void fd_axis_pts(const StepParams<R>& P, const TileSmem<R>& sm, int npt, const int* pts,
+                                            int ghost, R u_a, R invW0, R inv_rho0, R* gam_a, FDAccum<R>& acc)
 {
-    R v[5], w[5];
-    const bool dir = ghost != 0 && P.solid_isothermal;
-#pragma unroll
-    for (int j = 0; j < 5; ++j) {
-        v[j] = sm.rho[pts[j]];
-        if (dir && ((ghost >> j) & 1)) v[j] = R(2) * eos(P, P.T_solid, sm.invW[pts[j]]) - v[j];
-    }
-    const R drho = fd_d1(v);
-    const R drho_r = fdiv(drho, rho0);
-#pragma unroll
-    for (int j = 0; j < 5; ++j) {
-        v[j] = sm.T[pts[j]];
-        if (dir && ((ghost >> j) & 1)) v[j] = R(2) * P.T_solid - v[j];
-    }
-    // next to a wall the axis is centred: both are formed and one is kept,
-    // so that a warp mixing wall and interior cells does not branch
-    const bool near = ghost != 0;
-    const R wT = weno3_deriv_fast(v, u_a, P.epsT);
-    acc.conv_T += u_a * (near ? fd_c2(v) : wT);
-    acc.diff_T += P.alpha12 * (fd_D2(v) + drho_r * fd_D1(v));  // 12x stencils, alpha / 12
-#pragma unroll
-    for (int j = 0; j < 5; ++j) w[j] = sm.invW[pts[j]];
-    const R dinvW = fd_d1(w);
+    const bool dir = WALLS && ghost != 0 && P.solid_isothermal;
     R Wl[5];
+    auto line = [&](const R* f, R* v) {
 #pragma unroll
-    for (int j = 0; j < 5; ++j) Wl[j] = sm.X[pts[j]];  // W (the 3-D tile keeps W in the X slot)
-    R m[NSP], dm[NSP];
-    R M = R(0), dM = R(0);
+        for (int j = 0; j < 5; ++j) v[j] = f[pts[j]];
+    };
+    auto line_rho = [&](R* v) {
 #pragma unroll
-    for (int k = 0; k < NSP; ++k) {
+        for (int j = 0; j < 5; ++j) {
+            v[j] = sm.rho[pts[j]];
+            if (dir && ((ghost >> j) & 1)) v[j] = R(2) * eos(P, P.T_solid, sm.invW[pts[j]]) - v[j];
+        }
+    };
+    auto line_T = [&](R* v) {
 #pragma unroll
-        for (int j = 0; j < 5; ++j) v[j] = sm.Y[k * npt + pts[j]] * Wl[j];  // X_k W_k (1/W_k and 1/12 in a12)
-        const R dX = fd_D1(v), d2X = fd_D2(v);
-        m[k] = P.a12[k] * invW0 * dX;
-        dm[k] = P.a12[k] * (invW0 * d2X + dinvW * dX);
-        M += m[k];
-        dM += dm[k];
-    }
-    R sumL = R(0);
+        for (int j = 0; j < 5; ++j) {
+            v[j] = sm.T[pts[j]];
+            if (dir && ((ghost >> j) & 1)) v[j] = R(2) * P.T_solid - v[j];
+        }
+    };
+    auto line_invW = [&](R* v) {
+        line(sm.invW, v);
+        line(sm.X, Wl);  // W (the 3-D tile keeps W in the X slot)
+    };
+    fd_axis<WALLS, R>(
+        P, u_a, invW0, inv_rho0, ghost != 0, line_rho, line_T, line_invW,
+        [&](int k, R* v) {
 #pragma unroll
-    for (int k = 0; k < NSP; ++k) {
-#pragma unroll
-        for (int j = 0; j < 5; ++j) v[j] = sm.Y[k * npt + pts[j]];
-        const R wk = weno3_deriv_fast(v, u_a, P.epsY);
-        const R Lk = near ? fd_c2(v) : wk;
-        sumL += Lk;
-        const R dY = fd_d1(v);
-        const R dk = dm[k] - dY * M - Y0[k] * dM + (m[k] - Y0[k] * M) * drho_r;
-        acc.rhs_Y[k] += dk - u_a * Lk;
-        acc.lamY += P.inv_Wk[k] * dk;
-    }
-    const R us = u_a * sumL;
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) acc.rhs_Y[k] += Y0[k] * us;
-    return drho;
+            for (int j = 0; j < 5; ++j) v[j] = sm.Y[k * npt + pts[j]] * Wl[j];
+        },
+        [&](int k, R* v) { line(sm.Y + k * npt, v); }, gam_a, acc);
 }
 
 // the five points of an axis line after the mirror rule of Eq. 34 for a
@@ -169,17 +144,18 @@ __device__ __forceinline__ void stage_plane(const StepParams<R>& P, const TileSm
         if (cell[it] < 0) continue;
         const int pt = slot * G::NPP + tid + it * NTHR;
         const R invW = inv_molar_mass(P, Y[it]);
-        const R W = fdiv(R(1), invW);
+        R W, rho;
+        eos_w(P, T[it], invW, rho, W);
         sm.T[pt] = T[it];
 #pragma unroll
         for (int k = 0; k < NSP; ++k) sm.Y[k * NPT + pt] = Y[it][k];
         sm.X[pt] = W;  // the 3-D tile keeps W in the X slot
         sm.invW[pt] = invW;
-        sm.rho[pt] = fdiv(P.T_in * P.invW_in * W, T[it]);
+        sm.rho[pt] = rho;
     }
 }
 
-// SPLIT: steps a1-a7 only; Lambda and grad rho of every interior cell go
+// SPLIT: steps a1-a7 only; Lambda and grad rho / rho of every interior cell go
 // to aux (four planes) for step_kernel_collide3d, which does a8-a10
 template <typename S, typename R, int TX, int TY, int ZC, bool SPLIT = false, bool WALLS = false, bool HI1 = false>
 __device__ __forceinline__ void tiled3d_body(const StepParams<R>& P, const S* LBFD_RESTRICT g_in,
@@ -252,24 +228,13 @@ __device__ __forceinline__ void tiled3d_body(const StepParams<R>& P, const S* LB
         const int p0 = sc * NPP + q0;
         if (active) {
             const R T0 = sm.T[p0], invW0 = sm.invW[p0], rho0 = sm.rho[p0];
-            R Y0[NSP];
-#pragma unroll
-            for (int k = 0; k < NSP; ++k) Y0[k] = sm.Y[k * NPT + p0];
+            const R inv_rho0 = T0 * invW0 * P.inv_rho_c;
+            LowMoments<3, R> lm;
+            low_moments<3>(g, lm);
             R u[3];
-            {
-                const R inv = fdiv(R(3), rho0);
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    R m = R(0);
-#pragma unroll
-                    for (int i = 0; i < 27; ++i) {
-                        const int ci = ccomp<3>(i, a);
-                        if (ci) m += R(ci) * g[i];
-                    }
-                    u[a] = m * inv;
-                }
-            }
-            TileAccum<R> acc;
+            for (int a = 0; a < 3; ++a) u[a] = lm.m1[a] * (R(3) * inv_rho0);
+            FDAccum<R> acc;
             acc.clear();
             // the three axes share one copy of the FD code (a rolled loop keeps
             // the kernel small enough for the instruction cache)
@@ -289,24 +254,23 @@ __device__ __forceinline__ void tiled3d_body(const StepParams<R>& P, const S* LB
                     }
                 }
                 const R u_a = a == 0 ? u[0] : (a == 1 ? u[1] : u[2]);
-                const R drho = fd_axis_pts<R>(P, sm, NPT, pts, ghost, u_a, Y0, invW0, rho0, acc);
-                acc.grad_rho[0] = a == 0 ? drho : acc.grad_rho[0];
-                acc.grad_rho[1] = a == 1 ? drho : acc.grad_rho[1];
-                acc.grad_rho[2] = a == 2 ? drho : acc.grad_rho[2];
+                R gam;
+                fd_axis_pts<WALLS, R>(P, sm, NPT, pts, ghost, u_a, invW0, inv_rho0, &gam, acc);
+                acc.gam[0] = a == 0 ? gam : acc.gam[0];
+                acc.gam[1] = a == 1 ? gam : acc.gam[1];
+                acc.gam[2] = a == 2 ? gam : acc.gam[2];
             }
-            const R q = arrhenius(P, T0, pick_species(Y0, P.fuel), pick_species(Y0, P.oxid));
-            const R DT = acc.diff_T + P.Q_cp * q;
-            T_out[c] = S(T0 + (DT - acc.conv_T));
+            R Y0[NSP];
 #pragma unroll
-            for (int k = 0; k < NSP; ++k) Y_out[(long long)k * N + c] = S(Y0[k] + (acc.rhs_Y[k] + P.yield[k] * q));
-            const R lam_Y = acc.lamY + P.lam_yield * q;
-            const R Lam = fdiv(DT, T0) + fdiv(lam_Y, invW0);
+            for (int k = 0; k < NSP; ++k) Y0[k] = sm.Y[k * NPT + p0];
+            const R Lam = update_scalars<S, R>(P, c, T0, Y0, rho0 * invW0 * P.inv_rho_c, sm.X[p0], acc, T_out, Y_out);
             if constexpr (SPLIT) {
                 aux[c] = Lam;
 #pragma unroll
-                for (int a = 0; a < 3; ++a) aux[(long long)(1 + a) * N + c] = acc.grad_rho[a];
+                for (int a = 0; a < 3; ++a) aux[(long long)(1 + a) * N + c] = acc.gam[a];
             } else {
-                collide<3, R, R, HI1>(P, g, rho0, u, acc.grad_rho, Lam);
+                if constexpr (HI1) collide_hi1<3, R>(P, lm, rho0, inv_rho0, u, acc.gam, Lam, g);
+                else collide<3, R>(P, g, rho0, inv_rho0, u, acc.gam, Lam);
 #pragma unroll
                 for (int i = 0; i < 27; ++i) g_out[(long long)i * N + c] = S(g[i]);
             }
@@ -327,7 +291,7 @@ __global__ void __launch_bounds__(TX * TY) step_kernel_tiled3d(StepParams<R> P, 
 
 // interior cells and, from the same staging, the cells next to in-domain
 // solids (class 2): no separate wall-list kernel
-template <typename S, typename R, int TX, int TY, int ZC>
+template <typename S, typename R, int TX, int TY, int ZC, bool HI1>
 __global__ void __launch_bounds__(TX * TY) step_kernel_tiled3d_walls(StepParams<R> P, const S* LBFD_RESTRICT g_in,
                                                                      S* LBFD_RESTRICT g_out,
                                                                      const S* LBFD_RESTRICT T_in,
@@ -337,7 +301,7 @@ __global__ void __launch_bounds__(TX * TY) step_kernel_tiled3d_walls(StepParams<
                                                                      const uint8_t* LBFD_RESTRICT interior,
                                                                      const uint8_t* LBFD_RESTRICT solid)
 {
-    tiled3d_body<S, R, TX, TY, ZC, false, true>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, interior, nullptr, solid);
+    tiled3d_body<S, R, TX, TY, ZC, false, true, HI1>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, interior, nullptr, solid);
 }
 
 // the same with the registers capped so that MINB blocks fit on an SM
@@ -363,9 +327,9 @@ __global__ void __launch_bounds__(TX * TY, sizeof(R) == 4 ? 512 / (TX * TY) : 1)
 
 // a1, a2 and a8-a10 of the interior cells (the LB half of a split step):
 // the pull and the density are recomputed exactly as in the FD half, Lambda
-// and grad rho read from aux.  One thread per cell, 128 cells of an x-row
+// and grad rho / rho read from aux.  One thread per cell, 128 cells of an x-row
 // per block.
-template <typename S, typename R>
+template <typename S, typename R, bool HI1>
 __global__ void __launch_bounds__(128)
     step_kernel_collide3d(StepParams<R> P, const S* LBFD_RESTRICT g_in, S* LBFD_RESTRICT g_out,
                           const S* LBFD_RESTRICT T_in, const S* LBFD_RESTRICT Y_in,
@@ -399,27 +363,20 @@ __global__ void __launch_bounds__(128)
 #pragma unroll
     for (int k = 0; k < NSP; ++k) Y0[k] = R(Y_in[(long long)k * N + c]);
     const R invW0 = inv_molar_mass(P, Y0);
-    const R W = fdiv(R(1), invW0);
-    const R rho0 = fdiv(P.T_in * P.invW_in * W, T0);
+    R rho0, W0;
+    eos_w(P, T0, invW0, rho0, W0);
+    const R inv_rho0 = T0 * invW0 * P.inv_rho_c;
+    LowMoments<3, R> lm;
+    low_moments<3>(g, lm);
     R u[3];
-    {
-        const R inv = fdiv(R(3), rho0);
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            R m = R(0);
-#pragma unroll
-            for (int i = 0; i < 27; ++i) {
-                const int ci = ccomp<3>(i, a);
-                if (ci) m += R(ci) * g[i];
-            }
-            u[a] = m * inv;
-        }
-    }
+    for (int a = 0; a < 3; ++a) u[a] = lm.m1[a] * (R(3) * inv_rho0);
     const R Lam = aux[c];
-    R grad[3];
+    R gam[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) grad[a] = aux[(long long)(1 + a) * N + c];
-    collide<3, R>(P, g, rho0, u, grad, Lam);
+    for (int a = 0; a < 3; ++a) gam[a] = aux[(long long)(1 + a) * N + c];
+    if constexpr (HI1) collide_hi1<3, R>(P, lm, rho0, inv_rho0, u, gam, Lam, g);
+    else collide<3, R>(P, g, rho0, inv_rho0, u, gam, Lam);
 #pragma unroll
     for (int i = 0; i < 27; ++i) g_out[(long long)i * N + c] = S(g[i]);
 }

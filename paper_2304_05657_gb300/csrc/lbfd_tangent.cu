@@ -14,7 +14,7 @@
 
 namespace lbfd {
 
-template <int DIM, typename TT>
+template <int DIM, typename TT, bool HI1>
 __global__ void __launch_bounds__(128) step_kernel_tangent(StepParams<TT> P, const TT* __restrict__ g_in,
                                                            TT* __restrict__ g_out, const TT* __restrict__ T_in,
                                                            TT* __restrict__ T_out, const TT* __restrict__ Y_in,
@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(128) step_kernel_tangent(StepParams<TT> P, con
     const long long r = c / P.nx;
     p[1] = (int)(r % P.ny);
     p[2] = (int)(r / P.ny);
-    cell_step_general<DIM, TT, TT>(P, p, c, g_in, g_out, T_in, T_out, Y_in, Y_out, solid);
+    cell_step_general<DIM, TT, TT, true, HI1>(P, p, c, g_in, g_out, T_in, T_out, Y_in, Y_out, solid);
 }
 
 template <typename TT>
@@ -38,8 +38,9 @@ static cudaError_t step_tangent(int dim, const StepParams<TT>& P, StateView in, 
 {
     if (dim != 2) return cudaErrorInvalidValue;
     const unsigned blocks = (unsigned)((P.ncell + 127) / 128);
-    step_kernel_tangent<2, TT><<<blocks, 128, 0, stream>>>(P, (const TT*)in.g, (TT*)out.g, (const TT*)in.T,
-                                                           (TT*)out.T, (const TT*)in.Y, (TT*)out.Y, solid);
+    auto kern = val(P.omega_hi) == 1.0 ? step_kernel_tangent<2, TT, true> : step_kernel_tangent<2, TT, false>;
+    kern<<<blocks, 128, 0, stream>>>(P, (const TT*)in.g, (TT*)out.g, (const TT*)in.T, (TT*)out.T, (const TT*)in.Y,
+                                     (TT*)out.Y, solid);
     return cudaGetLastError();
 }
 cudaError_t launch_step_tangent(int dim, const StepParams<Tan>& P, StateView in, StateView out, const uint8_t* solid,
