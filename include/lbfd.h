@@ -231,25 +231,28 @@ int lbfd_set_wait_limit(lbfd_handle* h, long long ns);
  * planes) and a per-cell collision kernel (a8-a10), and 6..7 are 1..2 with
  * the cells next to in-domain solids updated in the tile kernel too (ghost
  * points by the mirror rule from the staged mask, bounce-back pulls).  The
- * cells the tiles leave out are listed at create.  In 2-D they go through
- * the general form.  In 3-D with staircase walls, a 64-bit neighbourhood
- * code per listed cell drives a compact form of the step: one list for the
- * cells next to in-domain solids (variants 1..5), one for the cells near
- * inlet and outlet faces of one axis.  The general form takes the other
- * cells near domain faces, and every listed cell when the walls are curved.
- * In FP32 with omega_hi = 1 the 3-D tile and coded kernels form only the
- * central moments of orders 0-2 (the relaxation sets the higher cumulants
- * to equilibrium).  All variants compute the same step up to rounding
- * order.  Default: 1 (0 for LBFD_TANGENT, which has the general form
- * only). */
+ * cells the tiles leave out are listed at create.  With staircase walls, a
+ * 64-bit neighbourhood code per listed cell drives a compact form of the
+ * step: in 2-D for every listed cell but those with a link through two open
+ * faces or a convective outlet without a fluid inner cell; in 3-D one list
+ * for the cells next to in-domain solids (variants 1..5) and one for the
+ * cells near inlet and outlet faces of one axis.  The general form takes the
+ * others, and every listed cell when the walls are curved.  2-D grids too
+ * small to fill the GPU with a variant's tiles (up to 311 296 cells in FP32,
+ * 622 592 in FP64, staircase walls) run as one launch of small tiles and the
+ * listed cells, whatever the variant (except 0).  With omega_hi = 1 the
+ * collision uses the moments of orders 0-2 of the populations alone (the
+ * relaxation sets the higher cumulants to equilibrium).  All variants
+ * compute the same step up to rounding order.  Default: 1 (0 for
+ * LBFD_TANGENT, which has the general form only). */
 int lbfd_num_variants(const lbfd_handle* h);
 int lbfd_get_variant(const lbfd_handle* h);
 int lbfd_set_variant(lbfd_handle* h, int variant);
-/* Kernel launches one step makes with the current variant: the tile
- * variants launch the tile kernel plus one kernel per non-empty list of
- * boundary cells (and the wall-tile kernel in 2-D variants 5..12, the
- * collision kernel in 3-D variants 4..5); curved walls add the ghost-fill
- * kernel. */
+/* Kernel launches one step makes with the current variant: one on small 2-D
+ * grids (above); else the tile variants launch the tile kernel plus one
+ * kernel per non-empty list of boundary cells (and the wall-tile kernel in
+ * 2-D variants 5..12, the collision kernel in 3-D variants 4..5); curved
+ * walls add the ghost-fill kernel. */
 int lbfd_launches_per_step(const lbfd_handle* h);
 
 /* Autotuner: time every variant over `reps` launches on the current state

@@ -46,6 +46,15 @@ struct lbfd_handle {
     long long* bndw;      // 3-D: the others (next to in-domain solids only)
     long long nbndw;
     unsigned long long* bndw_code;  // 3-D: their neighbourhood codes
+    // 2-D: bnd and bndf split into the cells that take the coded form, with
+    // their codes, and the rest (device lists)
+    struct Coded2 {
+        long long* cells;
+        unsigned long long* codes;
+        long long n;
+        long long* rest;
+        long long nrest;
+    } bnd2, bndf2;
     long long* bndfc;     // 3-D: the cells near faces that take the coded form (staircase walls)
     long long nbndfc;
     unsigned long long* bndfc_code;
@@ -264,6 +273,11 @@ void free_handle(lbfd_handle* h)
     if (h->bndf) cudaFree(h->bndf);
     if (h->bndw) cudaFree(h->bndw);
     if (h->bndw_code) cudaFree(h->bndw_code);
+    for (lbfd_handle::Coded2* l : {&h->bnd2, &h->bndf2}) {
+        if (l->cells) cudaFree(l->cells);
+        if (l->codes) cudaFree(l->codes);
+        if (l->rest) cudaFree(l->rest);
+    }
     if (h->bndfc) cudaFree(h->bndfc);
     if (h->bndfc_code) cudaFree(h->bndfc_code);
     if (h->bndfg) cudaFree(h->bndfg);
@@ -343,9 +357,28 @@ lbfd::BoundaryLists lists(const lbfd_handle* h)
             b.face_code = h->bndfc_code;
         }
     }
+    auto coded = [](const lbfd_handle::Coded2& l) { return lbfd::CodedList{l.cells, l.codes, l.n, l.rest, l.nrest}; };
+    b.all2 = coded(h->bnd2);
+    b.face2 = coded(h->bndf2);
     b.interior = h->interior;
     b.aux = h->aux;
     return b;
+}
+
+// whether kernel variant v of this handle runs as the one launch for small
+// grids (the shared-memory variants, staircase walls)
+bool runs_small(const lbfd_handle* h, int v, const lbfd::BoundaryLists& b)
+{
+    return h->dim == 2 && v > 0 && !is_tangent(h->precision) && !h->Pd.curved &&
+           lbfd::small2d_applies(h->precision, h->grid.nx, h->grid.ny, b);
+}
+
+// one FP64 or mixed step with kernel variant v
+cudaError_t launch_variant(const lbfd_handle* h, int v, StateView in, StateView out, cudaStream_t s)
+{
+    const lbfd::BoundaryLists b = lists(h);
+    if (runs_small(h, v, b)) return lbfd::launch_step_small2d(h->precision, h->Pd, h->Pf, in, out, b, s);
+    return lbfd::launch_step(h->dim, h->precision, v, h->Pd, h->Pf, in, out, h->solid, b, h->side, s);
 }
 
 // one step from buffer `from` to buffer `from ^ 1` with kernel variant v
@@ -360,8 +393,7 @@ cudaError_t launch_one(lbfd_handle* h, int from, int v, cudaStream_t s)
         return lbfd::launch_step_tangent(h->dim, h->Pt, view(h, from), view(h, from ^ 1), h->solid, s);
     if (h->precision == LBFD_TANGENT_MIXED)
         return lbfd::launch_step_tangent(h->dim, h->Ptf, view(h, from), view(h, from ^ 1), h->solid, s);
-    return lbfd::launch_step(h->dim, h->precision, v, h->Pd, h->Pf, view(h, from), view(h, from ^ 1), h->solid,
-                             lists(h), h->side, s);
+    return launch_variant(h, v, view(h, from), view(h, from ^ 1), s);
 }
 
 int num_variants_of(const lbfd_handle* h)
@@ -557,6 +589,28 @@ int lbfd_create(const lbfd_grid* grid, const uint8_t* solid_mask, const lbfd_mec
             }
         }
     }
+    if (h->dim == 2 && !is_tangent(h->precision)) {
+        lbfd_handle::Coded2* dst[2] = {&h->bnd2, &h->bndf2};
+        for (int j = 0; j < 2; ++j) {
+            std::vector<long long> cells, rest;
+            std::vector<unsigned long long> codes;
+            lbfd::list_codes2d(h->grid.nx, h->grid.ny, h->Pd.bc, m.data(), lists_host[j], cells, codes, rest);
+            dst[j]->n = (long long)cells.size();
+            dst[j]->nrest = (long long)rest.size();
+            auto put = [&](void** to, const void* from, size_t bytes) {
+                if (bytes == 0) return cudaSuccess;
+                const cudaError_t pe = cudaMalloc(to, bytes);
+                return pe != cudaSuccess ? pe : cudaMemcpy(*to, from, bytes, cudaMemcpyHostToDevice);
+            };
+            if ((e = put((void**)&dst[j]->cells, cells.data(), cells.size() * sizeof(long long))) != cudaSuccess ||
+                (e = put((void**)&dst[j]->codes, codes.data(), codes.size() * sizeof(unsigned long long))) !=
+                    cudaSuccess ||
+                (e = put((void**)&dst[j]->rest, rest.data(), rest.size() * sizeof(long long))) != cudaSuccess) {
+                free_handle(h);
+                return cuda_fail(e, "2-D boundary lists");
+            }
+        }
+    }
     if (h->dim == 2) {
         std::vector<int> tiles;
         lbfd::wall_tiles(h->grid.nx, h->grid.ny, lists_host[0], lists_host[1], tiles);
@@ -739,7 +793,9 @@ int lbfd_launches_per_step(const lbfd_handle* h)
                  (h->variant == 4 || h->variant == 5 ? 1 : 0);
         } else {
             const bool wv = h->variant >= 5 && b.nwall_tiles > 0;
-            n += ((wv ? b.nface : b.nall) > 0 ? 1 : 0) + (wv ? 1 : 0);
+            const lbfd::CodedList& cl = wv ? b.face2 : b.all2;
+            if (h->Pd.curved) n += b.nall > 0 ? 1 : 0;
+            else if (!runs_small(h, h->variant, b)) n += (cl.n > 0 ? 1 : 0) + (cl.nrest > 0 ? 1 : 0) + (wv ? 1 : 0);
         }
     }
     return n + (h->nghost > 0 ? 1 : 0);
@@ -1227,7 +1283,6 @@ static int adjoint_backward_pass(lbfd_handle* h, double seed, int maxn, double* 
     }
     // backward pass: each segment recomputed from its checkpoint with the
     // forward kernels (FP32 in the mixed form), every step's adjoint in FP64
-    const lbfd::BoundaryLists b = lists(h);
     const int G = w[0].slots;
     for (int g = nseg - 1; g >= 0; --g) {
         const int len = steps - g * K < K ? steps - g * K : K;
@@ -1235,9 +1290,8 @@ static int adjoint_backward_pass(lbfd_handle* h, double seed, int maxn, double* 
             AK(cudaMemcpyAsync(seg + (size_t)j * sbytes, h->adj_ck + (size_t)g * sbytes, sbytes,
                                cudaMemcpyDeviceToDevice, s));
         for (int j = 1; j < len; ++j)
-            AK(lbfd::launch_step(h->dim, h->precision, h->variant, h->Pd, h->Pf,
-                                 view_of(h, seg + (size_t)(j - 1) * sbytes), view_of(h, seg + (size_t)j * sbytes),
-                                 h->solid, b, h->side, s));
+            AK(launch_variant(h, h->variant, view_of(h, seg + (size_t)(j - 1) * sbytes),
+                              view_of(h, seg + (size_t)j * sbytes), s));
         if (!pipelined) {  // one step at a time (j0 == j1), recorded and swept in chunks of cells
             for (int j = len - 1; j >= 0; --j) {
                 AK(cudaMemsetAsync(lam0, 0, lbytes, s));

@@ -75,6 +75,25 @@ __device__ __forceinline__ int extent(const StepParams<R>& P, int a)
     return a == 0 ? P.nx : (a == 1 ? P.ny : P.nz);
 }
 
+// type and wall temperature of a face known only at run time, without
+// indexing the parameter arrays (which would copy them to local memory)
+template <typename R>
+__device__ __forceinline__ int face_type(const StepParams<R>& P, int f)
+{
+    int t = P.bc[0];
+#pragma unroll
+    for (int j = 1; j < 6; ++j) t = f == j ? P.bc[j] : t;
+    return t;
+}
+template <typename R>
+__device__ __forceinline__ R face_T_wall(const StepParams<R>& P, int f)
+{
+    R t = P.T_wall[0];
+#pragma unroll
+    for (int j = 1; j < 6; ++j) t = f == j ? P.T_wall[j] : t;
+    return t;
+}
+
 template <typename R>
 __device__ __forceinline__ long long cell_of(const StepParams<R>& P, int x, int y, int z)
 {
@@ -193,6 +212,15 @@ __device__ __forceinline__ R fd_D2(const R* v)  // 12 x the 4th-order central se
     return R(16) * (v[1] + v[3]) - (v[0] + v[4]) - R(30) * v[2];
 }
 
+// a product rounded before it is added to anything
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+template <typename R>
+__device__ __forceinline__ R mul_rn(const R& a, const R& b)
+{
+    return R(a * b);
+}
+
 // Upwind side of a velocity component (u < 0; u = 0 takes the u >= 0 side)
 // and the velocity along it: the FD terms use mirrored lines and |u|, since
 // u L(v) = |u| L(v mirrored) for u < 0.
@@ -272,7 +300,9 @@ struct FDAccum {
 // (the density terms of the expanded form collected in b), its sum over
 // dk / W_k closes with sum_k dY_k / W_k = d(1/W), and the terms along Y_k
 // (-F and the convective correction u sum_j L_j of Eq. 26) are kept as one
-// factor applied once per cell: 37 FP32 instructions per species and axis
+// factor applied once per cell.  Each axis' share is rounded before it joins
+// the sums, so that the two axes may be evaluated by different lanes with
+// the same result.  37 FP32 instructions per species and axis
 // instead of 58 (counted).  a12 = D_k / 12 (W_k cancels against the Y_k W lines).
 template <bool CENTRED, typename R, typename PR, typename LRho, typename LT, typename LW, typename LX, typename LY>
 __device__ __forceinline__ void fd_axis(const StepParams<PR>& P, R u_a, R invW0, R inv_rho0, bool near, LRho line_rho,
@@ -287,8 +317,8 @@ __device__ __forceinline__ void fd_axis(const StepParams<PR>& P, R u_a, R invW0,
     const R gam = R(fd_D1(v)) * R(inv_rho0 * twelfth);
     *gam_a = gam;
     line_T(v);
-    acc.conv_T += ua * conv_deriv<CENTRED>(v, neg, R(P.epsT), near);
-    acc.diff_T += R(P.alpha12) * R(fd_D2(v) + gam * fd_D1(v));
+    acc.conv_T += mul_rn(ua, conv_deriv<CENTRED>(v, neg, R(P.epsT), near));
+    acc.diff_T += mul_rn(R(P.alpha12), R(fd_D2(v) + gam * fd_D1(v)));
     line_invW(v);
     const R dinvW = R(fd_D1(v)) * twelfth;
     const R b = dinvW + invW0 * gam;
@@ -306,18 +336,16 @@ __device__ __forceinline__ void fd_axis(const StepParams<PR>& P, R u_a, R invW0,
     }
     M = M * invW0;
     const R M12 = M * twelfth;
-    acc.lamY += lam - M * dinvW;
-    acc.lamY -= invW0 * F;
+    acc.lamY += R(R(lam - M * dinvW) - invW0 * F);
     R sumL = R(0);
 #pragma unroll
     for (int k = 0; k < NSP; ++k) {
         line_Y(k, v);
         const R L = conv_deriv<CENTRED>(v, neg, R(P.epsY), near);
         sumL += L;
-        acc.rhs_Y[k] += f[k] - M12 * fd_D1(v);
-        acc.rhs_Y[k] -= ua * L;
+        acc.rhs_Y[k] += R(R(f[k] - M12 * fd_D1(v)) - ua * L);
     }
-    acc.along += ua * sumL - F;
+    acc.along += R(ua * sumL - F);
 }
 
 // ---------------------------------------------------------------------------

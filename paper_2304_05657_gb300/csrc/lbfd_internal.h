@@ -57,6 +57,13 @@ cudaError_t launch_prio(void (*kern)(Exp...), dim3 grid, dim3 block, size_t smem
 // `all` every non-interior fluid cell; `face` only those whose stencil
 // reaches a domain face (for the 2-D variants that handle in-domain solid
 // neighbours themselves).  Unused by the general variant.
+struct CodedList {
+    const long long* cells;
+    const unsigned long long* codes;
+    long long n;
+    const long long* rest;
+    long long nrest;
+};
 struct BoundaryLists {
     const long long* all;
     long long nall;
@@ -70,6 +77,9 @@ struct BoundaryLists {
     const long long* face_coded;  // 3-D: cells near inlet/outlet faces taken by cell_step_coded<FACES>
     long long nface_coded;        // (then `face` holds the other cells near faces)
     const unsigned long long* face_code;
+    // 2-D, staircase walls: `all` and `face` split into the cells that
+    // cell_step_coded takes (list_codes2d) and the rest (general form)
+    CodedList all2, face2;
     const uint8_t* interior;  // per cell, 1 for the cells the interior tile kernels update
     void* aux;                // 3-D: 4 planes of the compute type for the split variants
 };
@@ -84,6 +94,13 @@ cudaError_t launch_step(int dim, int precision, int variant, const StepParams<do
                         const StepParams<float>& Pf, StateView in, StateView out, const uint8_t* solid,
                         const BoundaryLists& b, const SideStream& side, cudaStream_t stream);
 int num_variants(int dim);
+
+// One launch for a whole 2-D step on a grid too small to fill the GPU with
+// the tiles of the variants (lbfd_step_small.cu): whether it applies (a rule
+// on the grid and the precision), and the launch.
+bool small2d_applies(int precision, int nx, int ny, const BoundaryLists& b);
+cudaError_t launch_step_small2d(int precision, const StepParams<double>& Pd, const StepParams<float>& Pf, StateView in,
+                                StateView out, const BoundaryLists& b, cudaStream_t stream);
 
 // 3-D tile kernels (variants 1..2 in 3-D), lbfd_step3d.cu
 cudaError_t launch_step3d_tiled(int precision, int variant, const StepParams<double>& Pd, const StepParams<float>& Pf,
@@ -100,6 +117,13 @@ void wall_codes(int nx, int ny, int nz, const int* bc, const uint8_t* solid, con
 // (general form).  Both in the order of `cells`.
 void face_codes(int nx, int ny, int nz, const int* bc, const uint8_t* solid, const std::vector<long long>& cells,
                 std::vector<long long>& coded, std::vector<unsigned long long>& codes, std::vector<long long>& rest);
+
+// The cells of a 2-D boundary list that cell_step_coded<2, FACES> takes,
+// with their codes, and the others (a link that leaves through two open
+// faces, or a convective outlet without a fluid inner cell).  Both in the
+// order of `cells`.
+void list_codes2d(int nx, int ny, const int* bc, const uint8_t* solid, const std::vector<long long>& cells,
+                  std::vector<long long>& coded, std::vector<unsigned long long>& codes, std::vector<long long>& rest);
 
 // Fluid cells that are not interior for the tile kernels (host, at create);
 // faces_only (2-D): only cells whose stencil leaves the domain.

@@ -2,10 +2,10 @@
 //
 // One cooperative launch of as many 128-thread blocks as fit on the GPU
 // at once.  Every step, the blocks take work items from a shared counter:
-// first the chunks of 128 cells near domain faces (general form, the
-// slowest items), then the wall tiles (64 x 2, the cells next to in-domain
-// solids), then the interior tiles (32 x 4 cells), with the same per-cell
-// code as the multi-kernel step of variant 6; then all blocks meet at a
+// first the chunks of 128 boundary cells (general form, then by their
+// neighbourhood codes: the slowest items), then the wall tiles (64 x 2, the
+// cells next to in-domain solids), then the interior tiles (32 x 4 cells),
+// with the same per-cell code as variant 6; then all blocks meet at a
 // grid-wide barrier before the buffers swap roles.  The barrier's wait is
 // bounded: a block that waits longer than the limit records the failure
 // and returns, the others see the record and return too, and the host
@@ -90,14 +90,15 @@ __device__ bool grid_wait(PersistentWait* w, unsigned nblocks, long long limit_n
 template <typename S, typename R, bool HI1>
 __global__ void __launch_bounds__(PT_THREADS, sizeof(R) == 4 ? 4 : 2)
     step_kernel_persistent2d(StepParams<R> P, StateView a, StateView b, int n, const uint8_t* solid,
-                             const uint8_t* interior, const int* wall_tiles, int nwall_tiles,
-                             const long long* cells, long long ncells, PersistentWait* w, long long limit_ns)
+                             const uint8_t* interior, const int* wall_tiles, int nwall_tiles, CodedList cl,
+                             PersistentWait* w, long long limit_ns)
 {
     __shared__ unsigned item_sh;
     const int tid = threadIdx.x;
     const int gx = (P.nx + PT_TX - 1) / PT_TX, gy = (P.ny + PT_TY - 1) / PT_TY;
     const int wgx = (P.nx + WALL_TX - 1) / WALL_TX;
-    const unsigned nchunk = (unsigned)((ncells + PT_THREADS - 1) / PT_THREADS);
+    const unsigned nrest = (unsigned)((cl.nrest + PT_THREADS - 1) / PT_THREADS);
+    const unsigned nchunk = nrest + (unsigned)((cl.n + PT_THREADS - 1) / PT_THREADS);
     const unsigned nitems = nchunk + (unsigned)nwall_tiles + (unsigned)(gx * gy);
     for (int s = 0; s < n; ++s) {
         const StateView in = (s & 1) ? b : a, out = (s & 1) ? a : b;
@@ -113,12 +114,19 @@ __global__ void __launch_bounds__(PT_THREADS, sizeof(R) == 4 ? 4 : 2)
             const unsigned it = item_sh;
             __syncthreads();  // item_sh is rewritten by the next grab
             if (it >= nitems) break;
-            if (it < nchunk) {
+            if (it < nrest) {
                 const long long i = (long long)it * PT_THREADS + tid;
-                if (i < ncells) {
-                    const long long c = cells[i];
+                if (i < cl.nrest) {
+                    const long long c = cl.rest[i];
                     const int p[3] = {(int)(c % P.nx), (int)(c / P.nx), 0};
                     cell_step_general<2, S, R, true, HI1>(P, p, c, g_in, g_out, T_in, T_out, Y_in, Y_out, solid);
+                }
+            } else if (it < nchunk) {
+                const long long i = (long long)(it - nrest) * PT_THREADS + tid;
+                if (i < cl.n) {
+                    const long long c = cl.cells[i];
+                    const int p[3] = {(int)(c % P.nx), (int)(c / P.nx), 0};
+                    cell_step_coded<2, S, R, true, HI1>(P, p, c, cl.codes[i], g_in, g_out, T_in, T_out, Y_in, Y_out);
                 }
             } else if (it < nchunk + (unsigned)nwall_tiles) {
                 const int wt = wall_tiles[it - nchunk];
@@ -156,11 +164,9 @@ cudaError_t launch_pers(const StepParams<R>& P, StateView a, StateView b, int n,
     if (per_sm < 1) return cudaErrorLaunchOutOfResources;
     const unsigned nb = (unsigned)(per_sm * sms);
     *blocks = (int)nb;
-    // wall tiles only when the variant-6 split has them; otherwise every
-    // non-interior cell goes through the general form
-    const bool walls = bl.nwall_tiles > 0;
-    const long long* cells = walls ? bl.face : bl.all;
-    const long long ncells = walls ? bl.nface : bl.nall;
+    // the cells that variant 6 would give to its wall tiles go through their
+    // codes on the grids where it runs as one launch
+    const bool walls = bl.nwall_tiles > 0 && !small2d_applies(sizeof(R) == 8 ? 0 : 1, P.nx, P.ny, bl);
     if ((e = cudaMemsetAsync(w, 0, sizeof(PersistentWait), stream)) != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nb);
@@ -173,8 +179,8 @@ cudaError_t launch_pers(const StepParams<R>& P, StateView a, StateView b, int n,
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, P, a, b, n, solid, (const uint8_t*)bl.interior,
-                              walls ? bl.wall_tiles : (const int*)nullptr, walls ? (int)bl.nwall_tiles : 0, cells,
-                              ncells, w, limit_ns);
+                              walls ? bl.wall_tiles : (const int*)nullptr, walls ? (int)bl.nwall_tiles : 0,
+                              walls ? bl.face2 : bl.all2, w, limit_ns);
 }
 
 }  // namespace

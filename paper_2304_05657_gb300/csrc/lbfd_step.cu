@@ -66,9 +66,12 @@ static cudaError_t launch_tiled(const StepParams<R>& P, StateView in, StateView 
     // (WALLS variants, cells next to in-domain solids) and the boundary
     // kernel (the rest)
     const bool walls = WALLS && !P.curved && b.nwall_tiles > 0;
-    const long long* bl = walls ? b.face : b.all;
-    const long long nb = walls ? b.nface : b.nall;
-    const bool fork = (nb > 0 || walls) && side.stream != nullptr;
+    const CodedList& cl = walls ? b.face2 : b.all2;
+    // with curved walls every listed cell takes the general form
+    const long long* bl = P.curved ? b.all : cl.rest;
+    const long long nb = P.curved ? b.nall : cl.nrest;
+    const long long nc = P.curved ? 0 : cl.n;
+    const bool fork = (nb > 0 || nc > 0 || walls) && side.stream != nullptr;
     cudaError_t e = cudaSuccess;
     if (fork) {
         if ((e = cudaEventRecord(side.fork, stream)) != cudaSuccess) return e;
@@ -76,10 +79,19 @@ static cudaError_t launch_tiled(const StepParams<R>& P, StateView in, StateView 
     }
     cudaStream_t bs = fork ? side.stream : stream;
     const int prio = fork ? side.priority : 0;
+    // one warp per block: the lists are short, and their cells are the
+    // step's longest-latency work, so they are spread over the SMs (FP64:
+    // an SM's one FP64 pipe would run four warps of a block in turn)
     if (nb > 0) {  // the longest-latency blocks first
-        const unsigned nbk = (unsigned)((nb + 127) / 128);
-        e = launch_prio(step_kernel_boundary<2, S, R, true, HI1>, dim3(nbk), dim3(128), 0, bs, prio, P, (const S*)in.g,
+        const unsigned nbk = (unsigned)((nb + 31) / 32);
+        e = launch_prio(step_kernel_boundary<2, S, R, true, HI1>, dim3(nbk), dim3(32), 0, bs, prio, P, (const S*)in.g,
                         (S*)out.g, (const S*)in.T, (S*)out.T, (const S*)in.Y, (S*)out.Y, solid, bl, nb);
+        if (e != cudaSuccess) return e;
+    }
+    if (nc > 0) {
+        const unsigned nbk = (unsigned)((nc + 31) / 32);
+        e = launch_prio(step_kernel_wallcode<2, S, R, true, HI1>, dim3(nbk), dim3(32), 0, bs, prio, P, (const S*)in.g,
+                        (S*)out.g, (const S*)in.T, (S*)out.T, (const S*)in.Y, (S*)out.Y, cl.cells, cl.codes, nc);
         if (e != cudaSuccess) return e;
     }
     if (walls) {
@@ -299,6 +311,91 @@ void face_codes(int nx, int ny, int nz, const int* bc, const uint8_t* solid, con
                 int qo[3] = {p[0], p[1], p[2]}, fo = -1;
                 qo[a] -= side;
                 const unsigned opp = w != 0 && kind(qo, &fo) != 0 ? 1u : 0u;
+                const unsigned b3 = w | (opp << 2);
+                bits6 |= side < 0 ? b3 : b3 << 3;
+                faces2 |= face << (side < 0 ? 0 : 1);
+            }
+            code |= (unsigned long long)bits6 << (32 + 6 * a);
+            code |= (unsigned long long)faces2 << (50 + 2 * a);
+        }
+        if (ok) {
+            coded.push_back(c);
+            codes.push_back(code);
+        } else {
+            rest.push_back(c);
+        }
+    }
+}
+
+void list_codes2d(int nx, int ny, const int* bc, const uint8_t* solid, const std::vector<long long>& cells,
+                  std::vector<long long>& coded, std::vector<unsigned long long>& codes, std::vector<long long>& rest)
+{
+    const int n[2] = {nx, ny};
+    coded.clear();
+    codes.clear();
+    rest.clear();
+    auto is_open = [&](int f) { return bc[f] == BC_INLET || bc[f] == BC_OUTLET || bc[f] == BC_OUTLET_PRESSURE; };
+    // point q: 0 fluid, 1 solid, 2 beyond a non-periodic face (periodic axes wrapped)
+    auto kind = [&](int q[2]) {
+        for (int a = 0; a < 2; ++a) {
+            if (q[a] >= 0 && q[a] < n[a]) continue;
+            if (bc[2 * a + (q[a] < 0 ? 0 : 1)] != BC_PERIODIC) return 2;
+            q[a] = ((q[a] % n[a]) + n[a]) % n[a];
+        }
+        return solid[(long long)q[0] + (long long)nx * q[1]] ? 1 : 0;
+    };
+    for (const long long c : cells) {
+        const int p[2] = {(int)(c % nx), (int)(c / nx)};
+        bool ok = true;
+        unsigned long long code = 0;
+        for (int i = 0; i < 9 && ok; ++i) {  // the rules of pull_general, in its order
+            const int ci[2] = {cx_of(i), cy_of(i)};
+            int q[2] = {p[0] - ci[0], p[1] - ci[1]};
+            int nopen = 0, face = -1;
+            bool wall = false;
+            for (int a = 0; a < 2; ++a) {
+                const int f = q[a] < 0 ? 2 * a : (q[a] >= n[a] ? 2 * a + 1 : -1);
+                if (f < 0) continue;
+                if (bc[f] == BC_PERIODIC) {
+                    q[a] = ((q[a] % n[a]) + n[a]) % n[a];
+                } else {
+                    if (is_open(f)) {
+                        ++nopen;
+                        face = f;
+                    } else {
+                        wall = true;
+                    }
+                    q[a] = q[a] < 0 ? 0 : n[a] - 1;  // the boundary column
+                }
+            }
+            if (wall || solid[(long long)q[0] + (long long)nx * q[1]]) {
+                code |= 1ull << i;
+                continue;
+            }
+            if (nopen > 1) ok = false;
+            if (nopen == 1 && bc[face] == BC_OUTLET) {
+                const int a = face / 2, ns = (face % 2 == 1) ? 1 : -1;
+                int qi[2] = {p[0], p[1]};
+                qi[a] -= ns;
+                if (qi[a] < 0 || qi[a] >= n[a] || kind(qi) != 0) ok = false;
+            }
+        }
+        for (int a = 0; a < 2 && ok; ++a) {
+            unsigned bits6 = 0, faces2 = 0;
+            for (int side = -1; side <= 1; side += 2) {
+                unsigned w = 0, face = 0;
+                for (int j = 1; j <= 2 && !w; ++j) {
+                    int q[2] = {p[0], p[1]};
+                    q[a] += side * j;
+                    const int k = kind(q);
+                    if (k != 0) {
+                        w = (unsigned)j;
+                        face = k == 2 ? 1u : 0u;
+                    }
+                }
+                int qo[2] = {p[0], p[1]};
+                qo[a] -= side;
+                const unsigned opp = w != 0 && kind(qo) != 0 ? 1u : 0u;
                 const unsigned b3 = w | (opp << 2);
                 bits6 |= side < 0 ? b3 : b3 << 3;
                 faces2 |= face << (side < 0 ? 0 : 1);

@@ -324,14 +324,17 @@ __device__ __forceinline__ void fd_axis_points(const StepParams<R>& P, R u_a, in
 // and Lambda from the non-convective rates (Eq. 6)
 template <typename S, typename R>
 __device__ __forceinline__ R update_scalars(const StepParams<R>& P, long long c, R T0, const R* Y0, R inv_T0, R W0,
-                                            const FDAccum<R>& acc, S* LBFD_RESTRICT T_out, S* LBFD_RESTRICT Y_out)
+                                            const FDAccum<R>& acc, S* LBFD_RESTRICT T_out, S* LBFD_RESTRICT Y_out,
+                                            bool store = true)
 {
     const R q = arrhenius(P, T0, pick_species(Y0, P.fuel), pick_species(Y0, P.oxid));
     const R DT = acc.diff_T + P.Q_cp * q;
-    T_out[c] = S(T0 + (DT - acc.conv_T));
+    if (store) {
+        T_out[c] = S(T0 + (DT - acc.conv_T));
 #pragma unroll
-    for (int k = 0; k < NSP; ++k)
-        Y_out[(long long)k * P.N + c] = S(Y0[k] + ((acc.rhs_Y[k] + Y0[k] * acc.along) + P.yield[k] * q));
+        for (int k = 0; k < NSP; ++k)
+            Y_out[(long long)k * P.N + c] = S(Y0[k] + ((acc.rhs_Y[k] + Y0[k] * acc.along) + P.yield[k] * q));
+    }
     return DT * inv_T0 + (acc.lamY + P.lam_yield * q) * W0;
 }
 
@@ -411,9 +414,11 @@ __device__ __forceinline__ void cell_step_general(const StepParams<R>& P, const 
 // ---------------------------------------------------------------------------
 // The same update for a cell next to in-domain solids whose stencils reach
 // no non-periodic face (staircase walls), or (FACES) for a cell near inlet
-// and outlet faces of one axis, with its neighbourhood given by a code
-// computed at create instead of mask reads:
-//   bits 0..26   population i is pulled from a solid cell (bounce-back)
+// and outlet faces of one axis (3-D) or near any faces (2-D), with its
+// neighbourhood given by a code computed at create instead of mask reads:
+//   bits 0..26   population i is pulled from a solid cell, or (2-D) its link
+//                leaves through a wall face or where the boundary column is
+//                solid (bounce-back)
 //   bits 32..49  per axis a (6 bits at 32 + 6a), per side (low 3 bits: -,
 //                high 3 bits: +): the distance 1 or 2 of the first point
 //                along the line that is not a fluid cell (0: none within 2)
@@ -421,7 +426,8 @@ __device__ __forceinline__ void cell_step_general(const StepParams<R>& P, const 
 //                side is not a fluid cell either
 //   bits 50..55  (FACES) per axis (2 bits at 50 + 2a, -: low, +: high): that
 //                first point lies beyond the domain face (inlet: Dirichlet
-//                T_in, Y_in ghosts; outlets: zero gradient), not in a solid
+//                T_in, Y_in ghosts; outlets: zero gradient; walls by their
+//                thermal condition), not in a solid
 // so that all loads of the cell can be issued at once.  A population whose
 // source lies beyond an inlet or outlet face takes the rules of Eq. 31, 32
 // or the constant-pressure outlet; the code builder leaves out the cells
@@ -458,9 +464,13 @@ __device__ __forceinline__ void coded_line(const StepParams<R>& P, const int p[3
         if (!w) continue;
         const bool opp_solid = (bits >> 2) & 1u;
         const bool face = (faces >> (side < 0 ? 0 : 1)) & 1u;
-        const int ftype = P.bc[2 * a + (side < 0 ? 0 : 1)];
-        const int mode = !face ? solid_mode : (ftype == BC_INLET ? G_INLET : G_NEUMANN);
-        const R TB = !face ? P.T_solid : (ftype == BC_INLET ? P.T_in : R(0));
+        const int ftype = face_type(P, 2 * a + (side < 0 ? 0 : 1));
+        int mode = !face ? solid_mode : (ftype == BC_INLET ? G_INLET : G_NEUMANN);
+        R TB = !face ? P.T_solid : (ftype == BC_INLET ? P.T_in : R(0));
+        if (DIM == 2 && face && ftype == BC_WALL_ISOTHERMAL) {  // the 2-D lists hold cells near wall faces too
+            mode = G_DIRICHLET_T;
+            TB = face_T_wall(P, 2 * a + (side < 0 ? 0 : 1));
+        }
 #pragma unroll
         for (int j = 1; j <= 2; ++j) {
             if (j < w) continue;
@@ -470,6 +480,130 @@ __device__ __forceinline__ void coded_line(const StepParams<R>& P, const int p[3
             L.TB[2 + side * j] = TB;
         }
     }
+}
+
+// a1 of a coded cell: pull, half-way bounce-back (Eq. 28) where the code
+// says so, and (FACES) the inlet and outlet rules
+template <int DIM, typename S, typename R, bool FACES>
+__device__ __forceinline__ void pull_coded(const StepParams<R>& P, const int p[3], long long c,
+                                           unsigned long long code, R rho0, R inv_rho0, const S* LBFD_RESTRICT g_in,
+                                           R* g)
+{
+    constexpr int Q = DIM == 2 ? 9 : 27;
+    const long long N = P.N;
+    const long long plane = (long long)P.nx * P.ny;
+    const long long oxm = p[0] == 0 ? P.nx - 1 : -1, oxp = p[0] == P.nx - 1 ? 1 - P.nx : 1;
+    const long long oym = p[1] == 0 ? (long long)(P.ny - 1) * P.nx : -(long long)P.nx;
+    const long long oyp = p[1] == P.ny - 1 ? (long long)(1 - P.ny) * P.nx : (long long)P.nx;
+    long long ozm = 0, ozp = 0;
+    if (DIM == 3) {
+        ozm = p[2] == 0 ? (P.nz - 1) * plane : -plane;
+        ozp = p[2] == P.nz - 1 ? (1 - P.nz) * plane : plane;
+    }
+    // FACES: the cell's own velocity for the outlet rules, when one of
+    // its populations comes from beyond an outlet face
+    R uc[3] = {R(0), R(0), R(0)}, mc[3] = {R(0), R(0), R(0)};
+    if constexpr (FACES) {
+        bool own = false;
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+            const int n = a == 0 ? P.nx : (a == 1 ? P.ny : P.nz);
+            const int pa = a == 0 ? p[0] : (a == 1 ? p[1] : p[2]);
+            const int lo = P.bc[2 * a], hi = P.bc[2 * a + 1];
+            own |= pa == 0 && (lo == BC_OUTLET || lo == BC_OUTLET_PRESSURE);
+            own |= pa == n - 1 && (hi == BC_OUTLET || hi == BC_OUTLET_PRESSURE);
+        }
+        if (own) {
+            R gc[Q];
+#pragma unroll
+            for (int j = 0; j < Q; ++j) gc[j] = R(g_in[(long long)j * N + c]);
+            const R inv = R(3) * inv_rho0;
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) {
+                R m = R(0);
+#pragma unroll
+                for (int j = 0; j < Q; ++j) {
+                    const int cj = ccomp<DIM>(j, a);
+                    if (cj != 0) m += R(cj) * gc[j];
+                }
+                mc[a] = m;
+                uc[a] = m * inv;
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const int cx = ccomp<DIM>(i, 0), cy = ccomp<DIM>(i, 1), cz = ccomp<DIM>(i, 2);
+        const long long s = c + (cx > 0 ? oxm : (cx < 0 ? oxp : 0)) + (cy > 0 ? oym : (cy < 0 ? oyp : 0)) +
+                            (cz > 0 ? ozm : (cz < 0 ? ozp : 0));
+        const bool bb = (code >> i) & 1ull;
+        if constexpr (FACES) {
+            // the face the source x - c_i lies beyond (at most one)
+            int f = -1;
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) {
+                const int ca = ccomp<DIM>(i, a);
+                const int n = a == 0 ? P.nx : (a == 1 ? P.ny : P.nz);
+                const int sa = (a == 0 ? p[0] : (a == 1 ? p[1] : p[2])) - ca;
+                if (ca > 0 && sa < 0 && P.bc[2 * a] != BC_PERIODIC) f = 2 * a;
+                if (ca < 0 && sa >= n && P.bc[2 * a + 1] != BC_PERIODIC) f = 2 * a + 1;
+            }
+            if (f >= 0 && !bb) {
+                const int ib = opposite<DIM>(i);
+                const R gib = R(g_in[(long long)ib * N + c]);
+                const int a = f / 2, t = face_type(P, f);
+                const R ci = R(f / 2 == 0 ? cx : (f / 2 == 1 ? cy : cz));
+                if (t == BC_INLET) {  // Eq. 31 applied to g, u_in along the inward normal
+                    R mag = P.u_in;
+                    if (DIM == 2 && P.poiseuille && a == 0) {
+                        const R ny = R(P.ny), y = R(p[1]) + R(0.5);
+                        mag = R(6) * P.u_in * y * (ny - y) / (ny * ny);
+                    }
+                    const R un = (f % 2 == 0) ? mag : -mag;
+                    g[i] = gib + R(2) * weight<DIM, R>(i) * P.rho_in * ci * un;
+                } else if (t == BC_OUTLET_PRESSURE) {  // constant P_h = 0: anti-bounce-back
+                    R cu = R(0), uu = R(0);
+#pragma unroll
+                    for (int b = 0; b < DIM; ++b) {
+                        cu += R(ccomp<DIM>(i, b)) * uc[b];
+                        uu += uc[b] * uc[b];
+                    }
+                    const R geq_even = weight<DIM, R>(i) * rho0 * (R(1.5) * cu * cu - R(0.5) * uu);
+                    g[i] = R(2) * geq_even - gib;
+                } else {  // Eq. 32 in lattice units, outward normal along a
+                    const int ns = (f % 2 == 1) ? 1 : -1;
+                    const R mom = R(ns) * (a == 0 ? mc[0] : (a == 1 ? mc[1] : mc[2]));
+                    const R un = R(3) * mom * inv_rho0;
+                    const long long st = a == 0 ? 1LL : (a == 1 ? (long long)P.nx : plane);
+                    const R inner = R(g_in[(long long)i * N + c - ns * st]);
+                    g[i] = (P.cs - un) * inner + (R(1) - P.cs + un) * R(g_in[(long long)i * N + c]);
+                }
+                continue;
+            }
+        }
+        g[i] = R(g_in[bb ? (long long)opposite<DIM>(i) * N + c : (long long)i * N + s]);
+    }
+}
+
+// the FD terms of a coded cell along axis a: every point's loads at once
+template <int DIM, typename S, typename R, bool FACES>
+__device__ __forceinline__ void fd_axis_coded(const StepParams<R>& P, const int p[3], long long c, int a,
+                                              unsigned long long code, const S* LBFD_RESTRICT T_in,
+                                              const S* LBFD_RESTRICT Y_in, R u_a, R invW0, R inv_rho0, R* gam_a,
+                                              FDAccum<R>& acc)
+{
+    LineDesc<R> L;
+    coded_line<DIM, R>(P, p, c, a, (unsigned)(code >> (32 + 6 * a)) & 63u,
+                       FACES ? (unsigned)(code >> (50 + 2 * a)) & 3u : 0u, L);
+    R Tl[5], Yl[NSP][5], invWl[5], Wl[5], rhol[5];
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+        R Yj[NSP];
+        line_point<S, R>(P, L, j, T_in, Y_in, Tl[j], Yj, invWl[j], Wl[j], rhol[j]);
+#pragma unroll
+        for (int k = 0; k < NSP; ++k) Yl[k][j] = Yj[k];
+    }
+    fd_axis_points<R>(P, u_a, L.near, Tl, Yl, invWl, Wl, rhol, invW0, inv_rho0, gam_a, acc);
 }
 
 template <int DIM, typename S, typename R, bool FACES = false, bool HI1 = false>
@@ -489,97 +623,8 @@ __device__ __forceinline__ void cell_step_coded(const StepParams<R>& P, const in
     R rho0, W0;
     eos_w(P, T0, invW0, rho0, W0);
     const R inv_rho0 = T0 * invW0 * P.inv_rho_c, inv_T0 = rho0 * invW0 * P.inv_rho_c;
-    // a1: pull, half-way bounce-back (Eq. 28) where the code says solid
     R g[Q];
-    {
-        const long long plane = (long long)P.nx * P.ny;
-        const long long oxm = p[0] == 0 ? P.nx - 1 : -1, oxp = p[0] == P.nx - 1 ? 1 - P.nx : 1;
-        const long long oym = p[1] == 0 ? (long long)(P.ny - 1) * P.nx : -(long long)P.nx;
-        const long long oyp = p[1] == P.ny - 1 ? (long long)(1 - P.ny) * P.nx : (long long)P.nx;
-        long long ozm = 0, ozp = 0;
-        if (DIM == 3) {
-            ozm = p[2] == 0 ? (P.nz - 1) * plane : -plane;
-            ozp = p[2] == P.nz - 1 ? (1 - P.nz) * plane : plane;
-        }
-        // FACES: the cell's own velocity for the outlet rules, when one of
-        // its populations comes from beyond an outlet face
-        R uc[3] = {R(0), R(0), R(0)}, mc[3] = {R(0), R(0), R(0)};
-        if constexpr (FACES) {
-            bool own = false;
-#pragma unroll
-            for (int a = 0; a < DIM; ++a) {
-                const int n = a == 0 ? P.nx : (a == 1 ? P.ny : P.nz);
-                const int pa = a == 0 ? p[0] : (a == 1 ? p[1] : p[2]);
-                const int lo = P.bc[2 * a], hi = P.bc[2 * a + 1];
-                own |= pa == 0 && (lo == BC_OUTLET || lo == BC_OUTLET_PRESSURE);
-                own |= pa == n - 1 && (hi == BC_OUTLET || hi == BC_OUTLET_PRESSURE);
-            }
-            if (own) {
-                R gc[Q];
-#pragma unroll
-                for (int j = 0; j < Q; ++j) gc[j] = R(g_in[(long long)j * N + c]);
-                const R inv = fdiv(R(3), rho0);
-#pragma unroll
-                for (int a = 0; a < DIM; ++a) {
-                    R m = R(0);
-#pragma unroll
-                    for (int j = 0; j < Q; ++j) {
-                        const int cj = ccomp<DIM>(j, a);
-                        if (cj != 0) m += R(cj) * gc[j];
-                    }
-                    mc[a] = m;
-                    uc[a] = m * inv;
-                }
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const int cx = ccomp<DIM>(i, 0), cy = ccomp<DIM>(i, 1), cz = ccomp<DIM>(i, 2);
-            const long long s = c + (cx > 0 ? oxm : (cx < 0 ? oxp : 0)) + (cy > 0 ? oym : (cy < 0 ? oyp : 0)) +
-                                (cz > 0 ? ozm : (cz < 0 ? ozp : 0));
-            const bool bb = (code >> i) & 1ull;
-            if constexpr (FACES) {
-                // the face the source x - c_i lies beyond (at most one)
-                int f = -1;
-#pragma unroll
-                for (int a = 0; a < DIM; ++a) {
-                    const int ca = ccomp<DIM>(i, a);
-                    const int n = a == 0 ? P.nx : (a == 1 ? P.ny : P.nz);
-                    const int sa = (a == 0 ? p[0] : (a == 1 ? p[1] : p[2])) - ca;
-                    if (ca > 0 && sa < 0 && P.bc[2 * a] != BC_PERIODIC) f = 2 * a;
-                    if (ca < 0 && sa >= n && P.bc[2 * a + 1] != BC_PERIODIC) f = 2 * a + 1;
-                }
-                if (f >= 0) {
-                    const int ib = opposite<DIM>(i);
-                    const R gib = R(g_in[(long long)ib * N + c]);
-                    const int a = f / 2, t = P.bc[f];
-                    const R ci = R(f / 2 == 0 ? cx : (f / 2 == 1 ? cy : cz));
-                    if (t == BC_INLET) {  // Eq. 31 applied to g, u_in along the inward normal
-                        const R un = (f % 2 == 0) ? P.u_in : -P.u_in;
-                        g[i] = gib + R(2) * weight<DIM, R>(i) * P.rho_in * ci * un;
-                    } else if (t == BC_OUTLET_PRESSURE) {  // constant P_h = 0: anti-bounce-back
-                        R cu = R(0), uu = R(0);
-#pragma unroll
-                        for (int b = 0; b < DIM; ++b) {
-                            cu += R(ccomp<DIM>(i, b)) * uc[b];
-                            uu += uc[b] * uc[b];
-                        }
-                        const R geq_even = weight<DIM, R>(i) * rho0 * (R(1.5) * cu * cu - R(0.5) * uu);
-                        g[i] = R(2) * geq_even - gib;
-                    } else {  // Eq. 32 in lattice units, outward normal along a
-                        const int ns = (f % 2 == 1) ? 1 : -1;
-                        const R mom = R(ns) * (a == 0 ? mc[0] : (a == 1 ? mc[1] : mc[2]));
-                        const R un = fdiv(R(3) * mom, rho0);
-                        const long long st = a == 0 ? 1LL : (a == 1 ? (long long)P.nx : plane);
-                        const R inner = R(g_in[(long long)i * N + c - ns * st]);
-                        g[i] = (P.cs - un) * inner + (R(1) - P.cs + un) * R(g_in[(long long)i * N + c]);
-                    }
-                    continue;
-                }
-            }
-            g[i] = R(g_in[bb ? (long long)opposite<DIM>(i) * N + c : (long long)i * N + s]);
-        }
-    }
+    pull_coded<DIM, S, R, FACES>(P, p, c, code, rho0, inv_rho0, g_in, g);
     LowMoments<DIM, R> lm;
     low_moments<DIM>(g, lm);
     R u[3] = {R(0), R(0), R(0)};
@@ -588,20 +633,8 @@ __device__ __forceinline__ void cell_step_coded(const StepParams<R>& P, const in
     FDAccum<R> acc;
     acc.clear();
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-        LineDesc<R> L;
-        coded_line<DIM, R>(P, p, c, a, (unsigned)(code >> (32 + 6 * a)) & 63u,
-                           FACES ? (unsigned)(code >> (50 + 2 * a)) & 3u : 0u, L);
-        R Tl[5], Yl[NSP][5], invWl[5], Wl[5], rhol[5];
-#pragma unroll
-        for (int j = 0; j < 5; ++j) {  // every point's loads at once
-            R Yj[NSP];
-            line_point<S, R>(P, L, j, T_in, Y_in, Tl[j], Yj, invWl[j], Wl[j], rhol[j]);
-#pragma unroll
-            for (int k = 0; k < NSP; ++k) Yl[k][j] = Yj[k];
-        }
-        fd_axis_points<R>(P, u[a], L.near, Tl, Yl, invWl, Wl, rhol, invW0, inv_rho0, &acc.gam[a], acc);
-    }
+    for (int a = 0; a < DIM; ++a)
+        fd_axis_coded<DIM, S, R, FACES>(P, p, c, a, code, T_in, Y_in, u[a], invW0, inv_rho0, &acc.gam[a], acc);
     // a6-a7
     const R Lam = update_scalars<S, R>(P, c, T0, Y0, inv_T0, W0, acc, T_out, Y_out);
     // a8-a10

@@ -149,13 +149,7 @@ __global__ void __launch_bounds__(TXP * TY, MINB)
     constexpr int SX = G::SX, NPT = G::NPT;
     static_assert(SX % 2 == 0 && NPT % 2 == 0, "pairs need 8-byte aligned shared rows");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    TileSmem<float> sm;
-    sm.T = reinterpret_cast<float*>(smem_raw);
-    sm.Y = sm.T + NPT;
-    sm.X = sm.Y + NSP * NPT;
-    sm.invW = sm.X + NSP * NPT;
-    sm.rho = sm.invW + NPT;
-    sm.mask = reinterpret_cast<uint8_t*>(sm.rho + NPT);
+    const TileSmem<float> sm = tile_smem<float, TX, TY>(smem_raw);
 
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
     const int x = x0 + 2 * threadIdx.x, y = y0 + threadIdx.y;

@@ -41,6 +41,21 @@ __host__ __device__ constexpr size_t tile_smem_bytes()
     return sizeof(R) * (size_t)TileGeom<TX, TY>::NPT * (3 + 2 * NSP) + (size_t)TileGeom<TX, TY>::NPT;
 }
 
+// the tile's arrays in the block's dynamic shared memory
+template <typename R, int TX, int TY>
+__device__ __forceinline__ TileSmem<R> tile_smem(unsigned char* raw)
+{
+    constexpr int NPT = TileGeom<TX, TY>::NPT;
+    TileSmem<R> sm;
+    sm.T = reinterpret_cast<R*>(raw);
+    sm.Y = sm.T + NPT;
+    sm.X = sm.Y + NSP * NPT;
+    sm.invW = sm.X + NSP * NPT;
+    sm.rho = sm.invW + NPT;
+    sm.mask = reinterpret_cast<uint8_t*>(sm.rho + NPT);
+    return sm;
+}
+
 // FD terms along one axis of an interior cell from the staged tile:
 // `line(f, v)` gathers the five points of the staged field f along the axis
 // into v.  R is the compute type (float, double, or F2 for a pair of
@@ -252,13 +267,7 @@ __device__ __forceinline__ void tiled2d_body(const StepParams<R>& P, const S* LB
     using G = TileGeom<TX, TY>;
     constexpr int SX = G::SX, NPT = G::NPT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    TileSmem<R> sm;
-    sm.T = reinterpret_cast<R*>(smem_raw);
-    sm.Y = sm.T + NPT;
-    sm.X = sm.Y + NSP * NPT;
-    sm.invW = sm.X + NSP * NPT;
-    sm.rho = sm.invW + NPT;
-    sm.mask = reinterpret_cast<uint8_t*>(sm.rho + NPT);
+    const TileSmem<R> sm = tile_smem<R, TX, TY>(smem_raw);
 
     const int x0 = bx * TX, y0 = by * TY;
     const int tid = tx + TX * ty;
