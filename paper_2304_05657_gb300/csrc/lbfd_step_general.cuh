@@ -461,7 +461,6 @@ __device__ __forceinline__ void coded_line(const StepParams<R>& P, const int p[3
     for (int side = -1; side <= 1; side += 2) {
         const unsigned bits = side < 0 ? (code & 7u) : (code >> 3);
         const int w = (int)(bits & 3u);
-        if (!w) continue;
         const bool opp_solid = (bits >> 2) & 1u;
         const bool face = (faces >> (side < 0 ? 0 : 1)) & 1u;
         const int ftype = face_type(P, 2 * a + (side < 0 ? 0 : 1));
@@ -471,14 +470,16 @@ __device__ __forceinline__ void coded_line(const StepParams<R>& P, const int p[3
             mode = G_DIRICHLET_T;
             TB = face_T_wall(P, 2 * a + (side < 0 ? 0 : 1));
         }
-#pragma unroll
-        for (int j = 1; j <= 2; ++j) {
-            if (j < w) continue;
-            const int m = 2 * w - 1 - j;  // mirror offset on this side (Eq. 34)
-            L.src[2 + side * j] = m >= 0 ? L.src[2 + side * m] : (opp_solid ? c : raw[2 - side]);
-            L.mode[2 + side * j] = mode;
-            L.TB[2 + side * j] = TB;
-        }
+        // the ghost at distance j >= w mirrors the point at offset 2w - 1 - j
+        // on this side (Eq. 34): the centre, or the neighbour beyond it (the
+        // centre when that is no fluid cell), or this side's neighbour
+        L.src[2 + side] = w == 1 ? c : raw[2 + side];
+        L.mode[2 + side] = w == 1 ? mode : G_DIRECT;
+        L.TB[2 + side] = TB;
+        L.src[2 + 2 * side] = w == 0 ? raw[2 + 2 * side]
+                                     : (w == 2 ? raw[2 + side] : (opp_solid ? c : raw[2 - side]));
+        L.mode[2 + 2 * side] = w != 0 ? mode : G_DIRECT;
+        L.TB[2 + 2 * side] = TB;
     }
 }
 

@@ -1,7 +1,7 @@
 // lbfd_step_tiled3d.cuh -- 3-D (D3Q27) fused coupled step, 2.5-D tiling.
 //
 // A block of TX x TY threads owns a TX x TY column of cells and marches it
-// through ZC consecutive z-planes.  Shared memory holds a ring of five
+// through zc consecutive z-planes.  Shared memory holds a ring of five
 // z-planes (z-2 .. z+2) of the tile plus its 2-cell x/y halo, with T, Y_k
 // and the derived W, 1/W, rho of every point (X_k = Y_k W / W_k is formed
 // when used); each plane is loaded once per column pass.  Interior cells
@@ -157,8 +157,8 @@ __device__ __forceinline__ void stage_plane(const StepParams<R>& P, const TileSm
 
 // SPLIT: steps a1-a7 only; Lambda and grad rho / rho of every interior cell go
 // to aux (four planes) for step_kernel_collide3d, which does a8-a10
-template <typename S, typename R, int TX, int TY, int ZC, bool SPLIT = false, bool WALLS = false, bool HI1 = false>
-__device__ __forceinline__ void tiled3d_body(const StepParams<R>& P, const S* LBFD_RESTRICT g_in,
+template <typename S, typename R, int TX, int TY, bool SPLIT = false, bool WALLS = false, bool HI1 = false>
+__device__ __forceinline__ void tiled3d_body(const StepParams<R>& P, int zc, const S* LBFD_RESTRICT g_in,
                                              S* LBFD_RESTRICT g_out, const S* LBFD_RESTRICT T_in,
                                              S* LBFD_RESTRICT T_out, const S* LBFD_RESTRICT Y_in,
                                              S* LBFD_RESTRICT Y_out, const uint8_t* LBFD_RESTRICT interior,
@@ -176,7 +176,7 @@ __device__ __forceinline__ void tiled3d_body(const StepParams<R>& P, const S* LB
     sm.rho = sm.invW + NPT;
     sm.mask = reinterpret_cast<uint8_t*>(sm.rho + NPT);
 
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, zb = blockIdx.z * ZC;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, zb = blockIdx.z * zc;
     const long long N = P.N;
     const long long plane = (long long)P.nx * P.ny;
     // ring slot of grid plane z: (z + 5*big) % 5 keeps it non-negative
@@ -186,7 +186,7 @@ __device__ __forceinline__ void tiled3d_body(const StepParams<R>& P, const S* LB
     if constexpr (WALLS) __syncthreads();  // the masks of planes z-1..z+1 are read by the first pull
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
     const int q0 = (threadIdx.y + 2) * SX + threadIdx.x + 2;  // in-plane point of this thread
-    const int zend = zb + ZC < P.nz ? zb + ZC : P.nz;
+    const int zend = zb + zc < P.nz ? zb + zc : P.nz;
     const bool inside = x < P.nx && y < P.ny;
     for (int z = zb; z < zend; ++z) {
         // a1 issued before the staging of plane z+2, so that the population
@@ -279,20 +279,20 @@ __device__ __forceinline__ void tiled3d_body(const StepParams<R>& P, const S* LB
     }
 }
 
-template <typename S, typename R, int TX, int TY, int ZC, bool HI1 = false>
-__global__ void __launch_bounds__(TX * TY) step_kernel_tiled3d(StepParams<R> P, const S* LBFD_RESTRICT g_in,
+template <typename S, typename R, int TX, int TY, bool HI1>
+__global__ void __launch_bounds__(TX * TY) step_kernel_tiled3d(StepParams<R> P, int zc, const S* LBFD_RESTRICT g_in,
                                                                S* LBFD_RESTRICT g_out, const S* LBFD_RESTRICT T_in,
                                                                S* LBFD_RESTRICT T_out, const S* LBFD_RESTRICT Y_in,
                                                                S* LBFD_RESTRICT Y_out,
                                                                const uint8_t* LBFD_RESTRICT interior)
 {
-    tiled3d_body<S, R, TX, TY, ZC, false, false, HI1>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, interior);
+    tiled3d_body<S, R, TX, TY, false, false, HI1>(P, zc, g_in, g_out, T_in, T_out, Y_in, Y_out, interior);
 }
 
 // interior cells and, from the same staging, the cells next to in-domain
 // solids (class 2): no separate wall-list kernel
-template <typename S, typename R, int TX, int TY, int ZC, bool HI1>
-__global__ void __launch_bounds__(TX * TY) step_kernel_tiled3d_walls(StepParams<R> P, const S* LBFD_RESTRICT g_in,
+template <typename S, typename R, int TX, int TY, bool HI1>
+__global__ void __launch_bounds__(TX * TY) step_kernel_tiled3d_walls(StepParams<R> P, int zc, const S* LBFD_RESTRICT g_in,
                                                                      S* LBFD_RESTRICT g_out,
                                                                      const S* LBFD_RESTRICT T_in,
                                                                      S* LBFD_RESTRICT T_out,
@@ -301,28 +301,28 @@ __global__ void __launch_bounds__(TX * TY) step_kernel_tiled3d_walls(StepParams<
                                                                      const uint8_t* LBFD_RESTRICT interior,
                                                                      const uint8_t* LBFD_RESTRICT solid)
 {
-    tiled3d_body<S, R, TX, TY, ZC, false, true, HI1>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, interior, nullptr, solid);
+    tiled3d_body<S, R, TX, TY, false, true, HI1>(P, zc, g_in, g_out, T_in, T_out, Y_in, Y_out, interior, nullptr, solid);
 }
 
 // the same with the registers capped so that MINB blocks fit on an SM
-template <typename S, typename R, int TX, int TY, int ZC, int MINB, bool HI1 = false>
+template <typename S, typename R, int TX, int TY, int MINB, bool HI1>
 __global__ void __launch_bounds__(TX * TY, MINB)
-    step_kernel_tiled3d_capped(StepParams<R> P, const S* LBFD_RESTRICT g_in, S* LBFD_RESTRICT g_out,
+    step_kernel_tiled3d_capped(StepParams<R> P, int zc, const S* LBFD_RESTRICT g_in, S* LBFD_RESTRICT g_out,
                                const S* LBFD_RESTRICT T_in, S* LBFD_RESTRICT T_out, const S* LBFD_RESTRICT Y_in,
                                S* LBFD_RESTRICT Y_out, const uint8_t* LBFD_RESTRICT interior)
 {
-    tiled3d_body<S, R, TX, TY, ZC, false, false, HI1>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, interior);
+    tiled3d_body<S, R, TX, TY, false, false, HI1>(P, zc, g_in, g_out, T_in, T_out, Y_in, Y_out, interior);
 }
 
 // a1-a7 of the interior cells (the FD half of a split step); FP32 held to
 // four 128-thread blocks per SM
-template <typename S, typename R, int TX, int TY, int ZC>
+template <typename S, typename R, int TX, int TY>
 __global__ void __launch_bounds__(TX * TY, sizeof(R) == 4 ? 512 / (TX * TY) : 1)
-    step_kernel_fd3d(StepParams<R> P, const S* LBFD_RESTRICT g_in, const S* LBFD_RESTRICT T_in, S* LBFD_RESTRICT T_out,
+    step_kernel_fd3d(StepParams<R> P, int zc, const S* LBFD_RESTRICT g_in, const S* LBFD_RESTRICT T_in, S* LBFD_RESTRICT T_out,
                      const S* LBFD_RESTRICT Y_in, S* LBFD_RESTRICT Y_out, const uint8_t* LBFD_RESTRICT interior,
                      R* LBFD_RESTRICT aux)
 {
-    tiled3d_body<S, R, TX, TY, ZC, true>(P, g_in, nullptr, T_in, T_out, Y_in, Y_out, interior, aux);
+    tiled3d_body<S, R, TX, TY, true>(P, zc, g_in, nullptr, T_in, T_out, Y_in, Y_out, interior, aux);
 }
 
 // a1, a2 and a8-a10 of the interior cells (the LB half of a split step):
