@@ -56,11 +56,12 @@ struct lbfd_handle {
         long long nrest;
     } bnd2, bndf2;
     long long* bndfc;     // 3-D: the cells near faces that take the coded form (staircase walls)
-    long long nbndfc;
+    long long nbndfc, nbndfx;  // (the first nbndfx of them are not for the tile kernel)
     unsigned long long* bndfc_code;
     long long* bndfg;     // 3-D: the other cells near faces (general form)
     long long nbndfg;
-    uint8_t* interior;    // per cell, 1 = updated by the interior tile kernels
+    uint8_t* interior;    // 2-D, per cell: 1 = updated by the interior tile kernels
+    unsigned long long* words;  // 3-D, per cell: interior, coded (with its code) or other
     void* aux;            // 3-D: Lambda and grad rho planes of the split variants
     int* wtiles;          // tiles holding the other boundary cells (2-D)
     long long nwtiles;
@@ -188,6 +189,7 @@ void fill_params(const lbfd_handle* h, StepParams<R>& P)
     P.inv_rho_c = (R)(1.0 / (p.T_in * invW_in));
     P.rho_in = (R)1.0;  // EOS reference state (T_in, Y_in)
     P.T_solid = (R)p.T_solid;
+    P.rho_solid = (R)(p.T_in * invW_in / p.T_solid);  // (FP64 and mixed 3-D tiles)
     P.solid_isothermal = p.solid_isothermal;
     P.poiseuille = p.poiseuille_inlet;
     for (int f = 0; f < 6; ++f) {
@@ -282,6 +284,7 @@ void free_handle(lbfd_handle* h)
     if (h->bndfc_code) cudaFree(h->bndfc_code);
     if (h->bndfg) cudaFree(h->bndfg);
     if (h->interior) cudaFree(h->interior);
+    if (h->words) cudaFree(h->words);
     if (h->aux) cudaFree(h->aux);
     if (h->wtiles) cudaFree(h->wtiles);
     if (h->pwait) cudaFree(h->pwait);
@@ -341,7 +344,7 @@ lbfd::BoundaryLists lists(const lbfd_handle* h)
     b.nwall = 0;
     b.wall_code = nullptr;
     b.face_coded = nullptr;
-    b.nface_coded = 0;
+    b.nface_coded = b.nface_tile = 0;
     b.face_code = nullptr;
     if (h->dim == 3) {  // the general form takes curved walls in both lists
         b.face = h->bndf;
@@ -354,6 +357,7 @@ lbfd::BoundaryLists lists(const lbfd_handle* h)
             b.nface = h->nbndfg;
             b.face_coded = h->bndfc;
             b.nface_coded = h->nbndfc;
+            b.nface_tile = h->nbndfx;
             b.face_code = h->bndfc_code;
         }
     }
@@ -361,6 +365,7 @@ lbfd::BoundaryLists lists(const lbfd_handle* h)
     b.all2 = coded(h->bnd2);
     b.face2 = coded(h->bndf2);
     b.interior = h->interior;
+    b.words = h->words;
     b.aux = h->aux;
     return b;
 }
@@ -517,7 +522,7 @@ int lbfd_create(const lbfd_grid* grid, const uint8_t* solid_mask, const lbfd_mec
             return cuda_fail(e, "cudaMemcpy(boundary list)");
         }
     }
-    {
+    if (h->dim == 2) {
         // per-cell flag of the cells the tile kernels update (fluid cells
         // outside the boundary list)
         std::vector<uint8_t> inter((size_t)h->ncell, 0);
@@ -534,20 +539,10 @@ int lbfd_create(const lbfd_grid* grid, const uint8_t* solid_mask, const lbfd_mec
         std::set_difference(lists_host[0].begin(), lists_host[0].end(), lists_host[1].begin(), lists_host[1].end(),
                             std::back_inserter(wl));
         h->nbndw = (long long)wl.size();
-        // class 2: next to in-domain solids, no domain face in reach (the
-        // wall-aware tiles update these cells themselves)
-        if (!wl.empty()) {
-            std::vector<uint8_t> cls((size_t)h->ncell);
-            if ((e = cudaMemcpy(cls.data(), h->interior, (size_t)h->ncell, cudaMemcpyDeviceToHost)) != cudaSuccess) {
-                free_handle(h);
-                return cuda_fail(e, "interior flags");
-            }
-            for (long long c : wl) cls[c] = 2;
-            if ((e = cudaMemcpy(h->interior, cls.data(), (size_t)h->ncell, cudaMemcpyHostToDevice)) != cudaSuccess) {
-                free_handle(h);
-                return cuda_fail(e, "interior flags");
-            }
-        }
+        // what each cell is: interior, coded or another kernel's
+        std::vector<unsigned long long> words((size_t)h->ncell);
+        for (long long c = 0; c < h->ncell; ++c) words[c] = m[c] ? ~0ull : 0ull;
+        for (long long c : lists_host[0]) words[c] = ~0ull;
         // the Lambda / grad rho planes of the split variants
         if (!is_tangent(h->precision) &&
             (e = cudaMalloc(&h->aux, (size_t)4 * h->stride * h->esz)) != cudaSuccess) {
@@ -560,6 +555,31 @@ int lbfd_create(const lbfd_grid* grid, const uint8_t* solid_mask, const lbfd_mec
             lbfd::face_codes(h->grid.nx, h->grid.ny, h->grid.nz, h->Pd.bc, m.data(), lists_host[1], fc, fcodes, fg);
             h->nbndfc = (long long)fc.size();
             h->nbndfg = (long long)fg.size();
+            // first the cells that the tile kernel leaves to their codes'
+            // list: next to a face, with a convective outlet there or no
+            // fluid cell on the other side (their ghost does not mirror the
+            // staged plane)
+            std::vector<long long> fl;
+            std::vector<unsigned long long> fl_codes;
+            for (int in_tile = 0; in_tile <= 1; ++in_tile) {
+                for (size_t t = 0; t < fc.size(); ++t) {
+                    bool tile = true;
+                    for (int a = 0; a < 3; ++a)
+                        for (int side = 0; side < 2; ++side)
+                            if ((fcodes[t] >> (50 + 2 * a + side)) & 1u)
+                            {
+                                const unsigned w = (unsigned)(fcodes[t] >> (32 + 6 * a + 3 * side)) & 7u;
+                                tile = tile && w != 5u && !(w == 1u && h->Pd.bc[2 * a + side] == LBFD_BC_OUTLET);
+                            }
+                    if (tile != (in_tile != 0)) continue;
+                    fl.push_back(fc[t]);
+                    fl_codes.push_back(fcodes[t]);
+                    if (tile) words[fc[t]] = fcodes[t] | 1ull << 63;
+                }
+                if (!in_tile) h->nbndfx = (long long)fl.size();
+            }
+            fc.swap(fl);
+            fcodes.swap(fl_codes);
             if ((!fc.empty() &&
                  ((e = cudaMalloc(&h->bndfc, fc.size() * sizeof(long long))) != cudaSuccess ||
                   (e = cudaMemcpy(h->bndfc, fc.data(), fc.size() * sizeof(long long), cudaMemcpyHostToDevice)) !=
@@ -578,6 +598,7 @@ int lbfd_create(const lbfd_grid* grid, const uint8_t* solid_mask, const lbfd_mec
         if (!wl.empty()) {
             std::vector<unsigned long long> codes;
             lbfd::wall_codes(h->grid.nx, h->grid.ny, h->grid.nz, h->Pd.bc, m.data(), wl, codes);
+            for (size_t t = 0; t < wl.size(); ++t) words[wl[t]] = codes[t];
             if ((e = cudaMalloc(&h->bndw, wl.size() * sizeof(long long))) != cudaSuccess ||
                 (e = cudaMemcpy(h->bndw, wl.data(), wl.size() * sizeof(long long), cudaMemcpyHostToDevice)) !=
                     cudaSuccess ||
@@ -587,6 +608,12 @@ int lbfd_create(const lbfd_grid* grid, const uint8_t* solid_mask, const lbfd_mec
                 free_handle(h);
                 return cuda_fail(e, "wall list");
             }
+        }
+        if ((e = cudaMalloc(&h->words, words.size() * sizeof(words[0]))) != cudaSuccess ||
+            (e = cudaMemcpy(h->words, words.data(), words.size() * sizeof(words[0]), cudaMemcpyHostToDevice)) !=
+                cudaSuccess) {
+            free_handle(h);
+            return cuda_fail(e, "cell words");
         }
     }
     if (h->dim == 2 && !is_tangent(h->precision)) {
@@ -788,9 +815,10 @@ int lbfd_launches_per_step(const lbfd_handle* h)
     int n = 1;
     if (h->variant > 0 && !is_tangent(h->precision)) {
         if (h->dim == 3) {
-            const bool wall_list = b.nwall > 0 && (h->variant < 6 || h->Pd.curved);
-            n += (b.nface > 0 ? 1 : 0) + (b.nface_coded > 0 ? 1 : 0) + (wall_list ? 1 : 0) +
-                 (h->variant == 4 || h->variant == 5 ? 1 : 0);
+            const bool split = h->variant == 4 || h->variant == 5;
+            const bool face_list = (h->variant >= 4 ? b.nface_coded : b.nface_tile) > 0;  // (empty with curved walls)
+            n += (b.nface > 0 ? 1 : 0) + (face_list ? 1 : 0) + (b.nwall > 0 && (split || h->Pd.curved) ? 1 : 0) +
+                 (split ? 1 : 0);
         } else {
             const bool wv = h->variant >= 5 && b.nwall_tiles > 0;
             const lbfd::CodedList& cl = wv ? b.face2 : b.all2;

@@ -261,9 +261,10 @@ __device__ __forceinline__ R upwind_sel(bool neg, const R& a, const R& b)
 // two faces).  Plain FP64 takes one division for both terms (its pipe issues
 // one warp instruction per 16 cycles and SM, a division is about nine);
 // there the product of two smoothness squares cannot leave the range, in
-// FP32 it can.  CENTRED: `near` selects the centred 2nd-order derivative.
+// FP32 it can.  CENTRED: `near` selects the centred 2nd-order derivative
+// (any_near: false, uniformly over the warp, when no lane does).
 template <bool CENTRED, typename R, typename N>
-__device__ __forceinline__ R conv_deriv(const R* v, N neg, R eps, bool near)
+__device__ __forceinline__ R conv_deriv(const R* v, N neg, R eps, bool near, bool any_near)
 {
     using Sc = scalar_t<R>;
     const R a = upwind_sel(neg, v[4], v[0]), b = upwind_sel(neg, v[3], v[1]), d = upwind_sel(neg, v[1], v[3]);
@@ -276,8 +277,10 @@ __device__ __forceinline__ R conv_deriv(const R* v, N neg, R eps, bool near)
     if constexpr (std::is_same<R, double>::value) w = fdiv((s - q) * d0 + (q - p) * d1, d1 * d0);
     else w = R(s - q) * frcp(d1) + R(q - p) * frcp(d0);
     const R r = q + R(R(Sc(0.5)) * B) * w;
-    if constexpr (CENTRED) return near ? R(R(Sc(0.5)) * (d - b)) : r;
-    else return r;
+    if constexpr (CENTRED) {
+        if (any_near) return near ? R(R(Sc(0.5)) * (d - b)) : r;
+    }
+    return r;
 }
 
 // Sums of the FD terms over the axes: T's convective and non-convective
@@ -315,7 +318,8 @@ struct FDAccum {
 // the same result.  37 FP32 instructions per species and axis
 // instead of 58 (counted).  a12 = D_k / 12 (W_k cancels against the Y_k W lines).
 template <bool CENTRED, typename R, typename PR, typename LRho, typename LT, typename LW, typename LX, typename LY>
-__device__ __forceinline__ void fd_axis(const StepParams<PR>& P, R u_a, R invW0, R inv_rho0, bool near, LRho line_rho,
+__device__ __forceinline__ void fd_axis(const StepParams<PR>& P, R u_a, R invW0, R inv_rho0, bool near, bool any_near,
+                                        LRho line_rho,
                                         LT line_T, LW line_invW, LX line_X, LY line_Y, R* gam_a, FDAccum<R>& acc)
 {
     using Sc = scalar_t<R>;
@@ -327,7 +331,7 @@ __device__ __forceinline__ void fd_axis(const StepParams<PR>& P, R u_a, R invW0,
     const R gam = R(fd_D1(v)) * R(inv_rho0 * twelfth);
     *gam_a = gam;
     line_T(v);
-    acc.conv_T += mul_rn(ua, conv_deriv<CENTRED>(v, neg, R(P.epsT), near));
+    acc.conv_T += mul_rn(ua, conv_deriv<CENTRED>(v, neg, R(P.epsT), near, any_near));
     acc.diff_T += mul_rn(R(P.alpha12), R(fd_D2(v) + gam * fd_D1(v)));
     line_invW(v);
     const R dinvW = R(fd_D1(v)) * twelfth;
@@ -351,7 +355,7 @@ __device__ __forceinline__ void fd_axis(const StepParams<PR>& P, R u_a, R invW0,
 #pragma unroll
     for (int k = 0; k < NSP; ++k) {
         line_Y(k, v);
-        const R L = conv_deriv<CENTRED>(v, neg, R(P.epsY), near);
+        const R L = conv_deriv<CENTRED>(v, neg, R(P.epsY), near, any_near);
         sumL += L;
         acc.rhs_Y[k] += R(R(f[k] - M12 * fd_D1(v)) - ua * L);
     }

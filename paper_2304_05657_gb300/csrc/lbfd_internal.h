@@ -76,11 +76,15 @@ struct BoundaryLists {
     const unsigned long long* wall_code;  // 3-D: their neighbourhood codes (cell_step_coded)
     const long long* face_coded;  // 3-D: cells near inlet/outlet faces taken by cell_step_coded<FACES>
     long long nface_coded;        // (then `face` holds the other cells near faces)
+    long long nface_tile;         // the first of them, which the tile kernel leaves to the list
     const unsigned long long* face_code;
     // 2-D, staircase walls: `all` and `face` split into the cells that
     // cell_step_coded takes (list_codes2d) and the rest (general form)
     CodedList all2, face2;
-    const uint8_t* interior;  // per cell, 1 for the cells the interior tile kernels update
+    const uint8_t* interior;  // 2-D, per cell: 1 for the cells the interior tile kernels update
+    // 3-D, per cell: 0 interior, the neighbourhood code of a coded cell (bit
+    // 63 set for those near open faces), ~0 for the others
+    const unsigned long long* words;
     void* aux;                // 3-D: 4 planes of the compute type for the split variants
 };
 

@@ -38,7 +38,7 @@ struct StepParams {
     R omega_s, omega_b, omega_hi;
     R u_in, T_in, Y_in[NSP], invW_in, rho_in;
     R rho_c, inv_rho_c;  // EOS: rho = rho_c / (T invW), rho_c = T_in invW_in
-    R T_solid;
+    R T_solid, rho_solid;  // rho_solid = rho_c / T_solid
     int solid_isothermal;
     int poiseuille;
     R epsY, epsT;

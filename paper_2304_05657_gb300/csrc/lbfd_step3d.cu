@@ -14,26 +14,37 @@ struct Tile3Shape {
     static constexpr int TX = sizeof(R) == 8 ? 16 : 32, TY = 128 / TX;
 };
 
-// z-planes a block marches through, at most zmax: the cost of a launch is
-// (planes + the ring's fill of 4 staged planes, ~0.15 of a plane's work
-// each) times the larger of the blocks of the fullest SM (its issue slots or
-// FP64 pipe are shared) and the waves of resident blocks times the factor by
-// which a block alone on an SM is slower than its share of a full one.
-// Without it a 101x53x47 FP64 grid ran as 168 blocks of 16 planes (two on
-// 16 of the 152 SMs), a 128x64x64 FP32 grid as 128 of 32 planes or 256 of
-// 16; now as 147 of 16 and 512 of 8.
+// z-planes a block marches through, at most zmax.  Few planes per block
+// balance the SMs and keep their blocks resident together; each block pays
+// for 4 staged planes more (~0.25 of a plane's work each).  A step is
+// modelled from the measured us per plane of 1 .. R blocks sharing an SM (R
+// resident): blocks in rounds of R on the fullest SM, or, with many rounds,
+// the steady rate and half a round of tail.  Measured us per step over z:
+//   128x64x64 FP32:   4: 91   7: 85   8: 94  16: 140  32: 209  64: 405
+//   256x128x128 FP32: 4: 517  8: 504 11: 493 16: 531  32: 598  64: 694
+//   101x53x47 FP64:   4: 945  8: 939 16: 1049 32: 2085
+//   128x64x64 FP64:   5: 1686 7: 1647 8: 1861 16: 1989 32: 2099
 static int planes_per_block(bool fp64, long long columns, int nz, int zmax)
 {
-    const double fill = 4 * 0.15, alone = fp64 ? 1.3 : 2.3;
-    const long long sms = 152, resident = sms * (fp64 ? 2 : 4);
+    static const double us32[] = {0.0, 6.4, 7.9, 9.4, 10.9}, us64[] = {0.0, 63.0, 109.0};
+    const double* us = fp64 ? us64 : us32;
+    const int R = fp64 ? 2 : 4;
+    const double steady = fp64 ? 109.0 : 8.4, sms = 152.0, fill = 4 * 0.25;
     int best = 1;
     double cost = 1e300;
     for (int z = nz < zmax ? nz : zmax; z >= 1; --z) {
-        const long long blocks = columns * ((nz + z - 1) / z);
-        const double c = (z + fill) * fmax((double)((blocks + sms - 1) / sms),
-                                           alone * (double)((blocks + resident - 1) / resident));
-        if (c < cost * 0.999) {
-            cost = c;
+        const double n = (double)columns * nz / z / sms;  // blocks per SM
+        double t;
+        if (n > 2 * R) {
+            t = (n / R * steady + 0.5 * us[R]) * (z + fill);
+        } else {  // whole pieces, then the last, shorter ones
+            const int full = (int)ceil((double)columns * (nz / z) / sms);
+            const int all = (int)ceil((double)columns * ((nz + z - 1) / z) / sms);
+            auto rounds = [&](int k) { return k / R * us[R] + us[k % R]; };
+            t = rounds(full) * (z + fill) + (rounds(all) - rounds(full)) * (nz % z + fill);
+        }
+        if (t < cost * 0.999) {
+            cost = t;
             best = z;
         }
     }
@@ -46,36 +57,32 @@ static int planes_per_block(bool fp64, long long columns, int nz, int zmax)
 // other cells near domain faces (b.face), and the cells next to in-domain
 // solids (b.wall) go through their coded neighbourhoods (or, with curved
 // walls, the general form with the face rules compiled out).
-// the tile kernel instance: MINB > 0 caps its registers for MINB blocks per SM
-template <typename S, typename R, int TX, int TY, int MINB, bool HI1>
-static auto tile3_kernel()
-{
-    if constexpr (MINB > 0) return step_kernel_tiled3d_capped<S, R, TX, TY, MINB, HI1>;
-    else return step_kernel_tiled3d<S, R, TX, TY, HI1>;
-}
-
 // SPLIT: the tile kernel does a1-a7 and a per-cell kernel a8-a10 (two
 // smaller kernels instead of one; Lambda and grad rho pass through aux)
-// WALLS: the wall-aware tile kernel also updates the cells next to
-// in-domain solids, so the wall list runs only with curved walls
-template <bool HI1, typename S, typename R, int MINB = 0, bool SPLIT = false, bool WALLS = false>
-static cudaError_t launch_t3(int zmax, const StepParams<R>& P, StateView in, StateView out, const uint8_t* solid,
+// Otherwise the tile kernel updates the coded cells too, next to in-domain
+// solids and (faces) near inlet and outlet faces; with curved walls both
+// go through the general form.
+// MINB: resident blocks per SM.  FP32: four (128 registers) when the
+// collision needs only the low moments, else three; FP64: two.
+template <bool HI1, typename S, typename R, int MINB, bool SPLIT = false>
+static cudaError_t launch_t3(int zmax, bool faces, const StepParams<R>& P, StateView in, StateView out, const uint8_t* solid,
                              const BoundaryLists& bin, const SideStream& side, cudaStream_t stream)
 {
     constexpr int TX = Tile3Shape<R>::TX, TY = Tile3Shape<R>::TY;
     constexpr size_t smem = tile3_smem_bytes<R, TX, TY>();
-    auto kern = tile3_kernel<S, R, TX, TY, MINB, HI1>();
+    auto kern = step_kernel_tiled3d<S, R, TX, TY, MINB, HI1>;
     auto fkern = step_kernel_fd3d<S, R, TX, TY>;
-    auto wkern = step_kernel_tiled3d_walls<S, R, TX, TY, HI1>;
     auto fcode = step_kernel_wallcode<3, S, R, true, HI1>;
     auto wcode = step_kernel_wallcode<3, S, R, false, HI1>;
-    cudaError_t e = SPLIT   ? cudaFuncSetAttribute(fkern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                    : WALLS ? cudaFuncSetAttribute(wkern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                            : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = SPLIT ? cudaFuncSetAttribute(fkern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                          : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    if (bin.interior == nullptr || (SPLIT && bin.aux == nullptr)) return cudaErrorInvalidValue;
+    if (bin.words == nullptr || (SPLIT && bin.aux == nullptr)) return cudaErrorInvalidValue;
     BoundaryLists b = bin;
-    if (WALLS && !P.curved) b.nwall = 0;
+    if (!SPLIT && !P.curved) {
+        b.nwall = 0;
+        if (faces) b.nface_coded = b.nface_tile;
+    }
     const bool fork = (b.nface > 0 || b.nface_coded > 0 || b.nwall > 0) && side.stream != nullptr;
     if (fork) {
         if ((e = cudaEventRecord(side.fork, stream)) != cudaSuccess) return e;
@@ -113,16 +120,13 @@ static cudaError_t launch_t3(int zmax, const StepParams<R>& P, StateView in, Sta
     grid.z = (P.nz + zc - 1) / zc;
     if constexpr (SPLIT) {
         fkern<<<grid, dim3(TX, TY), smem, stream>>>(P, zc, (const S*)in.g, (const S*)in.T, (S*)out.T, (const S*)in.Y,
-                                                    (S*)out.Y, b.interior, (R*)b.aux);
+                                                    (S*)out.Y, b.words, (R*)b.aux);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         step_kernel_collide3d<S, R, HI1><<<dim3((P.nx + 127) / 128, P.ny, P.nz), 128, 0, stream>>>(
-            P, (const S*)in.g, (S*)out.g, (const S*)in.T, (const S*)in.Y, b.interior, (const R*)b.aux);
-    } else if constexpr (WALLS) {
-        wkern<<<grid, dim3(TX, TY), smem, stream>>>(P, zc, (const S*)in.g, (S*)out.g, (const S*)in.T, (S*)out.T,
-                                                    (const S*)in.Y, (S*)out.Y, b.interior, solid);
+            P, (const S*)in.g, (S*)out.g, (const S*)in.T, (const S*)in.Y, b.words, (const R*)b.aux);
     } else {
         kern<<<grid, dim3(TX, TY), smem, stream>>>(P, zc, (const S*)in.g, (S*)out.g, (const S*)in.T, (S*)out.T,
-                                                   (const S*)in.Y, (S*)out.Y, b.interior);
+                                                   (const S*)in.Y, (S*)out.Y, b.words, P.curved ? 0 : (faces ? 2 : 1));
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (fork) {
@@ -138,18 +142,19 @@ static cudaError_t launch_3d_tiles(int variant, const StepParams<R>& P, StateVie
                                    const uint8_t* solid, const BoundaryLists& b, const SideStream& side,
                                    cudaStream_t stream)
 {
+    constexpr int MINB = sizeof(R) == 8 ? 2 : (HI1 ? 4 : 3);
     switch (variant) {
-    case 1: return launch_t3<HI1, S, R>(16, P, in, out, solid, b, side, stream);
-    case 2: return launch_t3<HI1, S, R>(32, P, in, out, solid, b, side, stream);
+    case 1: return launch_t3<HI1, S, R, MINB>(16, true, P, in, out, solid, b, side, stream);
+    case 2: return launch_t3<HI1, S, R, MINB>(32, true, P, in, out, solid, b, side, stream);
     // variant 3: as 1 with the registers capped for four blocks per SM (FP32)
-    case 3: return launch_t3<HI1, S, R, sizeof(R) == 4 ? 4 : 0>(16, P, in, out, solid, b, side, stream);
+    case 3: return launch_t3<HI1, S, R, sizeof(R) == 4 ? 4 : 2>(16, true, P, in, out, solid, b, side, stream);
     // variants 4, 5: as 1, 2 split into an FD tile kernel and a collision kernel
-    case 4: return launch_t3<HI1, S, R, 0, true>(16, P, in, out, solid, b, side, stream);
-    case 5: return launch_t3<HI1, S, R, 0, true>(32, P, in, out, solid, b, side, stream);
-    // variants 6, 7: as 1, 2 with the cells next to in-domain solids in the
-    // tile kernel (wall-aware), no wall list
-    case 6: return launch_t3<HI1, S, R, 0, false, true>(16, P, in, out, solid, b, side, stream);
-    case 7: return launch_t3<HI1, S, R, 0, false, true>(32, P, in, out, solid, b, side, stream);
+    case 4: return launch_t3<HI1, S, R, MINB, true>(16, false, P, in, out, solid, b, side, stream);
+    case 5: return launch_t3<HI1, S, R, MINB, true>(32, false, P, in, out, solid, b, side, stream);
+    // variants 6, 7: as 1, 2 with the cells near open faces in a list kernel
+    // of their own
+    case 6: return launch_t3<HI1, S, R, MINB>(16, false, P, in, out, solid, b, side, stream);
+    case 7: return launch_t3<HI1, S, R, MINB>(32, false, P, in, out, solid, b, side, stream);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -311,7 +311,7 @@ __device__ __forceinline__ void fd_axis_points(const StepParams<R>& P, R u_a, in
         for (int j = 0; j < 5; ++j) v[j] = f[j];
     };
     fd_axis<true, R>(
-        P, u_a, invW0, inv_rho0, near != 0, [&](R* v) { copy(rhol, v); }, [&](R* v) { copy(Tl, v); },
+        P, u_a, invW0, inv_rho0, near != 0, true, [&](R* v) { copy(rhol, v); }, [&](R* v) { copy(Tl, v); },
         [&](R* v) { copy(invWl, v); },
         [&](int k, R* v) {
 #pragma unroll

@@ -65,7 +65,7 @@ __device__ __forceinline__ void fd_axis_tile(const StepParams<PR>& P, const Tile
                                              int a, R u_a, R invW0, R inv_rho0, FDAccum<R>& acc)
 {
     fd_axis<false, R>(
-        P, u_a, invW0, inv_rho0, false, [&](R* v) { line(sm.rho, v); }, [&](R* v) { line(sm.T, v); },
+        P, u_a, invW0, inv_rho0, false, false, [&](R* v) { line(sm.rho, v); }, [&](R* v) { line(sm.T, v); },
         [&](R* v) { line(sm.invW, v); }, [&](int k, R* v) { line(sm.X + k * npt, v); },
         [&](int k, R* v) { line(sm.Y + k * npt, v); }, &acc.gam[a], acc);
 }
@@ -113,7 +113,7 @@ __device__ __forceinline__ void fd_axis_smem_walls(const StepParams<R>& P, const
         }
     };
     fd_axis<true, R>(
-        P, u_a, invW0, inv_rho0, ghost != 0, line_rho, line_T, [&](R* v) { line(sm.invW, v); },
+        P, u_a, invW0, inv_rho0, ghost != 0, true, line_rho, line_T, [&](R* v) { line(sm.invW, v); },
         [&](int k, R* v) { line(sm.X + k * npt, v); }, [&](int k, R* v) { line(sm.Y + k * npt, v); }, &acc.gam[a],
         acc);
 }
