@@ -16,7 +16,7 @@ struct Tile3Shape {
 
 // z-planes a block marches through, at most zmax.  Few planes per block
 // balance the SMs and keep their blocks resident together; each block pays
-// for 4 staged planes more (~0.25 of a plane's work each).  A step is
+// for 4 staged planes more (~0.2 of a plane's work each).  A step is
 // modelled from the measured us per plane of 1 .. R blocks sharing an SM (R
 // resident): blocks in rounds of R on the fullest SM, or, with many rounds,
 // the steady rate and half a round of tail.  Measured us per step over z:
@@ -29,10 +29,10 @@ static int planes_per_block(bool fp64, long long columns, int nz, int zmax)
     static const double us32[] = {0.0, 6.4, 7.9, 9.4, 10.9}, us64[] = {0.0, 63.0, 109.0};
     const double* us = fp64 ? us64 : us32;
     const int R = fp64 ? 2 : 4;
-    const double steady = fp64 ? 109.0 : 8.4, sms = 152.0, fill = 4 * 0.25;
-    int best = 1;
-    double cost = 1e300;
-    for (int z = nz < zmax ? nz : zmax; z >= 1; --z) {
+    const double steady = fp64 ? 109.0 : 8.4, sms = 152.0, fill = 4 * 0.2;
+    const int top = nz < zmax ? nz : zmax, low = top < 4 ? top : 4;  // (fewer than 4 measured slower)
+    double cost[64], least = 1e300;
+    for (int z = low; z <= top; ++z) {
         const double n = (double)columns * nz / z / sms;  // blocks per SM
         double t;
         if (n > 2 * R) {
@@ -43,11 +43,11 @@ static int planes_per_block(bool fp64, long long columns, int nz, int zmax)
             auto rounds = [&](int k) { return k / R * us[R] + us[k % R]; };
             t = rounds(full) * (z + fill) + (rounds(all) - rounds(full)) * (nz % z + fill);
         }
-        if (t < cost * 0.999) {
-            cost = t;
-            best = z;
-        }
+        cost[z] = t;
+        least = t < least ? t : least;
     }
+    int best = low;  // the fewest planes within the model's accuracy
+    while (cost[best] > 1.02 * least) ++best;
     return best;
 }
 
