@@ -470,7 +470,8 @@ int lbfd_create(const lbfd_grid* grid, const uint8_t* solid_mask, const lbfd_mec
         }
     }
     if ((e = cudaMalloc(&h->solid, (size_t)h->ncell)) != cudaSuccess ||
-        (e = cudaMalloc(&h->red, lbfd::RED_WORDS * sizeof(double))) != cudaSuccess ||
+        (e = cudaMalloc(&h->red, (lbfd::RED_WORDS + lbfd::DIAG_WORDS) * sizeof(double))) != cudaSuccess ||
+        (e = cudaMemset(h->red, 0, lbfd::RED_WORDS * sizeof(double))) != cudaSuccess ||
         (e = cudaMalloc(&h->tmp, (size_t)h->ncell * sizeof(double))) != cudaSuccess) {
         free_handle(h);
         cuda_fail(e, "cudaMalloc");
@@ -982,7 +983,8 @@ int lbfd_diagnostics_rows(lbfd_handle* h, int y0, int y1, double* out)
     NvtxRange nvtx_("lbfd_diagnostics");
     if (!h || !out || y0 < 0 || y1 > h->grid.ny || y0 >= y1) return LBFD_EINVAL;
     double r[lbfd::RED_WORDS];
-    CK(lbfd::launch_diagnostics(h->dim, h->precision, h->Pd, view(h, h->cur), h->solid, y0, y1, h->red, h->stream));
+    CK(lbfd::launch_diagnostics(h->dim, h->precision, h->Pd, view(h, h->cur), h->solid, y0, y1, h->red,
+                                h->red + lbfd::RED_WORDS, h->stream));
     CK(cudaMemcpyAsync(r, h->red, sizeof r, cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     unsigned long long u[lbfd::RED_WORDS];
@@ -1017,8 +1019,9 @@ int lbfd_column_peaks(lbfd_handle* h, int y0, int y1, double* peak, double* wall
     const int nx = h->grid.nx;
     double* out = h->tmp;
     double* own = nullptr;
-    if (h->ncell < 2LL * nx) {  // a one-row grid: tmp holds nx values only
-        if (cudaMalloc((void**)&own, 2 * (size_t)nx * sizeof(double)) != cudaSuccess) return LBFD_ENOMEM;
+    const size_t need = lbfd::column_peaks_words(nx, y0, y1);
+    if ((size_t)h->ncell < need) {  // a few rows: the read-out buffer holds one value per cell
+        if (cudaMalloc((void**)&own, need * sizeof(double)) != cudaSuccess) return LBFD_ENOMEM;
         out = own;
     }
     std::vector<double> r(2 * (size_t)nx);
@@ -1725,7 +1728,7 @@ extern "C" int lbfd_diagnostics_noalloc(const lbfd_grid* grid, const lbfd_mechan
     v.Y = const_cast<void*>(Y);
     cudaStream_t s = (cudaStream_t)stream;
     // launch_diagnostics clears the words it accumulates into before use
-    CK(lbfd::launch_diagnostics(tmp.dim, tmp.precision, P, v, solid, 0, tmp.grid.ny, (double*)red, s));
+    CK(lbfd::launch_diagnostics(tmp.dim, tmp.precision, P, v, solid, 0, tmp.grid.ny, (double*)red, nullptr, s));
     double r[lbfd::RED_WORDS];
     CK(cudaMemcpyAsync(r, red, sizeof r, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));

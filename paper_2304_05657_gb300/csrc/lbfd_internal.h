@@ -135,14 +135,17 @@ void boundary_cells(int dim, int nx, int ny, int nz, const int* bc, const uint8_
                     bool faces_only, const int* face_solid);
 
 // Diagnostics reduction over the rows y0 <= y < y1 (all x, all z) into the
-// device scratch `red` (RED_WORDS words, zeroed by the launcher); FP64
-// accumulation.
+// device scratch `red` (RED_WORDS words); FP64 accumulation.  part: DIAG_WORDS
+// more words for sums in a fixed order (red's word 10 zero before the first
+// call), or null (atomic sums; red zeroed by the launcher).
 cudaError_t launch_diagnostics(int dim, int precision, const StepParams<double>& Pd, StateView st,
-                               const uint8_t* solid, int y0, int y1, double* red, cudaStream_t stream);
+                               const uint8_t* solid, int y0, int y1, double* red, double* part,
+                               cudaStream_t stream);
 
 // Column peaks of the heat release over rows y0 <= y < y1 of a 2-D grid
 // (FP64 or mixed state): out[x] = peak, out[nx + x] = its distance to the
-// nearer band edge (device, 2 nx doubles).
+// nearer band edge (device, column_peaks_words doubles: the rest is scratch).
+size_t column_peaks_words(int nx, int y0, int y1);
 cudaError_t launch_column_peaks(int precision, const StepParams<double>& P, StateView st, const uint8_t* solid,
                                 int y0, int y1, double* out, cudaStream_t stream);
 
@@ -244,5 +247,8 @@ cudaError_t launch_step_persistent(int precision, const StepParams<double>& Pd, 
 
 // Number of words of the reduction scratch.
 constexpr int RED_WORDS = 16;
+// Blocks of the diagnostics reduction (eight 256-thread blocks per SM), and
+// the words of their sums.
+constexpr int DIAG_BLOCKS = 152 * 8, DIAG_WORDS = 8 * DIAG_BLOCKS;
 
 }  // namespace lbfd

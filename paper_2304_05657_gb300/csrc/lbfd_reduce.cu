@@ -34,96 +34,11 @@ __device__ __forceinline__ double hrr_of(const StepParams<double>& P, double T, 
     return rho * P.Q_cp * q;
 }
 
-// red layout: [0] sum Y_F, [1] mass, [2] hrr, [3] fuel, [4] max-T key (u64),
-// [5] non-finite count (u64), [6] fluid count (u64), [7] x=0 section count (u64),
-// [8] centre-line max hrr, [9] its x
+// Heat-release maximum on the line y = (y0 + y1)/2, z = nz/2 by one block of
+// 256 threads: red[8] = value, red[9] = its x (the smaller on ties).
 template <int DIM, typename S>
-__global__ void __launch_bounds__(256) diag_kernel(StepParams<double> P, const S* __restrict__ g,
-                                                   const S* __restrict__ T, const S* __restrict__ Y,
-                                                   const uint8_t* __restrict__ solid, int y0, int y1, double* red)
-{
-    constexpr int Q = DIM == 2 ? 9 : 27;
-    double s[4] = {0.0, 0.0, 0.0, 0.0};
-    unsigned long long tkey = 0ull, nonf = 0ull, nfl = 0ull, sec = 0ull;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    const int rows = y1 - y0;
-    const long long ncount = (long long)P.nx * rows * P.nz;  // cells with y0 <= y < y1
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < ncount; t += stride) {
-        const long long r = t / P.nx;
-        const long long c = t % P.nx + (long long)P.nx * (y0 + r % rows + (long long)P.ny * (r / rows));
-        if (solid[c]) continue;
-        ++nfl;
-        if (c % P.nx == 0) ++sec;
-        const double Tc = val(T[c]);
-        double Yc[NSP];
-        bool bad = !isfinite(Tc);
-#pragma unroll
-        for (int k = 0; k < NSP; ++k) {
-            Yc[k] = val(Y[(long long)k * P.N + c]);
-            bad |= !isfinite(Yc[k]);
-        }
-#pragma unroll
-        for (int i = 0; i < Q; ++i) bad |= !isfinite(val(g[(long long)i * P.N + c]));
-        if (bad) {
-            ++nonf;
-            continue;
-        }
-        double rho, q;
-        const double h = hrr_of<S>(P, Tc, Yc, &rho, &q);
-        s[0] += Yc[P.fuel];
-        s[1] += rho;
-        s[2] += h;
-        s[3] += rho * q;
-        const unsigned long long k = order_key(Tc);
-        tkey = k > tkey ? k : tkey;
-    }
-    // warp then block reduction
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) s[j] += __shfl_down_sync(0xffffffffu, s[j], off);
-        const unsigned long long o = __shfl_down_sync(0xffffffffu, tkey, off);
-        tkey = o > tkey ? o : tkey;
-        nonf += __shfl_down_sync(0xffffffffu, nonf, off);
-        nfl += __shfl_down_sync(0xffffffffu, nfl, off);
-        sec += __shfl_down_sync(0xffffffffu, sec, off);
-    }
-    __shared__ double sh[8][4];
-    __shared__ unsigned long long shk[8][4];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) sh[wid][j] = s[j];
-        shk[wid][0] = tkey;
-        shk[wid][1] = nonf;
-        shk[wid][2] = nfl;
-        shk[wid][3] = sec;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const int nw = blockDim.x >> 5;
-        for (int w = 1; w < nw; ++w) {
-            for (int j = 0; j < 4; ++j) s[j] += sh[w][j];
-            tkey = shk[w][0] > tkey ? shk[w][0] : tkey;
-            nonf += shk[w][1];
-            nfl += shk[w][2];
-            sec += shk[w][3];
-        }
-        for (int j = 0; j < 4; ++j) atomicAdd(&red[j], s[j]);
-        unsigned long long* ru = reinterpret_cast<unsigned long long*>(red);
-        atomicMax(&ru[4], tkey);
-        atomicAdd(&ru[5], nonf);
-        atomicAdd(&ru[6], nfl);
-        atomicAdd(&ru[7], sec);
-    }
-}
-
-// one block: argmax of the heat release on the line y = ny/2, z = nz/2
-template <int DIM, typename S>
-__global__ void __launch_bounds__(1024) centreline_kernel(StepParams<double> P, const S* __restrict__ T,
-                                                          const S* __restrict__ Y,
-                                                          const uint8_t* __restrict__ solid, int y0, int y1,
-                                                          double* red)
+__device__ void centreline(const StepParams<double>& P, const S* __restrict__ T, const S* __restrict__ Y,
+                           const uint8_t* __restrict__ solid, int y0, int y1, double* red)
 {
     double best = -INFINITY;
     int bx = -1;
@@ -177,38 +92,168 @@ __global__ void __launch_bounds__(1024) centreline_kernel(StepParams<double> P, 
     }
 }
 
+// red layout: [0] sum Y_F, [1] mass, [2] hrr, [3] fuel, [4] max-T key (u64),
+// [5] non-finite count (u64), [6] fluid count (u64), [7] x=0 section count (u64),
+// [8] centre-line max hrr, [9] its x, [10] count of finished blocks (u32,
+// back to 0 at the end).  With `part` (8 words per block) the block sums are
+// stored there and the last block adds them in block order, so that the
+// result does not depend on the order in which blocks finish; without it
+// (the fixed scratch of the allocation-free form) they are added to `red`
+// atomically.  The last block also scans the centre line: one launch.
+template <int DIM, typename S>
+__global__ void __launch_bounds__(256) diag_kernel(StepParams<double> P, const S* __restrict__ g,
+                                                   const S* __restrict__ T, const S* __restrict__ Y,
+                                                   const uint8_t* __restrict__ solid, int y0, int y1, double* red,
+                                                   double* part)
+{
+    constexpr int Q = DIM == 2 ? 9 : 27;
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    unsigned long long tkey = 0ull, nonf = 0ull, nfl = 0ull, sec = 0ull;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    const int rows = y1 - y0;
+    const long long ncount = (long long)P.nx * rows * P.nz;  // cells with y0 <= y < y1
+    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < ncount; t += stride) {
+        const long long r = t / P.nx;
+        const long long c = t % P.nx + (long long)P.nx * (y0 + r % rows + (long long)P.ny * (r / rows));
+        if (solid[c]) continue;
+        ++nfl;
+        if (c % P.nx == 0) ++sec;
+        const double Tc = val(T[c]);
+        double Yc[NSP];
+        bool bad = !isfinite(Tc);
+#pragma unroll
+        for (int k = 0; k < NSP; ++k) {
+            Yc[k] = val(Y[(long long)k * P.N + c]);
+            bad |= !isfinite(Yc[k]);
+        }
+#pragma unroll
+        for (int i = 0; i < Q; ++i) bad |= !isfinite(val(g[(long long)i * P.N + c]));
+        if (bad) {
+            ++nonf;
+            continue;
+        }
+        double rho, q;
+        const double h = hrr_of<S>(P, Tc, Yc, &rho, &q);
+        s[0] += Yc[P.fuel];
+        s[1] += rho;
+        s[2] += h;
+        s[3] += rho * q;
+        const unsigned long long k = order_key(Tc);
+        tkey = k > tkey ? k : tkey;
+    }
+    // warp then block reduction
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s[j] += __shfl_down_sync(0xffffffffu, s[j], off);
+        const unsigned long long o = __shfl_down_sync(0xffffffffu, tkey, off);
+        tkey = o > tkey ? o : tkey;
+        nonf += __shfl_down_sync(0xffffffffu, nonf, off);
+        nfl += __shfl_down_sync(0xffffffffu, nfl, off);
+        sec += __shfl_down_sync(0xffffffffu, sec, off);
+    }
+    __shared__ double sh[8][4];
+    __shared__ unsigned long long shk[8][4];
+    __shared__ bool last;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (lane == 0) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) sh[wid][j] = s[j];
+        shk[wid][0] = tkey;
+        shk[wid][1] = nonf;
+        shk[wid][2] = nfl;
+        shk[wid][3] = sec;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const int nw = blockDim.x >> 5;
+        for (int w = 1; w < nw; ++w) {
+            for (int j = 0; j < 4; ++j) s[j] += sh[w][j];
+            tkey = shk[w][0] > tkey ? shk[w][0] : tkey;
+            nonf += shk[w][1];
+            nfl += shk[w][2];
+            sec += shk[w][3];
+        }
+        unsigned long long* ru = reinterpret_cast<unsigned long long*>(red);
+        if (part) {
+            double* pb = part + 8 * (size_t)blockIdx.x;
+            unsigned long long* pu = reinterpret_cast<unsigned long long*>(pb);
+            for (int j = 0; j < 4; ++j) pb[j] = s[j];
+            pu[4] = tkey;
+            pu[5] = nonf;
+            pu[6] = nfl;
+            pu[7] = sec;
+        } else {
+            for (int j = 0; j < 4; ++j) atomicAdd(&red[j], s[j]);
+            atomicMax(&ru[4], tkey);
+            atomicAdd(&ru[5], nonf);
+            atomicAdd(&ru[6], nfl);
+            atomicAdd(&ru[7], sec);
+        }
+        __threadfence();  // this block's sums before its count
+        last = atomicInc(reinterpret_cast<unsigned*>(&red[10]), gridDim.x - 1) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (part) {
+        // word j = thread % 8 of a run of consecutive blocks per thread, the 32
+        // runs then joined in order
+        __shared__ unsigned long long run[32][8];
+        const int j = threadIdx.x & 7, r = threadIdx.x >> 3;
+        const unsigned len = (gridDim.x + 31) / 32;
+        const unsigned long long* pu = reinterpret_cast<const unsigned long long*>(part) + j;
+        auto join = [&](double& d, unsigned long long& u, unsigned long long w) {
+            if (j < 4) d += __longlong_as_double((long long)w);
+            else if (j == 4) u = w > u ? w : u;
+            else u += w;
+        };
+        double d = 0.0;
+        unsigned long long u = 0ull;
+#pragma unroll 8
+        for (unsigned k = 0; k < len; ++k) {
+            const unsigned b = r * len + k;
+            if (b < gridDim.x) join(d, u, __ldcg(pu + 8 * (size_t)b));
+        }
+        run[r][j] = j < 4 ? (unsigned long long)__double_as_longlong(d) : u;
+        __syncthreads();
+        if (threadIdx.x < 8) {
+            d = 0.0;
+            u = 0ull;
+            for (int k = 0; k < 32; ++k) join(d, u, run[k][j]);
+            reinterpret_cast<unsigned long long*>(red)[j] = j < 4 ? (unsigned long long)__double_as_longlong(d) : u;
+        }
+    }
+    centreline<DIM, S>(P, T, Y, solid, y0, y1, red);
+}
+
 template <int DIM, typename S>
 static cudaError_t diag_launch(const StepParams<double>& P, StateView st, const uint8_t* solid, int y0, int y1,
-                               double* red, cudaStream_t stream)
+                               double* red, double* part, cudaStream_t stream)
 {
-    cudaError_t e = cudaMemsetAsync(red, 0, RED_WORDS * sizeof(double), stream);
-    if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    long long want = ((long long)P.nx * (y1 - y0) * P.nz + 255) / 256;
-    long long cap = (long long)(sms > 0 ? sms : 1) * 8;
-    const unsigned blocks = (unsigned)(want < cap ? (want > 0 ? want : 1) : cap);
+    if (!part) {
+        const cudaError_t e = cudaMemsetAsync(red, 0, RED_WORDS * sizeof(double), stream);
+        if (e != cudaSuccess) return e;
+    }
+    const long long want = ((long long)P.nx * (y1 - y0) * P.nz + 255) / 256;
+    const unsigned blocks = (unsigned)(want < DIAG_BLOCKS ? want : DIAG_BLOCKS);
     diag_kernel<DIM, S><<<blocks, 256, 0, stream>>>(P, (const S*)st.g, (const S*)st.T, (const S*)st.Y, solid, y0, y1,
-                                                    red);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    centreline_kernel<DIM, S><<<1, 1024, 0, stream>>>(P, (const S*)st.T, (const S*)st.Y, solid, y0, y1, red);
+                                                    red, part);
     return cudaGetLastError();
 }
 
 cudaError_t launch_diagnostics(int dim, int precision, const StepParams<double>& P, StateView st,
-                               const uint8_t* solid, int y0, int y1, double* red, cudaStream_t stream)
+                               const uint8_t* solid, int y0, int y1, double* red, double* part, cudaStream_t stream)
 {
     if (precision == 0)
-        return dim == 2 ? diag_launch<2, double>(P, st, solid, y0, y1, red, stream)
-                        : diag_launch<3, double>(P, st, solid, y0, y1, red, stream);
+        return dim == 2 ? diag_launch<2, double>(P, st, solid, y0, y1, red, part, stream)
+                        : diag_launch<3, double>(P, st, solid, y0, y1, red, part, stream);
     if (precision == 2)
-        return dim == 2 ? diag_launch<2, Tan>(P, st, solid, y0, y1, red, stream) : cudaErrorInvalidValue;
+        return dim == 2 ? diag_launch<2, Tan>(P, st, solid, y0, y1, red, part, stream) : cudaErrorInvalidValue;
     if (precision == 3)
-        return dim == 2 ? diag_launch<2, Tanf>(P, st, solid, y0, y1, red, stream) : cudaErrorInvalidValue;
-    return dim == 2 ? diag_launch<2, float>(P, st, solid, y0, y1, red, stream)
-                    : diag_launch<3, float>(P, st, solid, y0, y1, red, stream);
+        return dim == 2 ? diag_launch<2, Tanf>(P, st, solid, y0, y1, red, part, stream) : cudaErrorInvalidValue;
+    return dim == 2 ? diag_launch<2, float>(P, st, solid, y0, y1, red, part, stream)
+                    : diag_launch<3, float>(P, st, solid, y0, y1, red, part, stream);
 }
 
 // Per column x of a 2-D grid: the peak heat release over the fluid cells of
@@ -216,17 +261,24 @@ cudaError_t launch_diagnostics(int dim, int precision, const StepParams<double>&
 // IV.A) and the distance of that cell's centre to the nearer edge of the
 // row band (walls half-way between cells): out[x] = peak (0 when the column
 // has no fluid cell there), out[nx + x] = distance (smallest y on ties).
+// One warp per 32 columns and PEAK_ROWS rows (a cell's rate is about 70 FP64
+// instructions of 64 cycles: a thread per column took 70 to 230 us for 17 to
+// 65 rows), the chunks' maxima at part[chunk][2][nx]; then the maximum over
+// the chunks in row order.
+constexpr int PEAK_ROWS = 4;
 template <typename S>
-__global__ void __launch_bounds__(256) column_peaks_kernel(StepParams<double> P, const S* __restrict__ T,
-                                                           const S* __restrict__ Y,
-                                                           const uint8_t* __restrict__ solid, int y0, int y1,
-                                                           double* __restrict__ out)
+__global__ void __launch_bounds__(32) column_peaks_kernel(StepParams<double> P, const S* __restrict__ T,
+                                                          const S* __restrict__ Y,
+                                                          const uint8_t* __restrict__ solid, int y0, int y1,
+                                                          double* __restrict__ part)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned gx = (P.nx + 31) / 32;
+    const int x = (int)(blockIdx.x % gx) * 32 + threadIdx.x, chunk = (int)(blockIdx.x / gx);
     if (x >= P.nx) return;
+    const int ya = y0 + chunk * PEAK_ROWS, yb = ya + PEAK_ROWS < y1 ? ya + PEAK_ROWS : y1;
     double best = -1.0;
     int by = y0;
-    for (int y = y0; y < y1; ++y) {
+    for (int y = ya; y < yb; ++y) {
         const long long c = (long long)x + (long long)P.nx * y;
         if (solid[c]) continue;
         double Yc[NSP];
@@ -239,23 +291,48 @@ __global__ void __launch_bounds__(256) column_peaks_kernel(StepParams<double> P,
             by = y;
         }
     }
+    part[(size_t)(2 * chunk) * P.nx + x] = best;
+    part[(size_t)(2 * chunk + 1) * P.nx + x] = (double)by;
+}
+__global__ void __launch_bounds__(128) column_peaks_join_kernel(int nx, int chunks, int y0, int y1,
+                                                                const double* __restrict__ part,
+                                                                double* __restrict__ out)
+{
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= nx) return;
+    double best = -1.0, by = y0;
+    for (int j = 0; j < chunks; ++j) {
+        const double h = part[(size_t)(2 * j) * nx + x];
+        if (h > best) {
+            best = h;
+            by = part[(size_t)(2 * j + 1) * nx + x];
+        }
+    }
     const double d0 = by - y0 + 0.5, d1 = y1 - 0.5 - by;
     out[x] = best < 0.0 ? 0.0 : best;
-    out[P.nx + x] = d0 < d1 ? d0 : d1;
+    out[nx + x] = d0 < d1 ? d0 : d1;
 }
+
+static int peak_chunks(int y0, int y1) { return (y1 - y0 + PEAK_ROWS - 1) / PEAK_ROWS; }
+size_t column_peaks_words(int nx, int y0, int y1) { return (size_t)nx * (2 + 2 * (size_t)peak_chunks(y0, y1)); }
 
 cudaError_t launch_column_peaks(int precision, const StepParams<double>& P, StateView st, const uint8_t* solid,
                                 int y0, int y1, double* out, cudaStream_t stream)
 {
-    const unsigned nb = (unsigned)((P.nx + 255) / 256);
+    const int chunks = peak_chunks(y0, y1);
+    const unsigned grid = (unsigned)((P.nx + 31) / 32) * (unsigned)chunks;
+    double* part = out + 2 * (size_t)P.nx;
     if (precision == 0)
-        column_peaks_kernel<double><<<nb, 256, 0, stream>>>(P, (const double*)st.T, (const double*)st.Y, solid, y0,
-                                                            y1, out);
+        column_peaks_kernel<double><<<grid, 32, 0, stream>>>(P, (const double*)st.T, (const double*)st.Y, solid, y0,
+                                                             y1, part);
     else if (precision == 1)
-        column_peaks_kernel<float><<<nb, 256, 0, stream>>>(P, (const float*)st.T, (const float*)st.Y, solid, y0, y1,
-                                                           out);
+        column_peaks_kernel<float><<<grid, 32, 0, stream>>>(P, (const float*)st.T, (const float*)st.Y, solid, y0, y1,
+                                                            part);
     else
         return cudaErrorInvalidValue;
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    column_peaks_join_kernel<<<(unsigned)((P.nx + 127) / 128), 128, 0, stream>>>(P.nx, chunks, y0, y1, part, out);
     return cudaGetLastError();
 }
 
