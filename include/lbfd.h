@@ -62,8 +62,8 @@ extern "C" {
 #define LBFD_FP64 0  /* FP64 storage and arithmetic */
 #define LBFD_MIXED 1 /* FP32 storage and arithmetic; FP64 Arrhenius above T_fp64 */
 #define LBFD_TANGENT 2 /* FP64 values each carrying 4 derivatives (forward mode),
-                          with respect to theta = (ln A, Ta, T_wall, u_in); 2-D only,
-                          general-form kernel.  T_wall moves every isothermal wall face
+                          with respect to theta = (ln A, Ta, T_wall, u_in); 2-D only.
+                          T_wall moves every isothermal wall face
                           and, when solids are isothermal, T_solid together. */
 #define LBFD_TANGENT_MIXED 3 /* as LBFD_TANGENT with FP32 values and derivatives
                                 (FP32 forward), the Arrhenius rate and its derivatives

@@ -222,6 +222,8 @@ static StepParams<RevT<V>> rev_params(const StepParams<double>& D)
     P.omega_s = Rv(D.omega_s);
     P.omega_b = Rv(D.omega_b);
     P.omega_hi = Rv(D.omega_hi);
+    P.one_minus_omega_s = Rv(D.one_minus_omega_s);
+    P.omega_s_minus_b = Rv(D.omega_s_minus_b);
     P.alpha12 = Rv(D.alpha12);
     P.lam_yield = Rv(D.lam_yield);
     P.u_in = Rv(D.u_in, 3);

@@ -176,6 +176,8 @@ void fill_params(const lbfd_handle* h, StepParams<R>& P)
     P.omega_s = (R)omega_s;
     P.omega_b = (R)(p.omega_bulk > 0.0 ? p.omega_bulk : omega_s);
     P.omega_hi = (R)p.omega_hi;
+    P.one_minus_omega_s = (R)(1.0 - omega_s);
+    P.omega_s_minus_b = (R)(p.omega_bulk > 0.0 ? omega_s - p.omega_bulk : 0.0);
     P.alpha12 = (R)(alpha / 12.0);
     {
         double ly = 0.0;
@@ -395,9 +397,9 @@ cudaError_t launch_one(lbfd_handle* h, int from, int v, cudaStream_t s)
         if (e != cudaSuccess) return e;
     }
     if (h->precision == LBFD_TANGENT)
-        return lbfd::launch_step_tangent(h->dim, h->Pt, view(h, from), view(h, from ^ 1), h->solid, s);
+        return lbfd::launch_step_tangent(h->dim, h->Pt, view(h, from), view(h, from ^ 1), h->solid, lists(h), s);
     if (h->precision == LBFD_TANGENT_MIXED)
-        return lbfd::launch_step_tangent(h->dim, h->Ptf, view(h, from), view(h, from ^ 1), h->solid, s);
+        return lbfd::launch_step_tangent(h->dim, h->Ptf, view(h, from), view(h, from ^ 1), h->solid, lists(h), s);
     return launch_variant(h, v, view(h, from), view(h, from ^ 1), s);
 }
 
@@ -617,7 +619,7 @@ int lbfd_create(const lbfd_grid* grid, const uint8_t* solid_mask, const lbfd_mec
             return cuda_fail(e, "cell words");
         }
     }
-    if (h->dim == 2 && !is_tangent(h->precision)) {
+    if (h->dim == 2) {
         lbfd_handle::Coded2* dst[2] = {&h->bnd2, &h->bndf2};
         for (int j = 0; j < 2; ++j) {
             std::vector<long long> cells, rest;
@@ -814,6 +816,7 @@ int lbfd_launches_per_step(const lbfd_handle* h)
     if (!h) return -1;
     const lbfd::BoundaryLists b = lists(h);
     int n = 1;
+    if (is_tangent(h->precision) && h->prm.omega_hi == 1.0 && !h->Pd.curved && b.all2.nrest > 0) ++n;
     if (h->variant > 0 && !is_tangent(h->precision)) {
         if (h->dim == 3) {
             const bool split = h->variant == 4 || h->variant == 5;

@@ -9,7 +9,84 @@
 #pragma once
 #include <cmath>
 
+#include "lbfd_f2.cuh"
+
 namespace lbfd {
+
+// a constant: c * x, c + x cost one operation per derivative of x, where a
+// Dual factor without derivatives would cost two
+template <typename T>
+struct Cst {
+    T v;
+    constexpr __host__ __device__ explicit Cst(double x) : v(T(x)) {}
+};
+
+// Derivative vectors: r = s x, r = s x + t y, r += x, ... one operation per
+// derivative, or per two of them with the packed FP32 instructions.
+template <typename T, int N>
+struct Vec {
+    static __host__ __device__ __forceinline__ void scale(T* r, T s, const T* x)
+    {
+#pragma unroll
+        for (int k = 0; k < N; ++k) r[k] = s * x[k];
+    }
+    static __host__ __device__ __forceinline__ void comb(T* r, T s, const T* x, T t, const T* y)  // s x + t y
+    {
+#pragma unroll
+        for (int k = 0; k < N; ++k) r[k] = s * x[k] + t * y[k];
+    }
+    static __host__ __device__ __forceinline__ void axpy(T* r, T s, const T* x)  // r += s x
+    {
+#pragma unroll
+        for (int k = 0; k < N; ++k) r[k] += s * x[k];
+    }
+    static __host__ __device__ __forceinline__ void add(T* r, const T* x)
+    {
+#pragma unroll
+        for (int k = 0; k < N; ++k) r[k] += x[k];
+    }
+    static __host__ __device__ __forceinline__ void sub(T* r, const T* x)
+    {
+#pragma unroll
+        for (int k = 0; k < N; ++k) r[k] -= x[k];
+    }
+};
+#ifdef __CUDA_ARCH__
+template <>
+struct Vec<float, 4> {
+    static __device__ __forceinline__ float2 lo(const float* x) { return make_float2(x[0], x[1]); }
+    static __device__ __forceinline__ float2 hi(const float* x) { return make_float2(x[2], x[3]); }
+    static __device__ __forceinline__ float2 two(float s) { return make_float2(s, s); }
+    static __device__ __forceinline__ void put(float* r, float2 a, float2 b)
+    {
+        r[0] = a.x;
+        r[1] = a.y;
+        r[2] = b.x;
+        r[3] = b.y;
+    }
+    static __device__ __forceinline__ void scale(float* r, float s, const float* x)
+    {
+        put(r, __fmul2_rn(two(s), lo(x)), __fmul2_rn(two(s), hi(x)));
+    }
+    static __device__ __forceinline__ void comb(float* r, float s, const float* x, float t, const float* y)
+    {
+        put(r, __ffma2_rn(two(s), lo(x), __fmul2_rn(two(t), lo(y))),
+            __ffma2_rn(two(s), hi(x), __fmul2_rn(two(t), hi(y))));
+    }
+    static __device__ __forceinline__ void axpy(float* r, float s, const float* x)
+    {
+        put(r, __ffma2_rn(two(s), lo(x), lo(r)), __ffma2_rn(two(s), hi(x), hi(r)));
+    }
+    static __device__ __forceinline__ void add(float* r, const float* x)
+    {
+        put(r, __fadd2_rn(lo(r), lo(x)), __fadd2_rn(hi(r), hi(x)));
+    }
+    static __device__ __forceinline__ void sub(float* r, const float* x)
+    {
+        put(r, f2sub(lo(r), lo(x)), f2sub(hi(r), hi(x)));
+    }
+};
+#endif
 
 template <typename T, int N>
 struct Dual {
@@ -24,25 +101,23 @@ struct Dual {
         for (int k = 0; k < N; ++k) d[k] = T(0);
     }
     __host__ __device__ Dual(int x) : Dual(double(x)) {}
+    __host__ __device__ Dual(const Cst<T>& x) : Dual(double(x.v)) {}
 
     __host__ __device__ Dual& operator+=(const Dual& b)
     {
         v += b.v;
-#pragma unroll
-        for (int k = 0; k < N; ++k) d[k] += b.d[k];
+        Vec<T, N>::add(d, b.d);
         return *this;
     }
     __host__ __device__ Dual& operator-=(const Dual& b)
     {
         v -= b.v;
-#pragma unroll
-        for (int k = 0; k < N; ++k) d[k] -= b.d[k];
+        Vec<T, N>::sub(d, b.d);
         return *this;
     }
     __host__ __device__ Dual& operator*=(const Dual& b)
     {
-#pragma unroll
-        for (int k = 0; k < N; ++k) d[k] = d[k] * b.v + v * b.d[k];
+        Vec<T, N>::comb(d, b.v, d, v, b.d);
         v *= b.v;
         return *this;
     }
@@ -69,8 +144,7 @@ __host__ __device__ inline Dual<T, N> operator/(const Dual<T, N>& a, const Dual<
     Dual<T, N> r;
     const T inv = T(1) / b.v;
     r.v = a.v * inv;
-#pragma unroll
-    for (int k = 0; k < N; ++k) r.d[k] = (a.d[k] - r.v * b.d[k]) * inv;
+    Vec<T, N>::comb(r.d, inv, a.d, -r.v * inv, b.d);
     return r;
 }
 template <typename T, int N>
@@ -78,6 +152,41 @@ __host__ __device__ inline Dual<T, N>& operator/=(Dual<T, N>& a, const Dual<T, N
 {
     a = a / b;
     return a;
+}
+
+template <typename T, int N>
+struct ConstOf<Dual<T, N>> {
+    using type = Cst<T>;
+};
+template <typename T, int N>
+__host__ __device__ inline Dual<T, N> operator*(const Cst<T>& c, Dual<T, N> a)
+{
+    a.v *= c.v;
+    Vec<T, N>::scale(a.d, c.v, a.d);
+    return a;
+}
+template <typename T, int N>
+__host__ __device__ inline Dual<T, N> operator*(const Dual<T, N>& a, const Cst<T>& c) { return c * a; }
+template <typename T, int N>
+__host__ __device__ inline Dual<T, N> operator+(const Cst<T>& c, Dual<T, N> a)
+{
+    a.v += c.v;
+    return a;
+}
+template <typename T, int N>
+__host__ __device__ inline Dual<T, N> operator+(const Dual<T, N>& a, const Cst<T>& c) { return c + a; }
+template <typename T, int N>
+__host__ __device__ inline Dual<T, N> operator-(Dual<T, N> a, const Cst<T>& c)
+{
+    a.v -= c.v;
+    return a;
+}
+template <typename T, int N>
+__host__ __device__ inline Dual<T, N> operator-(const Cst<T>& c, const Dual<T, N>& a) { return c + (-a); }
+template <typename T>
+__host__ __device__ inline Cst<T> operator*(const Cst<T>& a, const Cst<T>& b)
+{
+    return Cst<T>((double)(a.v * b.v));
 }
 
 // comparisons act on the values

@@ -88,6 +88,21 @@ struct ScalarOf<F2> {
 template <typename R>
 using scalar_t = typename ScalarOf<R>::type;
 
+// the type of a constant that meets values of type R: R itself, except for
+// the forward-mode numbers, whose constants carry no derivatives
+// (lbfd_dual.cuh)
+template <typename R>
+struct ConstOf {
+    using type = R;
+};
+template <typename R>
+using const_t = typename ConstOf<R>::type;
+template <typename R>
+__host__ __device__ constexpr const_t<R> K(double x)
+{
+    return const_t<R>(x);
+}
+
 // upwind side per lane (the forms of upwind_neg, _abs and _sel for a pair)
 struct Neg2 {
     bool x, y;

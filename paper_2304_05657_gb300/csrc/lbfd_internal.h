@@ -160,9 +160,9 @@ cudaError_t launch_cells(int dim, int precision, const StepParams<double>& Pd, S
 // Dual<float, 4>; general form, 2-D), tangent read-out and objective
 // gradients (lbfd_tangent.cu).
 cudaError_t launch_step_tangent(int dim, const StepParams<Tan>& P, StateView in, StateView out, const uint8_t* solid,
-                                cudaStream_t stream);
+                                const BoundaryLists& b, cudaStream_t stream);
 cudaError_t launch_step_tangent(int dim, const StepParams<Tanf>& P, StateView in, StateView out, const uint8_t* solid,
-                                cudaStream_t stream);
+                                const BoundaryLists& b, cudaStream_t stream);
 cudaError_t launch_tangent_field(bool fp32, long long ncell, long long N, const void* state_base, int plane, int k,
                                  double* out, cudaStream_t stream);
 cudaError_t launch_objective(const StepParams<Tan>& P, StateView st, const uint8_t* solid, int objective,

@@ -36,6 +36,7 @@ struct StepParams {
     double A_lat_d, Ta_d;  // FP64 copies for the mixed-precision Arrhenius
     R T_fp64;
     R omega_s, omega_b, omega_hi;
+    R one_minus_omega_s, omega_s_minus_b;
     R u_in, T_in, Y_in[NSP], invW_in, rho_in;
     R rho_c, inv_rho_c;  // EOS: rho = rho_c / (T invW), rho_c = T_in invW_in
     R T_solid, rho_solid;  // rho_solid = rho_c / T_solid

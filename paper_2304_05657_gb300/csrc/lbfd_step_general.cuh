@@ -328,14 +328,14 @@ __device__ __forceinline__ R update_scalars(const StepParams<R>& P, long long c,
                                             bool store = true)
 {
     const R q = arrhenius(P, T0, pick_species(Y0, P.fuel), pick_species(Y0, P.oxid));
-    const R DT = acc.diff_T + P.Q_cp * q;
+    const R DT = acc.diff_T + par<R>(P.Q_cp) * q;
     if (store) {
         T_out[c] = S(T0 + (DT - acc.conv_T));
 #pragma unroll
         for (int k = 0; k < NSP; ++k)
-            Y_out[(long long)k * P.N + c] = S(Y0[k] + ((acc.rhs_Y[k] + Y0[k] * acc.along) + P.yield[k] * q));
+            Y_out[(long long)k * P.N + c] = S(Y0[k] + ((acc.rhs_Y[k] + Y0[k] * acc.along) + par<R>(P.yield[k]) * q));
     }
-    return DT * inv_T0 + (acc.lamY + P.lam_yield * q) * W0;
+    return DT * inv_T0 + (acc.lamY + par<R>(P.lam_yield) * q) * W0;
 }
 
 // ---------------------------------------------------------------------------
@@ -360,7 +360,7 @@ __device__ __forceinline__ void cell_step_general(const StepParams<R>& P, const 
     const R invW0 = inv_molar_mass(P, Y0);
     R rho0, W0;
     eos_w(P, T0, invW0, rho0, W0);
-    const R inv_rho0 = T0 * invW0 * P.inv_rho_c, inv_T0 = rho0 * invW0 * P.inv_rho_c;
+    const R inv_rho0 = T0 * invW0 * par<R>(P.inv_rho_c), inv_T0 = rho0 * invW0 * par<R>(P.inv_rho_c);
     // a1: a rolled loop (one copy of the boundary rules keeps this kernel
     // small enough for the instruction cache; the pulled values pass
     // through a local array)
@@ -384,7 +384,7 @@ __device__ __forceinline__ void cell_step_general(const StepParams<R>& P, const 
     low_moments<DIM>(g, lm);
     R u[3] = {R(0), R(0), R(0)};
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) u[a] = lm.m1[a] * (R(3) * inv_rho0);
+    for (int a = 0; a < DIM; ++a) u[a] = lm.m1[a] * (K<R>(3) * inv_rho0);
     // a3-a5
     FDAccum<R> acc;
     acc.clear();
@@ -623,19 +623,29 @@ __device__ __forceinline__ void cell_step_coded(const StepParams<R>& P, const in
     const R invW0 = inv_molar_mass(P, Y0);
     R rho0, W0;
     eos_w(P, T0, invW0, rho0, W0);
-    const R inv_rho0 = T0 * invW0 * P.inv_rho_c, inv_T0 = rho0 * invW0 * P.inv_rho_c;
+    const R inv_rho0 = T0 * invW0 * par<R>(P.inv_rho_c), inv_T0 = rho0 * invW0 * par<R>(P.inv_rho_c);
     R g[Q];
     pull_coded<DIM, S, R, FACES>(P, p, c, code, rho0, inv_rho0, g_in, g);
     LowMoments<DIM, R> lm;
     low_moments<DIM>(g, lm);
     R u[3] = {R(0), R(0), R(0)};
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) u[a] = lm.m1[a] * (R(3) * inv_rho0);
+    for (int a = 0; a < DIM; ++a) u[a] = lm.m1[a] * (K<R>(3) * inv_rho0);
     FDAccum<R> acc;
     acc.clear();
+    if constexpr (std::is_arithmetic<R>::value) {
 #pragma unroll
-    for (int a = 0; a < DIM; ++a)
-        fd_axis_coded<DIM, S, R, FACES>(P, p, c, a, code, T_in, Y_in, u[a], invW0, inv_rho0, &acc.gam[a], acc);
+        for (int a = 0; a < DIM; ++a)
+            fd_axis_coded<DIM, S, R, FACES>(P, p, c, a, code, T_in, Y_in, u[a], invW0, inv_rho0, &acc.gam[a], acc);
+    } else {  // forward mode (2-D): one copy of the FD code
+#pragma unroll 1
+        for (int a = 0; a < DIM; ++a) {
+            R gam;
+            fd_axis_coded<DIM, S, R, FACES>(P, p, c, a, code, T_in, Y_in, a ? u[1] : u[0], invW0, inv_rho0, &gam, acc);
+            if (a) acc.gam[1] = gam;
+            else acc.gam[0] = gam;
+        }
+    }
     // a6-a7
     const R Lam = update_scalars<S, R>(P, c, T0, Y0, inv_T0, W0, acc, T_out, Y_out);
     // a8-a10

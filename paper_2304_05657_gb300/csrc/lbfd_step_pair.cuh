@@ -217,8 +217,8 @@ __global__ void __launch_bounds__(TXP * TY, MINB)
     {
         auto line_x = [&](const float* f, F2* v) { pair_line<true, SX>(f, p0, v); };
         auto line_y = [&](const float* f, F2* v) { pair_line<false, SX>(f, p0, v); };
-        fd_axis_tile<F2>(P, sm, NPT, line_x, 0, u[0], invW0, inv_rho0, acc);
-        fd_axis_tile<F2>(P, sm, NPT, line_y, 1, u[1], invW0, inv_rho0, acc);
+        fd_axis_tile<F2>(P, sm, NPT, line_x, u[0], invW0, inv_rho0, &acc.gam[0], acc);
+        fd_axis_tile<F2>(P, sm, NPT, line_y, u[1], invW0, inv_rho0, &acc.gam[1], acc);
     }
     F2 Y0[NSP];
 #pragma unroll

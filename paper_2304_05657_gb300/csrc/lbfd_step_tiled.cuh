@@ -62,25 +62,25 @@ __device__ __forceinline__ TileSmem<R> tile_smem(unsigned char* raw)
 // cells), PR the parameters' type.
 template <typename R, typename PR, typename SR, typename Line>
 __device__ __forceinline__ void fd_axis_tile(const StepParams<PR>& P, const TileSmem<SR>& sm, int npt, Line line,
-                                             int a, R u_a, R invW0, R inv_rho0, FDAccum<R>& acc)
+                                             R u_a, R invW0, R inv_rho0, R* gam_a, FDAccum<R>& acc)
 {
     fd_axis<false, R>(
         P, u_a, invW0, inv_rho0, false, false, [&](R* v) { line(sm.rho, v); }, [&](R* v) { line(sm.T, v); },
         [&](R* v) { line(sm.invW, v); }, [&](int k, R* v) { line(sm.X + k * npt, v); },
-        [&](int k, R* v) { line(sm.Y + k * npt, v); }, &acc.gam[a], acc);
+        [&](int k, R* v) { line(sm.Y + k * npt, v); }, gam_a, acc);
 }
 
 // the same with the axis' point stride `st` (1 for x, SX for y) and the
 // centre point p0
 template <typename R>
 __device__ __forceinline__ void fd_axis_smem(const StepParams<R>& P, const TileSmem<R>& sm, int npt, int p0, int st,
-                                             int a, R u_a, R invW0, R inv_rho0, FDAccum<R>& acc)
+                                             R u_a, R invW0, R inv_rho0, R* gam_a, FDAccum<R>& acc)
 {
     auto line = [&](const R* f, R* v) {
 #pragma unroll
         for (int j = 0; j < 5; ++j) v[j] = f[p0 + (j - 2) * st];
     };
-    fd_axis_tile<R>(P, sm, npt, line, a, u_a, invW0, inv_rho0, acc);
+    fd_axis_tile<R>(P, sm, npt, line, u_a, invW0, inv_rho0, gam_a, acc);
 }
 
 // FD terms along one axis for a cell next to in-domain solid cells (staircase
@@ -326,10 +326,10 @@ __device__ __forceinline__ void tiled2d_body(const StepParams<R>& P, const S* LB
     }
     // a2
     const R T0 = sm.T[p0], invW0 = sm.invW[p0], rho0 = sm.rho[p0];
-    const R inv_rho0 = T0 * invW0 * P.inv_rho_c;
+    const R inv_rho0 = T0 * invW0 * par<R>(P.inv_rho_c);
     LowMoments<2, R> lm;
     low_moments<2>(g, lm);
-    const R u[3] = {lm.m1[0] * (R(3) * inv_rho0), lm.m1[1] * (R(3) * inv_rho0), R(0)};
+    const R u[3] = {lm.m1[0] * (K<R>(3) * inv_rho0), lm.m1[1] * (K<R>(3) * inv_rho0), R(0)};
     // a3-a5
     FDAccum<R> acc;
     acc.clear();
@@ -340,14 +340,24 @@ __device__ __forceinline__ void tiled2d_body(const StepParams<R>& P, const S* LB
         gh = wall_line(sm.mask, p0, SX, pts);
         fd_axis_smem_walls<R>(P, sm, NPT, pts, gh, 1, u[1], invW0, inv_rho0, acc);
     } else {
-        fd_axis_smem<R>(P, sm, NPT, p0, 1, 0, u[0], invW0, inv_rho0, acc);
-        fd_axis_smem<R>(P, sm, NPT, p0, SX, 1, u[1], invW0, inv_rho0, acc);
+        if constexpr (std::is_arithmetic<R>::value) {
+            fd_axis_smem<R>(P, sm, NPT, p0, 1, u[0], invW0, inv_rho0, &acc.gam[0], acc);
+            fd_axis_smem<R>(P, sm, NPT, p0, SX, u[1], invW0, inv_rho0, &acc.gam[1], acc);
+        } else {  // forward mode: one copy of the FD code (instruction fetch)
+#pragma unroll 1
+            for (int a = 0; a < 2; ++a) {
+                R gam;
+                fd_axis_smem<R>(P, sm, NPT, p0, a ? SX : 1, a ? u[1] : u[0], invW0, inv_rho0, &gam, acc);
+                if (a) acc.gam[1] = gam;
+                else acc.gam[0] = gam;
+            }
+        }
     }
     // a6-a7
     R Y0[NSP];
 #pragma unroll
     for (int k = 0; k < NSP; ++k) Y0[k] = sm.Y[k * NPT + p0];
-    const R rc = rho0 * P.inv_rho_c;
+    const R rc = rho0 * par<R>(P.inv_rho_c);
     const R Lam = update_scalars<S, R>(P, c, T0, Y0, rc * invW0, rc * T0, acc, T_out, Y_out);
     // a8-a10
     if constexpr (HI1) collide_hi1<2, R>(P, lm, rho0, inv_rho0, u, acc.gam, Lam, g);

@@ -148,8 +148,8 @@ __device__ __forceinline__ unsigned face_crossing(const StepParams<R>& P, int x,
 // Inlet and constant-pressure outlet rules (Eq. 31; anti-bounce-back) of a
 // cell at one open face: on entry the crossing populations hold the opposite
 // population of the cell itself, as for bounce-back.  Both rules are
-//   g_i = +-g_ibar + w_i (K + 3 rho (c_i.u)^2),
-// inlet: +, K = 2 rho_in u_in, u = 0; outlet: -, K = -rho u.u, u the cell's
+//   g_i = +-g_ibar + w_i (k0 + 3 rho (c_i.u)^2),
+// inlet: +, k0 = 2 rho_in u_in, u = 0; outlet: -, k0 = -rho u.u, u the cell's
 // velocity before streaming.
 template <typename S, typename R>
 __device__ __forceinline__ void face_rules(const StepParams<R>& P, unsigned cross, const S* LBFD_RESTRICT g_cell,
@@ -161,7 +161,7 @@ __device__ __forceinline__ void face_rules(const StepParams<R>& P, unsigned cros
                   : cross == pop_mask(1, -1) ? 3
                   : cross == pop_mask(2, 1)  ? 4
                                              : 5;
-    R u[3] = {R(0), R(0), R(0)}, K = R(2) * P.rho_in * P.u_in, sign = R(1);
+    R u[3] = {R(0), R(0), R(0)}, k0 = R(2) * P.rho_in * P.u_in, sign = R(1);
     if (face_type(P, f) != BC_INLET) {
         R own[27];
 #pragma unroll
@@ -169,8 +169,8 @@ __device__ __forceinline__ void face_rules(const StepParams<R>& P, unsigned cros
         LowMoments<3, R> m;
         low_moments<3>(own, m);
 #pragma unroll
-        for (int b = 0; b < 3; ++b) u[b] = m.m1[b] * (R(3) * inv_rho0);
-        K = -rho0 * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+        for (int b = 0; b < 3; ++b) u[b] = m.m1[b] * (K<R>(3) * inv_rho0);
+        k0 = -rho0 * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
         sign = R(-1);
     }
     const R r3 = R(3) * rho0;
@@ -178,7 +178,7 @@ __device__ __forceinline__ void face_rules(const StepParams<R>& P, unsigned cros
     for (int i = 0; i < 27; ++i) {
         if (i == 13 || !((cross >> i) & 1u)) continue;
         const R cu = R(cx_of(i)) * u[0] + R(cy_of(i)) * u[1] + R(cz_of(i)) * u[2];
-        g[i] = sign * g[i] + weight<3, R>(i) * (K + r3 * cu * cu);
+        g[i] = sign * g[i] + weight<3, R>(i) * (k0 + r3 * cu * cu);
     }
 }
 
@@ -359,7 +359,7 @@ __device__ __forceinline__ void tiled3d_body(const StepParams<R>& P, int zc, con
         const int p0 = ring[2] + q0;
         if (active) {
             const R T0 = sm.T[p0], invW0 = sm.invW[p0], rho0 = sm.rho[p0];
-            const R inv_rho0 = T0 * invW0 * P.inv_rho_c;
+            const R inv_rho0 = T0 * invW0 * par<R>(P.inv_rho_c);
             if constexpr (CODED) {
                 if (cross) face_rules<S, R>(P, cross, g_in + c, rho0, inv_rho0, g);
             }
@@ -367,7 +367,7 @@ __device__ __forceinline__ void tiled3d_body(const StepParams<R>& P, int zc, con
             low_moments<3>(g, lm);
             R u[3];
 #pragma unroll
-            for (int a = 0; a < 3; ++a) u[a] = lm.m1[a] * (R(3) * inv_rho0);
+            for (int a = 0; a < 3; ++a) u[a] = lm.m1[a] * (K<R>(3) * inv_rho0);
             FDAccum<R> acc;
             acc.clear();
             // the three axes share one copy of the FD code (a rolled loop keeps
@@ -394,7 +394,7 @@ __device__ __forceinline__ void tiled3d_body(const StepParams<R>& P, int zc, con
             R Y0[NSP];
 #pragma unroll
             for (int k = 0; k < NSP; ++k) Y0[k] = sm.Y[k * NPT + p0];
-            const R Lam = update_scalars<S, R>(P, c, T0, Y0, rho0 * invW0 * P.inv_rho_c, sm.X[p0], acc, T_out, Y_out);
+            const R Lam = update_scalars<S, R>(P, c, T0, Y0, rho0 * invW0 * par<R>(P.inv_rho_c), sm.X[p0], acc, T_out, Y_out);
             if constexpr (SPLIT) {
                 aux[c] = Lam;
 #pragma unroll
@@ -478,12 +478,12 @@ __global__ void __launch_bounds__(128)
     const R invW0 = inv_molar_mass(P, Y0);
     R rho0, W0;
     eos_w(P, T0, invW0, rho0, W0);
-    const R inv_rho0 = T0 * invW0 * P.inv_rho_c;
+    const R inv_rho0 = T0 * invW0 * par<R>(P.inv_rho_c);
     LowMoments<3, R> lm;
     low_moments<3>(g, lm);
     R u[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) u[a] = lm.m1[a] * (R(3) * inv_rho0);
+    for (int a = 0; a < 3; ++a) u[a] = lm.m1[a] * (K<R>(3) * inv_rho0);
     const R Lam = aux[c];
     R gam[3];
 #pragma unroll

@@ -1,7 +1,7 @@
 // lbfd_tangent.cu -- the coupled step in tangent-linear (forward-mode)
 // arithmetic, and the reductions of its objectives.
 //
-// The general-form step kernel is instantiated with Dual<double, 4> (or
+// The step's device functions are instantiated with Dual<double, 4> (or
 // Dual<float, 4> for the mixed tangent form): every state value carries its
 // derivative with respect to
 //   theta = (ln A, Ta, T_wall, u_in)
@@ -9,8 +9,10 @@
 // tangent step costs about five plain steps and gives the exact derivative
 // of the discrete scheme; for four parameters and scalar objectives this
 // needs no reverse sweep and no checkpoints.
+#define LBFD_LDG(p) (*(p))  // the state is structs here
 #include "lbfd_internal.h"
 #include "lbfd_step_general.cuh"
+#include "lbfd_step_small.cuh"
 
 namespace lbfd {
 
@@ -32,26 +34,62 @@ __global__ void __launch_bounds__(128) step_kernel_tangent(StepParams<TT> P, con
     cell_step_general<DIM, TT, TT, true, HI1>(P, p, c, g_in, g_out, T_in, T_out, Y_in, Y_out, solid);
 }
 
+// the cells of a list (general form)
+template <int DIM, typename TT>
+__global__ void __launch_bounds__(32) step_kernel_tangent_list(StepParams<TT> P, const TT* __restrict__ g_in,
+                                                               TT* __restrict__ g_out, const TT* __restrict__ T_in,
+                                                               TT* __restrict__ T_out, const TT* __restrict__ Y_in,
+                                                               TT* __restrict__ Y_out,
+                                                               const uint8_t* __restrict__ solid,
+                                                               const long long* __restrict__ cells, long long n)
+{
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n) return;
+    const long long c = cells[t];
+    const int p[3] = {(int)(c % P.nx), (int)(c / P.nx), 0};
+    cell_step_general<DIM, TT, TT, true, true>(P, p, c, g_in, g_out, T_in, T_out, Y_in, Y_out, solid);
+}
+
+// With omega_hi = 1 and staircase walls the tiles and coded cells of the
+// small-grid step in forward-mode arithmetic (two lanes per cell on the
+// smallest grids); else the general form.  The general form evaluates the
+// ten line points of every cell anew, where an 8x4 tile stages three points
+// per cell.  512x64 cells, us per step: FP64 610 -> 321 (the FP64 pipe: 4 140
+// instructions of 64 cycles per warp of 32 cells), mixed 46 -> 23 (the
+// latency of one warp's instructions; its derivatives in packed FP32, 32
+// without).  Two lanes per cell: FP64 64x16 204 -> 143, 256x64 219 -> 240;
+// mixed 64x16 16 -> 11, 512x64 27 -> 25, 512x128 35 -> 39.
 template <typename TT>
 static cudaError_t step_tangent(int dim, const StepParams<TT>& P, StateView in, StateView out, const uint8_t* solid,
-                                cudaStream_t stream)
+                                const BoundaryLists& b, cudaStream_t stream)
 {
     if (dim != 2) return cudaErrorInvalidValue;
+    const TT *g = (const TT*)in.g, *T = (const TT*)in.T, *Y = (const TT*)in.Y;
+    TT *go = (TT*)out.g, *To = (TT*)out.T, *Yo = (TT*)out.Y;
+    if (val(P.omega_hi) == 1.0 && !P.curved && b.interior) {
+        if (b.all2.nrest > 0) {
+            step_kernel_tangent_list<2, TT><<<(unsigned)((b.all2.nrest + 31) / 32), 32, 0, stream>>>(
+                P, g, go, T, To, Y, Yo, solid, b.all2.rest, b.all2.nrest);
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+        }
+        return small_warps(P.nx, P.ny) <= (sizeof(TT) == sizeof(Tan) ? 2 * PARTITIONS / 3 : 2 * PARTITIONS) ? launch_small<TT, TT, true, true>(P, in, out, b, stream)
+                                                             : launch_small<TT, TT, true, false>(P, in, out, b, stream);
+    }
     const unsigned blocks = (unsigned)((P.ncell + 127) / 128);
     auto kern = val(P.omega_hi) == 1.0 ? step_kernel_tangent<2, TT, true> : step_kernel_tangent<2, TT, false>;
-    kern<<<blocks, 128, 0, stream>>>(P, (const TT*)in.g, (TT*)out.g, (const TT*)in.T, (TT*)out.T, (const TT*)in.Y,
-                                     (TT*)out.Y, solid);
+    kern<<<blocks, 128, 0, stream>>>(P, g, go, T, To, Y, Yo, solid);
     return cudaGetLastError();
 }
 cudaError_t launch_step_tangent(int dim, const StepParams<Tan>& P, StateView in, StateView out, const uint8_t* solid,
-                                cudaStream_t stream)
+                                const BoundaryLists& b, cudaStream_t stream)
 {
-    return step_tangent(dim, P, in, out, solid, stream);
+    return step_tangent(dim, P, in, out, solid, b, stream);
 }
 cudaError_t launch_step_tangent(int dim, const StepParams<Tanf>& P, StateView in, StateView out, const uint8_t* solid,
-                                cudaStream_t stream)
+                                const BoundaryLists& b, cudaStream_t stream)
 {
-    return step_tangent(dim, P, in, out, solid, stream);
+    return step_tangent(dim, P, in, out, solid, b, stream);
 }
 
 // derivative k of a raw field (T, Y_k, g_i) into double out[ncell]
