@@ -327,14 +327,16 @@ int lbfd_gradient(lbfd_handle* h, int objective, double* value, double* grad);
  * theta = (ln A, Ta, T_wall, u_in) is the adjoint recursion
  * lambda^n = (dF/dx^n)^T lambda^{n+1} run backwards from
  * lambda^N = dJ/dx^N, plus (dF/dtheta)^T lambda^{n+1} summed over the steps
- * (and J's own dependence on theta).  Each step's adjoint is taken by
- * recording every fluid cell's step on a reverse-mode tape and sweeping it
- * backwards: the exact transpose of the derivative of the discrete step,
- * branches taken on the values.  The forward pass keeps a copy of the state
+ * (and J's own dependence on theta).  Each step's adjoint is the exact
+ * transpose of the derivative of the discrete step, branches taken on the
+ * values: by hand-derived local adjoints of every cell's step when
+ * omega_hi = 1 and there is neither a convective outlet nor a cell with a
+ * link through two open faces, else by recording every fluid cell's step on
+ * a reverse-mode tape and sweeping it backwards.  The forward pass keeps a copy of the state
  * every `checkpoint_every` steps; the backward pass recomputes each segment
  * from its copy with the forward kernels (FP32 ones for LBFD_MIXED) and
- * evaluates every step's adjoint at that trajectory, the step recorded in
- * FP64 (in FP32 for LBFD_MIXED: FP32 values and partials), accumulating
+ * evaluates every step's adjoint at that trajectory, the step differentiated
+ * in FP64 (by a tape for LBFD_MIXED: FP32 values and partials), accumulating
  * lambda and the gradient in FP64.
  *
  * lbfd_adjoint_setup: the checkpoint interval of later calls (default 200).

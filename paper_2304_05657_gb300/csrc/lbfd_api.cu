@@ -1195,6 +1195,92 @@ int lbfd_adjoint_record(lbfd_handle* h, int steps, int objective, double* value)
     return LBFD_OK;
 }
 
+// lambda^N = seed * dJ/dx^N of the recorded run in lam (FP64) and J's own
+// dependence on theta in dth, ordered on the handle's stream
+static int adjoint_seed(lbfd_handle* h, double seed, double* lam, double* dth)
+{
+    cudaStream_t s = h->stream;
+    const bool fp32 = h->precision == LBFD_MIXED;
+    CK(cudaMemsetAsync(dth, 0, lbfd::NTAN * sizeof(double), s));
+    CK(cudaMemsetAsync(lam, 0, h->planes * (size_t)h->stride * sizeof(double), s));
+    if (h->adj_obj == LBFD_OBJ_FLAME_POSITION) {
+        // x_f = dx sum_fluid Y_F / (Y_F,in * section)
+        const double scale = h->section > 0.0 ? seed * h->prm.dx / (h->prm.Y_in[h->mech.fuel] * h->section) : 0.0;
+        std::vector<double> v((size_t)h->stride, 0.0);
+        for (long long c = 0; c < h->ncell; ++c)
+            if (!h->mask_host[c]) v[c] = scale;
+        CK(cudaMemcpyAsync(lam + (size_t)(h->Q + 1 + h->mech.fuel) * h->stride, v.data(),
+                           (size_t)h->stride * sizeof(double), cudaMemcpyHostToDevice, s));
+        CK(cudaStreamSynchronize(s));
+    } else {
+        double r[2];
+        CK(lbfd::launch_quench_sums(h->Pd, view(h, h->cur), fp32, h->solid, h->qwgt, h->red, s));
+        CK(cudaMemcpyAsync(r, h->red, sizeof r, cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        if (r[0] > 0.0 && r[1] > 0.0)
+            CK(lbfd::launch_quench_seed(h->Pd, view(h, h->cur), fp32, h->solid, h->qwgt, r[0], r[1], h->adj_J, seed,
+                                        lam, dth, h->Q, s));
+    }
+    return LBFD_OK;
+}
+
+// The states of segment g of the recorded run, recomputed from its checkpoint
+// with the forward kernels into seg (slot j: the state before step j of the
+// segment; every slot starts as the checkpoint, solid cells never change)
+static int adjoint_segment(lbfd_handle* h, int g, int len, char* seg)
+{
+    cudaStream_t s = h->stream;
+    const size_t sbytes = h->planes * (size_t)h->stride * h->esz;
+    for (int j = 0; j < len; ++j)
+        CK(cudaMemcpyAsync(seg + (size_t)j * sbytes, h->adj_ck + (size_t)g * sbytes, sbytes, cudaMemcpyDeviceToDevice,
+                           s));
+    for (int j = 1; j < len; ++j)
+        CK(launch_variant(h, h->variant, view_of(h, seg + (size_t)(j - 1) * sbytes),
+                          view_of(h, seg + (size_t)j * sbytes), s));
+    return LBFD_OK;
+}
+
+// The backward pass by hand-derived adjoints: one launch per step
+// (lbfd_adjoint_direct.cu), no tape.
+static int adjoint_backward_direct(lbfd_handle* h, double seed, double* grad)
+{
+    const int steps = h->adj_steps, nseg = h->adj_nseg;
+    const int K = h->adj_K < steps ? h->adj_K : steps;
+    const bool fp32 = h->precision == LBFD_MIXED;
+    const size_t sbytes = h->planes * (size_t)h->stride * h->esz;
+    const size_t lbytes = h->planes * (size_t)h->stride * sizeof(double);
+    cudaStream_t s = h->stream;
+    char* mem = nullptr;  // the segment's states, two adjoint states, dJ/dtheta
+    if (cudaMalloc((void**)&mem, sbytes * K + 2 * lbytes + lbfd::NTAN * sizeof(double)) != cudaSuccess) {
+        snprintf(g_last_error, sizeof g_last_error, "cudaMalloc(adjoint states)");
+        return LBFD_ENOMEM;
+    }
+    double* lam1 = (double*)(mem + sbytes * K);
+    double* lam0 = lam1 + h->planes * (size_t)h->stride;
+    double* dth = lam0 + h->planes * (size_t)h->stride;
+    const lbfd::BoundaryLists b = lists(h);
+    auto run = [&]() -> int {
+        int st = adjoint_seed(h, seed, lam1, dth);
+        for (int g = nseg - 1; g >= 0 && st == LBFD_OK; --g) {
+            const int len = steps - g * K < K ? steps - g * K : K;
+            st = adjoint_segment(h, g, len, mem);
+            for (int j = len - 1; j >= 0 && st == LBFD_OK; --j) {
+                CK(cudaMemsetAsync(lam0, 0, lbytes, s));
+                CK(lbfd::launch_adjoint_step(h->Pd, view_of(h, mem + (size_t)j * sbytes), fp32, b, lam1, lam0, dth, s));
+                std::swap(lam0, lam1);
+            }
+        }
+        if (st != LBFD_OK) return st;
+        CK(cudaMemcpyAsync(grad, dth, lbfd::NTAN * sizeof(double), cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        return LBFD_OK;
+    };
+    const int st = run();
+    cudaStreamSynchronize(s);
+    cudaFree(mem);
+    return st;
+}
+
 // One backward sweep with tapes of maxn nodes per thread; *overflow is set
 // when a cell's step needed more.  The tapes of groups of steps are recorded
 // on a second stream into two alternating buffers while the steps of the
@@ -1294,38 +1380,25 @@ static int adjoint_backward_pass(lbfd_handle* h, double seed, int maxn, double* 
     }
     cudaStream_t rs = nbuf == 2 ? s2 : s;  // the stream of the records
     AK(cudaMemsetAsync(w[0].flags, 0, 2 * sizeof(int), s));
-    AK(cudaMemsetAsync(dth, 0, lbfd::NTAN * sizeof(double), s));
-    // the adjoint of J with respect to the final state (FP64), times seed
-    AK(cudaMemsetAsync(lam1, 0, lbytes, s));
-    if (h->adj_obj == LBFD_OBJ_FLAME_POSITION) {
-        // x_f = dx sum_fluid Y_F / (Y_F,in * section)
-        const double scale = h->section > 0.0 ? seed * h->prm.dx / (h->prm.Y_in[h->mech.fuel] * h->section) : 0.0;
-        std::vector<double> lam((size_t)h->stride, 0.0);
-        for (long long c = 0; c < h->ncell; ++c)
-            if (!h->mask_host[c]) lam[c] = scale;
-        AK(cudaMemcpyAsync(lam1 + (size_t)(h->Q + 1 + h->mech.fuel) * h->stride, lam.data(),
-                           (size_t)h->stride * sizeof(double), cudaMemcpyHostToDevice, s));
-        AK(cudaStreamSynchronize(s));
-    } else {
-        double r[2];
-        AK(lbfd::launch_quench_sums(h->Pd, view(h, h->cur), fp32, h->solid, h->qwgt, h->red, s));
-        AK(cudaMemcpyAsync(r, h->red, sizeof r, cudaMemcpyDeviceToHost, s));
-        AK(cudaStreamSynchronize(s));
-        if (r[0] > 0.0 && r[1] > 0.0)
-            AK(lbfd::launch_quench_seed(h->Pd, view(h, h->cur), fp32, h->solid, h->qwgt, r[0], r[1], h->adj_J, seed,
-                                        lam1, dth, h->Q, s));
+    {
+        const int st = adjoint_seed(h, seed, lam1, dth);
+        if (st != LBFD_OK) {
+            release();
+            return st;
+        }
     }
     // backward pass: each segment recomputed from its checkpoint with the
     // forward kernels (FP32 in the mixed form), every step's adjoint in FP64
     const int G = w[0].slots;
     for (int g = nseg - 1; g >= 0; --g) {
         const int len = steps - g * K < K ? steps - g * K : K;
-        for (int j = 0; j < len; ++j)  // every slot starts as the checkpoint (solid cells never change)
-            AK(cudaMemcpyAsync(seg + (size_t)j * sbytes, h->adj_ck + (size_t)g * sbytes, sbytes,
-                               cudaMemcpyDeviceToDevice, s));
-        for (int j = 1; j < len; ++j)
-            AK(launch_variant(h, h->variant, view_of(h, seg + (size_t)(j - 1) * sbytes),
-                              view_of(h, seg + (size_t)j * sbytes), s));
+        {
+            const int st = adjoint_segment(h, g, len, seg);
+            if (st != LBFD_OK) {
+                release();
+                return st;
+            }
+        }
         if (!pipelined) {  // one step at a time (j0 == j1), recorded and swept in chunks of cells
             for (int j = len - 1; j >= 0; --j) {
                 AK(cudaMemsetAsync(lam0, 0, lbytes, s));
@@ -1394,10 +1467,17 @@ int lbfd_adjoint_backward(lbfd_handle* h, double seed, double* grad)
     NvtxRange nvtx_("lbfd_adjoint_backward");
     if (!h || !grad) return LBFD_EINVAL;
     if (!h->adj_ck || h->adj_steps < 1) return LBFD_EINVAL;  // nothing recorded
+    double g[lbfd::NTAN];
+    if (lbfd::adjoint_direct_applies(h->Pd, lists(h))) {
+        const int st = adjoint_backward_direct(h, seed, g);
+        adjoint_release(h);
+        if (st != LBFD_OK) return st;
+        for (int k = 0; k < lbfd::NTAN; ++k) grad[k] = g[k];
+        return LBFD_OK;
+    }
     // tapes of 2048 nodes per cell and step hold every step of the 2-D
     // general form with room to spare; a step that needs more is taken again
     // with the 16-bit node limit's share of 4096
-    double g[lbfd::NTAN];
     bool overflow = false;
     for (int maxn : {2048, 4096}) {
         const int st = adjoint_backward_pass(h, seed, maxn, g, &overflow);

@@ -201,6 +201,13 @@ cudaError_t launch_adjoint_record(int dim, const StepParams<double>& Pd, int pla
 cudaError_t launch_adjoint_sweep(const StepParams<double>& Pd, int planes, int slot, bool fp32, const uint8_t* solid,
                                  long long c0, long long n, const double* lam_next, double* lam, double* dtheta,
                                  const AdjointWork& w, cudaStream_t stream);
+// The same transpose of one step from the state st by hand-derived local
+// adjoints, without a tape (lbfd_adjoint_direct.cu): omega_hi = 1, staircase
+// walls, no convective outlet and no cell outside the coded form.  lam zeroed
+// by the caller.
+bool adjoint_direct_applies(const StepParams<double>& P, const BoundaryLists& b);
+cudaError_t launch_adjoint_step(const StepParams<double>& P, StateView st, bool fp32, const BoundaryLists& b,
+                                const double* lam_next, double* lam, double* dtheta, cudaStream_t stream);
 // quenching-distance objective J = (S1/S0)^(-1/4), S0 = sum_fluid h,
 // S1 = sum_fluid h w (h the heat release of a cell, w = d^-4 its wall
 // weight): red[0..1] = S0, S1 of state st; and the adjoint seed

@@ -55,10 +55,10 @@ __global__ void __launch_bounds__(32) step_kernel_tangent_list(StepParams<TT> P,
 // smallest grids); else the general form.  The general form evaluates the
 // ten line points of every cell anew, where an 8x4 tile stages three points
 // per cell.  512x64 cells, us per step: FP64 610 -> 321 (the FP64 pipe: 4 140
-// instructions of 64 cycles per warp of 32 cells), mixed 46 -> 23 (the
-// latency of one warp's instructions; its derivatives in packed FP32, 32
-// without).  Two lanes per cell: FP64 64x16 204 -> 143, 256x64 219 -> 240;
-// mixed 64x16 16 -> 11, 512x64 27 -> 25, 512x128 35 -> 39.
+// instructions of 64 cycles per warp of 32 cells), mixed 46 -> 25 (the
+// latency of one warp's instructions; the packed FP32 derivatives took it
+// from 32).  One and two lanes per cell: FP64 64x16 204, 143 us, 256x64 219,
+// 240; mixed (before the packing) 64x16 22, 17, 512x64 34, 32, 512x128 43, 48.
 template <typename TT>
 static cudaError_t step_tangent(int dim, const StepParams<TT>& P, StateView in, StateView out, const uint8_t* solid,
                                 const BoundaryLists& b, cudaStream_t stream)
