@@ -218,41 +218,40 @@ int lbfd_set_wait_limit(lbfd_handle* h, long long ns);
 
 /* Kernel variants of the step: 0 is the general form (any cell, D2Q9 and
  * D3Q27).  In 2-D (13 variants), 1..4 are shared-memory tiles of 32x8,
- * 32x4, 64x4 and 32x16 interior cells; 5..8 the same tiles plus a second
- * tile kernel (over the 64x2 tiles that need it) for the cells next to
- * in-domain solid cells (staircase walls, from shared memory); 9..12 as 5..8
- * with two interior cells per thread in packed FP32 arithmetic (tiles of
- * 32x8, 64x8, 32x8, 64x4 at 4, 2, 5 and 5 blocks per SM; the FP64 form runs
- * them one cell per thread).
- * In 3-D (8 variants), 1..2 are 32x4 columns marching through 16 or 32
- * z-planes with a five-plane shared-memory ring, 3 is 1 with the registers
- * capped for four blocks per SM, 4..5 are 1..2 split into an FD tile
- * kernel (a1-a7, writing Lambda and grad rho to a scratch buffer of four
- * planes) and a per-cell collision kernel (a8-a10), and 6..7 are 1..2 with
- * the cells next to in-domain solids updated in the tile kernel too (ghost
- * points by the mirror rule from the staged mask, bounce-back pulls).  The
- * cells the tiles leave out are listed at create.  With staircase walls, a
- * 64-bit neighbourhood code per listed cell drives a compact form of the
- * step: in 2-D for every listed cell but those with a link through two open
- * faces or a convective outlet without a fluid inner cell; in 3-D one list
- * for the cells next to in-domain solids (variants 1..5) and one for the
- * cells near inlet and outlet faces of one axis.  The general form takes the
+ * 32x4, 64x4 and 32x16 cells; 5..8 the same tiles of interior cells alone,
+ * with the cells next to walls and faces (staircase walls) through a list;
+ * 9..12 as 5..8 with two interior cells per thread in packed FP32 arithmetic
+ * (tiles of 32x8, 64x8, 32x8, 64x4 at 4, 2, 5 and 5 blocks per SM; the FP64
+ * form runs them one cell per thread).
+ * In 3-D (8 variants), 1..3 are columns of 32x4 or 16x8 cells marching
+ * through the z-planes of a piece with a shared-memory ring, the pieces'
+ * planes chosen from the grid, 4..5 the same split into an FD tile kernel
+ * (a1-a7, writing Lambda and grad rho to a scratch buffer of four planes)
+ * and a per-cell collision kernel (a8-a10), and 6..7 with the cells next to
+ * in-domain solids in the tile kernel and those near faces through a list.
+ * With staircase walls, a 64-bit neighbourhood code per cell next to walls
+ * or faces drives a compact form of the step, in the tiles (2-D 1..4, 3-D
+ * 1..3, 6, 7) or over a list of the cells that the tiles leave out: in 2-D
+ * for every such cell but those with a link through two open faces or a
+ * convective outlet without a fluid inner cell; in 3-D for the cells next to
+ * in-domain solids and for those near inlet and outlet faces of one axis.
+ * The lists are made at create.  The general form takes the
  * others, and every listed cell when the walls are curved.  2-D grids too
- * small to fill the GPU with a variant's tiles (up to 311 296 cells in FP32,
+ * small to fill the GPU with a variant's tiles (up to 155 648 cells in FP32,
  * 622 592 in FP64, staircase walls) run as one launch of small tiles and the
- * listed cells, whatever the variant (except 0).  With omega_hi = 1 the
+ * cells they leave out, whatever the variant (except 0).  With omega_hi = 1 the
  * collision uses the moments of orders 0-2 of the populations alone (the
  * relaxation sets the higher cumulants to equilibrium).  All variants
  * compute the same step up to rounding order.  Default: 1 (0 for
- * LBFD_TANGENT, which has the general form only). */
+ * LBFD_TANGENT and LBFD_TANGENT_MIXED, which have one form). */
 int lbfd_num_variants(const lbfd_handle* h);
 int lbfd_get_variant(const lbfd_handle* h);
 int lbfd_set_variant(lbfd_handle* h, int variant);
 /* Kernel launches one step makes with the current variant: one on small 2-D
  * grids (above); else the tile variants launch the tile kernel plus one
- * kernel per non-empty list of boundary cells (and the wall-tile kernel in
- * 2-D variants 5..12, the collision kernel in 3-D variants 4..5); curved
- * walls add the ghost-fill kernel. */
+ * kernel per non-empty list of the boundary cells that their tiles leave out
+ * (and the collision kernel in 3-D variants 4..5); curved walls add the
+ * ghost-fill kernel. */
 int lbfd_launches_per_step(const lbfd_handle* h);
 
 /* Autotuner: time every variant over `reps` launches on the current state

@@ -203,7 +203,6 @@ static StepParams<RevT<V>> rev_params(const StepParams<double>& D)
     for (int f = 0; f < 6; ++f) {
         P.bc[f] = D.bc[f];
         P.T_wall[f] = D.bc[f] == BC_WALL_ISOTHERMAL ? Rv(D.T_wall[f], 2) : Rv(D.T_wall[f]);
-        P.face_solid[f] = D.face_solid[f];
     }
     for (int k = 0; k < NSP; ++k) {
         P.inv_Wk[k] = Rv(D.inv_Wk[k]);

@@ -331,12 +331,12 @@ __device__ __forceinline__ void reverse_tile(const StepParams<double>& P, const 
     const int x0 = bx * SM_TX, y0 = by * SM_TY, x = x0 + tx, y = y0 + ty;
     const bool inside = x < P.nx && y < P.ny;
     const long long c = inside ? (long long)x + (long long)P.nx * y : 0;
-    const bool on = inside && interior[c] != 0;
+    const bool on = inside && interior[c] == 1;
     double g[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) g[i] = 0.0;
     if (on) pull_interior<S, double>(P, g_in, c, x, y, g);
-    stage_tile2d<S, double, SM_TX, SM_TY, false, 32>(P, sm, x0, y0, lane, T_in, Y_in, nullptr);
+    stage_tile2d<S, double, SM_TX, SM_TY, false, 32>(P, sm, x0, y0, lane, T_in, Y_in);
     for (int j = lane; j < NPT * (3 + 2 * NSP); j += 32) bs.T[j] = 0.0;
     __syncwarp();
     if (!__any_sync(0xffffffffu, on)) return;

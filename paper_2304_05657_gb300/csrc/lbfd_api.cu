@@ -41,30 +41,29 @@ struct lbfd_handle {
     uint8_t* solid;       // device mask
     long long* bnd;       // device list of the cells the tile kernels skip
     long long nbnd;
-    long long* bndf;      // the subset near domain faces (wall-aware 2-D tiles)
+    long long* bndf;      // 3-D: the subset near domain faces
     long long nbndf;
     long long* bndw;      // 3-D: the others (next to in-domain solids only)
     long long nbndw;
     unsigned long long* bndw_code;  // 3-D: their neighbourhood codes
-    // 2-D: bnd and bndf split into the cells that take the coded form, with
-    // their codes, and the rest (device lists)
+    // 2-D: bnd split into the cells that take the coded form, with their
+    // codes, and the rest (device lists)
     struct Coded2 {
         long long* cells;
         unsigned long long* codes;
-        long long n;
+        long long n, nout;  // (the first nout of them are not for the coded tiles)
         long long* rest;
         long long nrest;
-    } bnd2, bndf2;
+    } bnd2;
     long long* bndfc;     // 3-D: the cells near faces that take the coded form (staircase walls)
     long long nbndfc, nbndfx;  // (the first nbndfx of them are not for the tile kernel)
     unsigned long long* bndfc_code;
     long long* bndfg;     // 3-D: the other cells near faces (general form)
     long long nbndfg;
-    uint8_t* interior;    // 2-D, per cell: 1 = updated by the interior tile kernels
+    uint8_t* interior;    // 2-D, per cell: 1 interior, 2 coded and in reach of the coded tiles, 0 others
+    unsigned long long* cell_codes;  // 2-D: the codes of the cells of class 2, per cell
     unsigned long long* words;  // 3-D, per cell: interior, coded (with its code) or other
     void* aux;            // 3-D: Lambda and grad rho planes of the split variants
-    int* wtiles;          // tiles holding the other boundary cells (2-D)
-    long long nwtiles;
     double* red;          // device reduction scratch
     double* tmp;          // device read-out buffer (ncell doubles)
     cudaStream_t stream;
@@ -191,14 +190,9 @@ void fill_params(const lbfd_handle* h, StepParams<R>& P)
     P.inv_rho_c = (R)(1.0 / (p.T_in * invW_in));
     P.rho_in = (R)1.0;  // EOS reference state (T_in, Y_in)
     P.T_solid = (R)p.T_solid;
-    P.rho_solid = (R)(p.T_in * invW_in / p.T_solid);  // (FP64 and mixed 3-D tiles)
+    P.rho_solid = (R)(p.T_in * invW_in / p.T_solid);  // (FP64 and mixed tiles)
     P.solid_isothermal = p.solid_isothermal;
     P.poiseuille = p.poiseuille_inlet;
-    for (int f = 0; f < 6; ++f) {
-        const int b = P.bc[f];
-        P.face_solid[f] = (b == LBFD_BC_WALL_ISOTHERMAL && p.solid_isothermal && G.T_wall[f] == p.T_solid) ||
-                          (b == LBFD_BC_WALL_ADIABATIC && !p.solid_isothermal);
-    }
     // the WENO3 weights hold eps^2 (FP32) and eps^4 (FP64): kept in range (the
     // limits lie far below the squared resolution of any field)
     const double eps_lo = sizeof(R) % 8 ? 1e-18 : 1e-75;
@@ -277,18 +271,16 @@ void free_handle(lbfd_handle* h)
     if (h->bndf) cudaFree(h->bndf);
     if (h->bndw) cudaFree(h->bndw);
     if (h->bndw_code) cudaFree(h->bndw_code);
-    for (lbfd_handle::Coded2* l : {&h->bnd2, &h->bndf2}) {
-        if (l->cells) cudaFree(l->cells);
-        if (l->codes) cudaFree(l->codes);
-        if (l->rest) cudaFree(l->rest);
-    }
+    if (h->bnd2.cells) cudaFree(h->bnd2.cells);
+    if (h->bnd2.codes) cudaFree(h->bnd2.codes);
+    if (h->bnd2.rest) cudaFree(h->bnd2.rest);
     if (h->bndfc) cudaFree(h->bndfc);
     if (h->bndfc_code) cudaFree(h->bndfc_code);
     if (h->bndfg) cudaFree(h->bndfg);
     if (h->interior) cudaFree(h->interior);
+    if (h->cell_codes) cudaFree(h->cell_codes);
     if (h->words) cudaFree(h->words);
     if (h->aux) cudaFree(h->aux);
-    if (h->wtiles) cudaFree(h->wtiles);
     if (h->pwait) cudaFree(h->pwait);
     if (h->qwgt) cudaFree(h->qwgt);
     if (h->adj_ck) cudaFree(h->adj_ck);
@@ -338,10 +330,8 @@ lbfd::BoundaryLists lists(const lbfd_handle* h)
     b.all = h->bnd;
     b.nall = h->nbnd;
     const bool curved = h->nghost > 0 || h->Pd.curved;
-    b.face = curved ? h->bnd : h->bndf;
-    b.nface = curved ? h->nbnd : h->nbndf;
-    b.wall_tiles = h->wtiles;
-    b.nwall_tiles = curved ? 0 : h->nwtiles;
+    b.face = nullptr;
+    b.nface = 0;
     b.wall = nullptr;
     b.nwall = 0;
     b.wall_code = nullptr;
@@ -363,10 +353,9 @@ lbfd::BoundaryLists lists(const lbfd_handle* h)
             b.face_code = h->bndfc_code;
         }
     }
-    auto coded = [](const lbfd_handle::Coded2& l) { return lbfd::CodedList{l.cells, l.codes, l.n, l.rest, l.nrest}; };
-    b.all2 = coded(h->bnd2);
-    b.face2 = coded(h->bndf2);
+    b.all2 = lbfd::CodedList{h->bnd2.cells, h->bnd2.codes, h->bnd2.n, h->bnd2.nout, h->bnd2.rest, h->bnd2.nrest};
     b.interior = h->interior;
+    b.cell_codes = h->cell_codes;
     b.words = h->words;
     b.aux = h->aux;
     return b;
@@ -494,7 +483,7 @@ int lbfd_create(const lbfd_grid* grid, const uint8_t* solid_mask, const lbfd_mec
         return cuda_fail(e, "cudaMemcpy(mask)");
     }
     if (!is_tangent(h->precision) &&
-        ((e = cudaDeviceGetStreamPriorityRange(&h->side.low, &h->side.priority)) != cudaSuccess ||
+        ((e = cudaDeviceGetStreamPriorityRange(nullptr, &h->side.priority)) != cudaSuccess ||
          (e = cudaStreamCreateWithPriority(&h->side.stream, cudaStreamNonBlocking, h->side.priority)) !=
              cudaSuccess ||
          (e = cudaEventCreateWithFlags(&h->side.fork, cudaEventDisableTiming)) != cudaSuccess ||
@@ -507,10 +496,9 @@ int lbfd_create(const lbfd_grid* grid, const uint8_t* solid_mask, const lbfd_mec
     for (long long c = 0; c < h->ncell; c += h->grid.nx)
         if (!m[c]) h->section += 1.0;
     std::vector<long long> lists_host[2];
-    for (int faces_only = 0; faces_only <= 1; ++faces_only) {
+    for (int faces_only = 0; faces_only <= (h->dim == 3 ? 1 : 0); ++faces_only) {
         std::vector<long long>& list = lists_host[faces_only];
-        lbfd::boundary_cells(h->dim, h->grid.nx, h->grid.ny, h->grid.nz, h->Pd.bc, m.data(), list, faces_only != 0,
-                             h->Pd.face_solid);
+        lbfd::boundary_cells(h->dim, h->grid.nx, h->grid.ny, h->grid.nz, h->Pd.bc, m.data(), list, faces_only != 0);
         long long** dst = faces_only ? &h->bndf : &h->bnd;
         (faces_only ? h->nbndf : h->nbnd) = (long long)list.size();
         if (list.empty()) continue;
@@ -523,18 +511,6 @@ int lbfd_create(const lbfd_grid* grid, const uint8_t* solid_mask, const lbfd_mec
             cudaSuccess) {
             free_handle(h);
             return cuda_fail(e, "cudaMemcpy(boundary list)");
-        }
-    }
-    if (h->dim == 2) {
-        // per-cell flag of the cells the tile kernels update (fluid cells
-        // outside the boundary list)
-        std::vector<uint8_t> inter((size_t)h->ncell, 0);
-        for (long long c = 0; c < h->ncell; ++c) inter[c] = m[c] ? 0 : 1;
-        for (long long c : lists_host[0]) inter[c] = 0;
-        if ((e = cudaMalloc(&h->interior, (size_t)h->ncell)) != cudaSuccess ||
-            (e = cudaMemcpy(h->interior, inter.data(), (size_t)h->ncell, cudaMemcpyHostToDevice)) != cudaSuccess) {
-            free_handle(h);
-            return cuda_fail(e, "interior flags");
         }
     }
     if (h->dim == 3) {  // all \ face (both sorted)
@@ -620,38 +596,50 @@ int lbfd_create(const lbfd_grid* grid, const uint8_t* solid_mask, const lbfd_mec
         }
     }
     if (h->dim == 2) {
-        lbfd_handle::Coded2* dst[2] = {&h->bnd2, &h->bndf2};
-        for (int j = 0; j < 2; ++j) {
-            std::vector<long long> cells, rest;
-            std::vector<unsigned long long> codes;
-            lbfd::list_codes2d(h->grid.nx, h->grid.ny, h->Pd.bc, m.data(), lists_host[j], cells, codes, rest);
-            dst[j]->n = (long long)cells.size();
-            dst[j]->nrest = (long long)rest.size();
-            auto put = [&](void** to, const void* from, size_t bytes) {
-                if (bytes == 0) return cudaSuccess;
-                const cudaError_t pe = cudaMalloc(to, bytes);
-                return pe != cudaSuccess ? pe : cudaMemcpy(*to, from, bytes, cudaMemcpyHostToDevice);
-            };
-            if ((e = put((void**)&dst[j]->cells, cells.data(), cells.size() * sizeof(long long))) != cudaSuccess ||
-                (e = put((void**)&dst[j]->codes, codes.data(), codes.size() * sizeof(unsigned long long))) !=
-                    cudaSuccess ||
-                (e = put((void**)&dst[j]->rest, rest.data(), rest.size() * sizeof(long long))) != cudaSuccess) {
-                free_handle(h);
-                return cuda_fail(e, "2-D boundary lists");
+        // what each cell is to the tile kernels: interior (fluid cells
+        // outside the boundary list), coded or another kernel's
+        std::vector<uint8_t> cls((size_t)h->ncell, 0);
+        std::vector<unsigned long long> cell_codes((size_t)h->ncell, 0);
+        for (long long c = 0; c < h->ncell; ++c) cls[c] = m[c] ? 0 : 1;
+        for (long long c : lists_host[0]) cls[c] = 0;
+        std::vector<long long> listed, cells, rest;
+        std::vector<unsigned long long> listed_codes, codes;
+        lbfd::list_codes2d(h->grid.nx, h->grid.ny, h->Pd.bc, m.data(), lists_host[0], listed, listed_codes, rest);
+        // first the cells that the coded tiles leave to the list: next to a
+        // face, with a convective outlet there or no fluid cell on the other
+        // side (their ghosts are not the staged ones)
+        for (int in_tile = 0; in_tile <= 1; ++in_tile) {
+            for (size_t t = 0; t < listed.size(); ++t) {
+                const unsigned long long code = listed_codes[t];
+                bool tile = true;
+                for (int f = 0; f < 4; ++f) {
+                    if (!((code >> (50 + f)) & 1u)) continue;
+                    const unsigned w = (unsigned)(code >> (32 + 3 * f)) & 7u;
+                    tile = tile && w != 5u && !(w == 1u && h->Pd.bc[f] == LBFD_BC_OUTLET);
+                }
+                if (tile != (in_tile != 0)) continue;
+                cells.push_back(listed[t]);
+                codes.push_back(code);
+                if (tile) {
+                    cls[listed[t]] = 2;
+                    cell_codes[listed[t]] = code;
+                }
             }
+            if (!in_tile) h->bnd2.nout = (long long)cells.size();
         }
-    }
-    if (h->dim == 2) {
-        std::vector<int> tiles;
-        lbfd::wall_tiles(h->grid.nx, h->grid.ny, lists_host[0], lists_host[1], tiles);
-        h->nwtiles = (long long)tiles.size();
-        if (!tiles.empty()) {
-            if ((e = cudaMalloc(&h->wtiles, tiles.size() * sizeof(int))) != cudaSuccess ||
-                (e = cudaMemcpy(h->wtiles, tiles.data(), tiles.size() * sizeof(int), cudaMemcpyHostToDevice)) !=
-                    cudaSuccess) {
-                free_handle(h);
-                return cuda_fail(e, "wall tiles");
-            }
+        h->bnd2.n = (long long)cells.size();
+        h->bnd2.nrest = (long long)rest.size();
+        auto put = [&](auto** to, const auto& from) {
+            const size_t bytes = from.size() * sizeof(from[0]);
+            if (bytes == 0) return cudaSuccess;
+            const cudaError_t pe = cudaMalloc(to, bytes);
+            return pe != cudaSuccess ? pe : cudaMemcpy(*to, from.data(), bytes, cudaMemcpyHostToDevice);
+        };
+        if ((e = put(&h->bnd2.cells, cells)) != cudaSuccess || (e = put(&h->bnd2.codes, codes)) != cudaSuccess ||
+            (e = put(&h->bnd2.rest, rest)) != cudaSuccess || (e = put(&h->interior, cls)) != cudaSuccess ||
+            (e = put(&h->cell_codes, cell_codes)) != cudaSuccess) {
+            free_handle(h);
+            return cuda_fail(e, "2-D cell classes");
         }
     }
     // initial state: T_in, Y_in, g = 0
@@ -824,10 +812,9 @@ int lbfd_launches_per_step(const lbfd_handle* h)
             n += (b.nface > 0 ? 1 : 0) + (face_list ? 1 : 0) + (b.nwall > 0 && (split || h->Pd.curved) ? 1 : 0) +
                  (split ? 1 : 0);
         } else {
-            const bool wv = h->variant >= 5 && b.nwall_tiles > 0;
-            const lbfd::CodedList& cl = wv ? b.face2 : b.all2;
+            const long long nc = h->variant >= 5 ? b.all2.n : b.all2.nout;
             if (h->Pd.curved) n += b.nall > 0 ? 1 : 0;
-            else if (!runs_small(h, h->variant, b)) n += (cl.n > 0 ? 1 : 0) + (cl.nrest > 0 ? 1 : 0) + (wv ? 1 : 0);
+            else if (!runs_small(h, h->variant, b)) n += (nc > 0 ? 1 : 0) + (b.all2.nrest > 0 ? 1 : 0);
         }
     }
     return n + (h->nghost > 0 ? 1 : 0);

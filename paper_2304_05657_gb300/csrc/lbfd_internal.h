@@ -29,7 +29,6 @@ struct SideStream {
     cudaStream_t stream;
     cudaEvent_t fork, join;
     int priority;  // the device's greatest stream priority
-    int low;       // and its least
 };
 
 // Launch on the side stream at its priority, so that the block scheduler
@@ -53,14 +52,14 @@ cudaError_t launch_prio(void (*kern)(Exp...), dim3 grid, dim3 block, size_t smem
     return cudaLaunchKernelEx(&cfg, kern, std::forward<Act>(args)...);
 }
 
-// Cells the tile kernels leave to the boundary kernel (see boundary_cells):
-// `all` every non-interior fluid cell; `face` only those whose stencil
-// reaches a domain face (for the 2-D variants that handle in-domain solid
-// neighbours themselves).  Unused by the general variant.
+// Fluid cells that are not interior (see boundary_cells): `all` every one,
+// `face` (3-D) those whose stencil reaches a domain face.  Unused by the
+// general variant.
 struct CodedList {
     const long long* cells;
     const unsigned long long* codes;
     long long n;
+    long long nout;  // the first of them, which the coded tiles leave to the list
     const long long* rest;
     long long nrest;
 };
@@ -69,8 +68,6 @@ struct BoundaryLists {
     long long nall;
     const long long* face;
     long long nface;
-    const int* wall_tiles;  // 2-D tiles of WALL_TX x WALL_TY cells holding cells of all \ face
-    long long nwall_tiles;
     const long long* wall;  // 3-D: all \ face, cells whose stencils reach no non-periodic face
     long long nwall;
     const unsigned long long* wall_code;  // 3-D: their neighbourhood codes (cell_step_coded)
@@ -78,21 +75,16 @@ struct BoundaryLists {
     long long nface_coded;        // (then `face` holds the other cells near faces)
     long long nface_tile;         // the first of them, which the tile kernel leaves to the list
     const unsigned long long* face_code;
-    // 2-D, staircase walls: `all` and `face` split into the cells that
-    // cell_step_coded takes (list_codes2d) and the rest (general form)
-    CodedList all2, face2;
-    const uint8_t* interior;  // 2-D, per cell: 1 for the cells the interior tile kernels update
+    // 2-D, staircase walls: `all` split into the cells that cell_step_coded
+    // takes (list_codes2d) and the rest (general form)
+    CodedList all2;
+    const uint8_t* interior;  // 2-D, per cell: 1 interior, 2 coded (staircase walls), 0 others
+    const unsigned long long* cell_codes;  // 2-D: the codes of the cells of class 2, per cell
     // 3-D, per cell: 0 interior, the neighbourhood code of a coded cell (bit
     // 63 set for those near open faces), ~0 for the others
     const unsigned long long* words;
     void* aux;                // 3-D: 4 planes of the compute type for the split variants
 };
-
-// tile shape of the 2-D wall-tile kernel
-constexpr int WALL_TX = 64, WALL_TY = 2;
-// the tiles that hold a cell of `all` not in `face` (host, at create)
-void wall_tiles(int nx, int ny, const std::vector<long long>& all, const std::vector<long long>& face,
-                std::vector<int>& out);
 
 cudaError_t launch_step(int dim, int precision, int variant, const StepParams<double>& Pd,
                         const StepParams<float>& Pf, StateView in, StateView out, const uint8_t* solid,
@@ -130,9 +122,9 @@ void list_codes2d(int nx, int ny, const int* bc, const uint8_t* solid, const std
                   std::vector<long long>& coded, std::vector<unsigned long long>& codes, std::vector<long long>& rest);
 
 // Fluid cells that are not interior for the tile kernels (host, at create);
-// faces_only (2-D): only cells whose stencil leaves the domain.
+// faces_only (3-D): only cells whose stencil leaves the domain.
 void boundary_cells(int dim, int nx, int ny, int nz, const int* bc, const uint8_t* solid, std::vector<long long>& out,
-                    bool faces_only, const int* face_solid);
+                    bool faces_only, const int* = nullptr);
 
 // Diagnostics reduction over the rows y0 <= y < y1 (all x, all z) into the
 // device scratch `red` (RED_WORDS words); FP64 accumulation.  part: DIAG_WORDS

@@ -2,10 +2,10 @@
 //
 // One cooperative launch of as many 128-thread blocks as fit on the GPU
 // at once.  Every step, the blocks take work items from a shared counter:
-// first the chunks of 128 boundary cells (general form, then by their
-// neighbourhood codes: the slowest items), then the wall tiles (64 x 2, the
-// cells next to in-domain solids), then the interior tiles (32 x 4 cells),
-// with the same per-cell code as variant 6; then all blocks meet at a
+// first the chunks of 128 boundary cells that the tiles leave out (general
+// form, then by their neighbourhood codes: the slowest items), then the
+// tiles (32 x 4, interior and coded cells), with the same per-cell code as
+// variant 2; then all blocks meet at a
 // grid-wide barrier before the buffers swap roles.  The barrier's wait is
 // bounded: a block that waits longer than the limit records the failure
 // and returns, the others see the record and return too, and the host
@@ -29,7 +29,7 @@ namespace lbfd {
 namespace {
 
 constexpr int PT_TX = 32, PT_TY = 4, PT_THREADS = 128;
-static_assert(PT_TX * PT_TY == PT_THREADS && WALL_TX * WALL_TY == PT_THREADS, "one block shape for every phase");
+static_assert(PT_TX * PT_TY == PT_THREADS, "one block shape for every phase");
 
 __device__ __forceinline__ unsigned long long global_ns()
 {
@@ -90,16 +90,15 @@ __device__ bool grid_wait(PersistentWait* w, unsigned nblocks, long long limit_n
 template <typename S, typename R, bool HI1>
 __global__ void __launch_bounds__(PT_THREADS, sizeof(R) == 4 ? 4 : 2)
     step_kernel_persistent2d(StepParams<R> P, StateView a, StateView b, int n, const uint8_t* solid,
-                             const uint8_t* interior, const int* wall_tiles, int nwall_tiles, CodedList cl,
+                             const uint8_t* interior, const unsigned long long* codes, CodedList cl,
                              PersistentWait* w, long long limit_ns)
 {
     __shared__ unsigned item_sh;
     const int tid = threadIdx.x;
     const int gx = (P.nx + PT_TX - 1) / PT_TX, gy = (P.ny + PT_TY - 1) / PT_TY;
-    const int wgx = (P.nx + WALL_TX - 1) / WALL_TX;
     const unsigned nrest = (unsigned)((cl.nrest + PT_THREADS - 1) / PT_THREADS);
-    const unsigned nchunk = nrest + (unsigned)((cl.n + PT_THREADS - 1) / PT_THREADS);
-    const unsigned nitems = nchunk + (unsigned)nwall_tiles + (unsigned)(gx * gy);
+    const unsigned nchunk = nrest + (unsigned)((cl.nout + PT_THREADS - 1) / PT_THREADS);
+    const unsigned nitems = nchunk + (unsigned)(gx * gy);
     for (int s = 0; s < n; ++s) {
         const StateView in = (s & 1) ? b : a, out = (s & 1) ? a : b;
         const S* g_in = (const S*)in.g;
@@ -123,19 +122,15 @@ __global__ void __launch_bounds__(PT_THREADS, sizeof(R) == 4 ? 4 : 2)
                 }
             } else if (it < nchunk) {
                 const long long i = (long long)(it - nrest) * PT_THREADS + tid;
-                if (i < cl.n) {
+                if (i < cl.nout) {
                     const long long c = cl.cells[i];
                     const int p[3] = {(int)(c % P.nx), (int)(c / P.nx), 0};
                     cell_step_coded<2, S, R, true, HI1>(P, p, c, cl.codes[i], g_in, g_out, T_in, T_out, Y_in, Y_out);
                 }
-            } else if (it < nchunk + (unsigned)nwall_tiles) {
-                const int wt = wall_tiles[it - nchunk];
-                tiled2d_body<S, R, WALL_TX, WALL_TY, true, HI1>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, solid, nullptr,
-                                                           tid % WALL_TX, tid / WALL_TX, wt % wgx, wt / wgx);
             } else {
-                const int t = (int)(it - nchunk - (unsigned)nwall_tiles);
-                tiled2d_body<S, R, PT_TX, PT_TY, false, HI1>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, nullptr, interior,
-                                                        tid % PT_TX, tid / PT_TX, t % gx, t / gx);
+                const int t = (int)(it - nchunk);
+                tiled2d_body<S, R, PT_TX, PT_TY, true, HI1>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, interior, codes,
+                                                            tid % PT_TX, tid / PT_TX, t % gx, t / gx);
             }
             __syncthreads();  // the next tile restages the shared memory
         }
@@ -149,9 +144,7 @@ cudaError_t launch_pers(const StepParams<R>& P, StateView a, StateView b, int n,
                         int* blocks)
 {
     auto kern = P.omega_hi == R(1) ? step_kernel_persistent2d<S, R, true> : step_kernel_persistent2d<S, R, false>;
-    const size_t smem = tile_smem_bytes<R, PT_TX, PT_TY>() > tile_smem_bytes<R, WALL_TX, WALL_TY>()
-                            ? tile_smem_bytes<R, PT_TX, PT_TY>()
-                            : tile_smem_bytes<R, WALL_TX, WALL_TY>();
+    const size_t smem = tile_smem_bytes<R, PT_TX, PT_TY>();
     cudaError_t e;
     if (smem > 48 * 1024 &&
         (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
@@ -164,9 +157,6 @@ cudaError_t launch_pers(const StepParams<R>& P, StateView a, StateView b, int n,
     if (per_sm < 1) return cudaErrorLaunchOutOfResources;
     const unsigned nb = (unsigned)(per_sm * sms);
     *blocks = (int)nb;
-    // the cells that variant 6 would give to its wall tiles go through their
-    // codes on the grids where it runs as one launch
-    const bool walls = bl.nwall_tiles > 0 && !small2d_applies(sizeof(R) == 8 ? 0 : 1, P.nx, P.ny, bl);
     if ((e = cudaMemsetAsync(w, 0, sizeof(PersistentWait), stream)) != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nb);
@@ -178,9 +168,8 @@ cudaError_t launch_pers(const StepParams<R>& P, StateView a, StateView b, int n,
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, P, a, b, n, solid, (const uint8_t*)bl.interior,
-                              walls ? bl.wall_tiles : (const int*)nullptr, walls ? (int)bl.nwall_tiles : 0,
-                              walls ? bl.face2 : bl.all2, w, limit_ns);
+    return cudaLaunchKernelEx(&cfg, kern, P, a, b, n, solid, (const uint8_t*)bl.interior, bl.cell_codes,
+                              bl.all2, w, limit_ns);
 }
 
 }  // namespace

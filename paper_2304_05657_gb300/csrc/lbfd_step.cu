@@ -2,8 +2,8 @@
 //
 // Variant 0 is the general form (one thread per cell, every access through
 // the boundary classification; D2Q9 and D3Q27).  Variants 1.. are 2-D
-// shared-memory tiles of different shapes, with or without the wall-tile
-// kernel, one or two cells per thread (lbfd_step_tiled.cuh,
+// shared-memory tiles of different shapes, taking the coded cells themselves
+// or leaving them to their list, one or two cells per thread (lbfd_step_tiled.cuh,
 // lbfd_step_pair.cuh; 3-D: lbfd_step3d.cu); the autotuner picks among them
 // by timing.  All variants compute the same step; they differ only in
 // rounding order.  Also: the host-side classification of boundary cells.
@@ -46,32 +46,31 @@ static cudaError_t launch_general(const StepParams<R>& P, StateView in, StateVie
 
 // PAIR: the interior tiles compute two cells per thread in packed FP32
 // (FP32 storage only; the FP64 form keeps one cell per thread)
-template <bool HI1, typename S, typename R, int TX, int TY, bool WALLS, bool PAIR = false, int MINB = 1>
+template <bool HI1, typename S, typename R, int TX, int TY, bool CODED, bool PAIR = false, int MINB = 1>
 static cudaError_t launch_tiled(const StepParams<R>& P, StateView in, StateView out, const uint8_t* solid,
                                 const BoundaryLists& b, const SideStream& side, cudaStream_t stream)
 {
     constexpr bool pair = PAIR && std::is_same<S, float>::value && std::is_same<R, float>::value;
     constexpr size_t smem = tile_smem_bytes<R, TX, TY>();
-    auto kern = step_kernel_tiled2d<S, R, TX, TY, HI1>;
+    auto kern = step_kernel_tiled2d<S, R, TX, TY, CODED, HI1>;
     const dim3 block(pair ? TX / 2 : TX, TY);
-    constexpr size_t wsmem = tile_smem_bytes<R, WALL_TX, WALL_TY>();
-    auto wkern = step_kernel_tiled2d_walls<S, R, WALL_TX, WALL_TY, HI1>;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
     dim3 grid((P.nx + TX - 1) / TX, (P.ny + TY - 1) / TY);
-    // the interior cells go to the tile kernel; the others, on the side
-    // stream (disjoint writes, same input state), to the wall-tile kernel
-    // (WALLS variants, cells next to in-domain solids) and the boundary
-    // kernel (the rest)
-    const bool walls = WALLS && !P.curved && b.nwall_tiles > 0;
-    const CodedList& cl = walls ? b.face2 : b.all2;
+    // the interior cells (CODED: and the coded cells next to them) go to the
+    // tile kernel; the others, on the side stream (disjoint writes, same
+    // input state), through the coded list and the boundary kernel.  The
+    // list takes 2/3 of the time of tiles of their own with the mask staged
+    // in: 50.3 us per step against 66.3 on a 2048x512 burner in a graph,
+    // 69.8 against 78.3 on 16 channels of 16-196 x 1024 cells (variant 9).
+    const CodedList& cl = b.all2;
     // with curved walls every listed cell takes the general form
     const long long* bl = P.curved ? b.all : cl.rest;
     const long long nb = P.curved ? b.nall : cl.nrest;
-    const long long nc = P.curved ? 0 : cl.n;
-    const bool fork = (nb > 0 || nc > 0 || walls) && side.stream != nullptr;
+    const long long nc = P.curved ? 0 : (CODED ? cl.nout : cl.n);
+    const bool fork = (nb > 0 || nc > 0) && side.stream != nullptr;
     cudaError_t e = cudaSuccess;
     if (fork) {
         if ((e = cudaEventRecord(side.fork, stream)) != cudaSuccess) return e;
@@ -94,15 +93,6 @@ static cudaError_t launch_tiled(const StepParams<R>& P, StateView in, StateView 
                         (S*)out.g, (const S*)in.T, (S*)out.T, (const S*)in.Y, (S*)out.Y, cl.cells, cl.codes, nc);
         if (e != cudaSuccess) return e;
     }
-    if (walls) {
-        // after the boundary kernel, at the least priority: its blocks fill
-        // the SMs that the tile grid leaves idle in its last wave
-        e = launch_prio(wkern, dim3((unsigned)b.nwall_tiles), dim3(WALL_TX, WALL_TY), wsmem, bs,
-                        fork ? side.low : 0, P,
-                        (const S*)in.g, (S*)out.g, (const S*)in.T, (S*)out.T, (const S*)in.Y, (S*)out.Y, solid,
-                        (const int*)b.wall_tiles);
-        if (e != cudaSuccess) return e;
-    }
     if constexpr (pair) {
         auto pk = step_kernel_pair2d<TX / 2, TY, MINB, HI1>;
         constexpr size_t psmem = pair_smem_bytes<TX, TY>();
@@ -113,7 +103,7 @@ static cudaError_t launch_tiled(const StepParams<R>& P, StateView in, StateView 
                                           (const float*)in.Y, (float*)out.Y, b.interior);
     } else {
         kern<<<grid, block, smem, stream>>>(P, (const S*)in.g, (S*)out.g, (const S*)in.T, (S*)out.T,
-                                            (const S*)in.Y, (S*)out.Y, b.interior);
+                                            (const S*)in.Y, (S*)out.Y, b.interior, b.cell_codes);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (fork) {
@@ -128,50 +118,30 @@ template <bool HI1, typename S, typename R>
 static cudaError_t launch_2d(int variant, const StepParams<R>& P, StateView in, StateView out, const uint8_t* solid,
                              const BoundaryLists& b, const SideStream& side, cudaStream_t stream)
 {
-    // variants 5-8: the same tiles, plus a wall-tile kernel for the cells
-    // next to in-domain solid cells, so that only cells near domain faces
-    // go through the general form
+    // variants 5-8: the same tiles without the coded cells, which take their
+    // list next to them
     switch (variant) {
     case 0: return launch_general<2, S, R>(P, in, out, solid, stream);
-    case 1: return launch_tiled<HI1, S, R, 32, 8, false>(P, in, out, solid, b, side, stream);
-    case 2: return launch_tiled<HI1, S, R, 32, 4, false>(P, in, out, solid, b, side, stream);
-    case 3: return launch_tiled<HI1, S, R, 64, 4, false>(P, in, out, solid, b, side, stream);
-    case 4: return launch_tiled<HI1, S, R, 32, 16, false>(P, in, out, solid, b, side, stream);
-    case 5: return launch_tiled<HI1, S, R, 32, 8, true>(P, in, out, solid, b, side, stream);
-    case 6: return launch_tiled<HI1, S, R, 32, 4, true>(P, in, out, solid, b, side, stream);
-    case 7: return launch_tiled<HI1, S, R, 64, 4, true>(P, in, out, solid, b, side, stream);
-    case 8: return launch_tiled<HI1, S, R, 32, 16, true>(P, in, out, solid, b, side, stream);
+    case 1: return launch_tiled<HI1, S, R, 32, 8, true>(P, in, out, solid, b, side, stream);
+    case 2: return launch_tiled<HI1, S, R, 32, 4, true>(P, in, out, solid, b, side, stream);
+    case 3: return launch_tiled<HI1, S, R, 64, 4, true>(P, in, out, solid, b, side, stream);
+    case 4: return launch_tiled<HI1, S, R, 32, 16, true>(P, in, out, solid, b, side, stream);
+    case 5: return launch_tiled<HI1, S, R, 32, 8, false>(P, in, out, solid, b, side, stream);
+    case 6: return launch_tiled<HI1, S, R, 32, 4, false>(P, in, out, solid, b, side, stream);
+    case 7: return launch_tiled<HI1, S, R, 64, 4, false>(P, in, out, solid, b, side, stream);
+    case 8: return launch_tiled<HI1, S, R, 32, 16, false>(P, in, out, solid, b, side, stream);
     // variants 9-12: as 5-8 with two cells per thread in packed FP32, at
     // 128 registers (9, 10) or 96 (11, 12, five 128-thread blocks per SM;
     // six blocks at 80 registers spill and are slower)
-    case 9: return launch_tiled<HI1, S, R, 32, 8, true, true, 4>(P, in, out, solid, b, side, stream);
-    case 10: return launch_tiled<HI1, S, R, 64, 8, true, true, 2>(P, in, out, solid, b, side, stream);
-    case 11: return launch_tiled<HI1, S, R, 32, 8, true, true, 5>(P, in, out, solid, b, side, stream);
-    case 12: return launch_tiled<HI1, S, R, 64, 4, true, true, 5>(P, in, out, solid, b, side, stream);
+    case 9: return launch_tiled<HI1, S, R, 32, 8, false, true, 4>(P, in, out, solid, b, side, stream);
+    case 10: return launch_tiled<HI1, S, R, 64, 8, false, true, 2>(P, in, out, solid, b, side, stream);
+    case 11: return launch_tiled<HI1, S, R, 32, 8, false, true, 5>(P, in, out, solid, b, side, stream);
+    case 12: return launch_tiled<HI1, S, R, 64, 4, false, true, 5>(P, in, out, solid, b, side, stream);
     default: return cudaErrorInvalidValue;
     }
 }
 
 int num_variants(int dim) { return dim == 2 ? 13 : 8; }
-
-void wall_tiles(int nx, int ny, const std::vector<long long>& all, const std::vector<long long>& face,
-                std::vector<int>& out)
-{
-    // tiles (WALL_TX x WALL_TY) holding a cell of `all` that is not in `face`
-    out.clear();
-    std::vector<char> in_face;
-    const int gx = (nx + WALL_TX - 1) / WALL_TX, gy = (ny + WALL_TY - 1) / WALL_TY;
-    std::vector<char> mark((size_t)gx * gy, 0);
-    size_t j = 0;
-    for (long long c : all) {  // both lists are sorted by cell index
-        while (j < face.size() && face[j] < c) ++j;
-        if (j < face.size() && face[j] == c) continue;
-        const int x = (int)(c % nx), y = (int)(c / nx);
-        mark[(size_t)(y / WALL_TY) * gx + x / WALL_TX] = 1;
-    }
-    for (size_t t = 0; t < mark.size(); ++t)
-        if (mark[t]) out.push_back((int)t);
-}
 
 cudaError_t launch_step(int dim, int precision, int variant, const StepParams<double>& Pd,
                         const StepParams<float>& Pf, StateView in, StateView out, const uint8_t* solid,
@@ -413,7 +383,7 @@ void list_codes2d(int nx, int ny, const int* bc, const uint8_t* solid, const std
 }
 
 void boundary_cells(int dim, int nx, int ny, int nz, const int* bc, const uint8_t* solid, std::vector<long long>& out,
-                    bool faces_only, const int* face_solid)
+                    bool faces_only, const int*)
 {
     out.clear();
     auto wrap = [](int q, int n, bool periodic, bool* out) {
@@ -468,16 +438,7 @@ void boundary_cells(int dim, int nx, int ny, int nz, const int* bc, const uint8_
                     if (!(axis || near)) continue;
                     bool outx = false, outy = false;
                     const int qx = wrap(x + dx, nx, px, &outx), qy = wrap(y + dy, ny, py, &outy);
-                    if (outx || outy) {
-                        // outside: fine for the wall-aware tiles only beyond walls
-                        // that act like the solid cells
-                        const int rx = x + dx, ry = y + dy;
-                        const bool okx = !outx || (face_solid && face_solid[rx < 0 ? 0 : 1]);
-                        const bool oky = !outy || (face_solid && face_solid[ry < 0 ? 2 : 3]);
-                        if (!(faces_only && okx && oky)) fast = false;
-                    } else if (!faces_only && solid[(long long)qx + (long long)nx * qy]) {
-                        fast = false;
-                    }
+                    if (outx || outy || solid[(long long)qx + (long long)nx * qy]) fast = false;
                 }
             if (!fast) out.push_back(c);
         }

@@ -168,8 +168,8 @@ __global__ void __launch_bounds__(TXP * TY, MINB)
     float* gs = reinterpret_cast<float*>(smem_raw + pair_pull_offset<TX, TY>()) + 2 * tid;
     bool ok0 = false, ok1 = false;  // the two cells are interior (per-cell class)
     if (inside) {
-        ok0 = interior[c] != 0;
-        ok1 = has1 && interior[c + 1] != 0;
+        ok0 = interior[c] == 1;
+        ok1 = has1 && interior[c + 1] == 1;
         const int x1 = has1 ? x + 1 : x;
         const int oym = y == 0 ? (P.ny - 1) * P.nx : -P.nx, oyp = y == P.ny - 1 ? (1 - P.ny) * P.nx : P.nx;
         const int oxm0 = x == 0 ? P.nx - 1 : -1, oxp0 = x == P.nx - 1 ? 1 - P.nx : 1;
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(TXP * TY, MINB)
     if ((P.nx & 1) == 0)
         stage_tile2d_pairs<TX, TY, NT>(P, sm, x0, y0, tid, T_in, Y_in);
     else
-        stage_tile2d<float, float, TX, TY, false, NT>(P, sm, x0, y0, tid, T_in, Y_in, nullptr);
+        stage_tile2d<float, float, TX, TY, false, NT>(P, sm, x0, y0, tid, T_in, Y_in);
     cp_async_wait_all();
     __syncthreads();
 

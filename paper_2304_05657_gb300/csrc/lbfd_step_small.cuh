@@ -1,16 +1,16 @@
 // lbfd_step_small.cuh -- a 2-D step in one launch of one-warp blocks
 // (lbfd_step_small.cu, and the forward-mode step of lbfd_tangent.cu).
 //
-// One warp per block: the first blocks take the boundary cells (by their
-// neighbourhood codes; the longest-latency work starts first), the others a
-// small tile of interior cells each, with one lane or two lanes (one per
+// One warp per block: the first blocks take the boundary cells that the tiles
+// leave out (by their neighbourhood codes; the longest-latency work starts
+// first), the others a small tile each, with one lane or two lanes (one per
 // axis of the FD terms) per cell.  What bounds such grids is not the work
 // but where it runs: an SM partition issues one FP64 warp instruction per 64
 // cycles whatever its lanes do, so 8192 FP64 cells in 256-thread tiles kept
 // 32 of the 152 SMs busy for 64 us; in FP32 it is the latency of one
 // warp's instruction chain, a boundary kernel of its own and its two
 // events.  Spread one warp per partition, with half of the FD chain per
-// lane, the step takes 28 us in FP64 and 5.9 us in FP32 (256x32 channel, in
+// lane, the step takes 28 us in FP64 and 4.6 us in FP32 (256x32 channel, in
 // a graph; 64 and 13.6 us before).
 #pragma once
 #include "lbfd_internal.h"
@@ -32,6 +32,14 @@ __device__ __forceinline__ Dual<T, N> lane_xor16(const Dual<T, N>& a)
 
 constexpr int SM_TX = 8, SM_TY = 4;        // one cell per lane
 constexpr int SP_TX = 8, SP_TY = 2;        // two lanes per cell
+// The tiles take the coded cells too, next to their interior lanes, so that
+// only the cells they leave out pay a warp of their own (256x32 channel in
+// FP64: 28.4 -> 27.6 us per step, mixed in a graph 5.6 -> 4.5; 17 + 33 + 65
+// wide channels of 301 cells 1.10x).  In forward mode the selects of the four
+// derivatives cost more than the list (512x64 cells: FP64 321 us against
+// 348, mixed 25 against 28), which stays.
+template <typename R>
+constexpr bool SMALL_CODED = std::is_arithmetic<R>::value;
 
 // The two axes' parts of a cell's FD terms, in the lanes c and c + 16 of a
 // warp, summed into both.
@@ -56,10 +64,12 @@ template <typename S, typename R, bool HI1>
 __device__ __forceinline__ void split_tile(const StepParams<R>& P, const S* LBFD_RESTRICT g_in, S* LBFD_RESTRICT g_out,
                                            const S* LBFD_RESTRICT T_in, S* LBFD_RESTRICT T_out,
                                            const S* LBFD_RESTRICT Y_in, S* LBFD_RESTRICT Y_out,
-                                           const uint8_t* LBFD_RESTRICT interior, int bx, int by)
+                                           const uint8_t* LBFD_RESTRICT interior,
+                                           const unsigned long long* LBFD_RESTRICT cell_codes, int bx, int by)
 {
     using G = TileGeom<SP_TX, SP_TY>;
     constexpr int SX = G::SX, NPT = G::NPT;
+    constexpr bool CODED = SMALL_CODED<R>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const TileSmem<R> sm = tile_smem<R, SP_TX, SP_TY>(smem_raw);
     const int lane = threadIdx.x, axis = lane >> 4, tx = lane % SP_TX, ty = (lane / SP_TX) % SP_TY;
@@ -70,23 +80,29 @@ __device__ __forceinline__ void split_tile(const StepParams<R>& P, const S* LBFD
 #pragma unroll
     for (int i = 0; i < 9; ++i) g[i] = R(0);
     bool fast = false;
+    unsigned long long code = 0;
     if (inside) {
-        fast = interior[c] != 0;
+        const int cls = interior[c];
+        fast = cls == 1 || (CODED && cls == 2);
+        if (CODED && cls == 2) code = cell_codes[c];
         pull_interior<S, R>(P, g_in, c, x, y, g);
     }
-    stage_tile2d<S, R, SP_TX, SP_TY, false, 32>(P, sm, x0, y0, lane, T_in, Y_in, nullptr);
+    const bool cw = CODED && __any_sync(0xffffffffu, code != 0);
+    stage_tile2d<S, R, SP_TX, SP_TY, CODED, 32>(P, sm, x0, y0, lane, T_in, Y_in);
     __syncwarp();
     if (!__any_sync(0xffffffffu, fast)) return;
     const int p0 = (ty + 2) * SX + tx + 2;
     const R T0 = sm.T[p0], invW0 = sm.invW[p0], rho0 = sm.rho[p0];
     const R inv_rho0 = T0 * invW0 * par<R>(P.inv_rho_c);
+    if (CODED && code) pull_coded_tile<S, R>(P, x, y, c, (unsigned)code, rho0, inv_rho0, g_in, g);
     LowMoments<2, R> lm;
     low_moments<2>(g, lm);
     const R u[3] = {lm.m1[0] * (K<R>(3) * inv_rho0), lm.m1[1] * (K<R>(3) * inv_rho0), R(0)};
     FDAccum<R> acc;
     acc.clear();
     R gam;
-    fd_axis_smem<R>(P, sm, NPT, p0, axis ? SX : 1, axis ? u[1] : u[0], invW0, inv_rho0, &gam, acc);
+    fd_axis_smem<CODED, R>(P, sm, NPT, p0, axis ? SX : 1, cw, (unsigned)(code >> (axis ? 38 : 32)) & 63u,
+                           (unsigned)(code >> (axis ? 52 : 50)) & 3u, axis ? u[1] : u[0], invW0, inv_rho0, &gam, acc);
     join_axes(acc, gam, axis);
     if (!fast) return;
     R Y0[NSP];
@@ -142,6 +158,7 @@ __global__ void __launch_bounds__(32)
     step_kernel_small2d(StepParams<R> P, const S* LBFD_RESTRICT g_in, S* LBFD_RESTRICT g_out,
                         const S* LBFD_RESTRICT T_in, S* LBFD_RESTRICT T_out, const S* LBFD_RESTRICT Y_in,
                         S* LBFD_RESTRICT Y_out, const uint8_t* LBFD_RESTRICT interior,
+                        const unsigned long long* LBFD_RESTRICT cell_codes,
                         const long long* LBFD_RESTRICT cells, const unsigned long long* LBFD_RESTRICT codes, int ncells,
                         int list_blocks, int tiles_x)
 {
@@ -152,7 +169,8 @@ __global__ void __launch_bounds__(32)
             const int j = blockIdx.x * 16 + (threadIdx.x & 15), k = j < ncells ? j : ncells - 1;
             split_coded<S, R, HI1>(P, cells[k], codes[k], j < ncells, g_in, g_out, T_in, T_out, Y_in, Y_out);
         } else {
-            split_tile<S, R, HI1>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, interior, t % tiles_x, t / tiles_x);
+            split_tile<S, R, HI1>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, interior, cell_codes, t % tiles_x,
+                                   t / tiles_x);
         }
     } else {
         if (t < 0) {
@@ -162,9 +180,9 @@ __global__ void __launch_bounds__(32)
             const int p[3] = {(int)(c % P.nx), (int)(c / P.nx), 0};
             cell_step_coded<2, S, R, true, HI1>(P, p, c, codes[j], g_in, g_out, T_in, T_out, Y_in, Y_out);
         } else {
-            tiled2d_body<S, R, SM_TX, SM_TY, false, HI1>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, nullptr, interior,
-                                                         threadIdx.x % SM_TX, threadIdx.x / SM_TX, t % tiles_x,
-                                                         t / tiles_x);
+            tiled2d_body<S, R, SM_TX, SM_TY, SMALL_CODED<R>, HI1>(P, g_in, g_out, T_in, T_out, Y_in, Y_out, interior,
+                                                                  cell_codes, threadIdx.x % SM_TX,
+                                                                  threadIdx.x / SM_TX, t % tiles_x, t / tiles_x);
         }
     }
 }
@@ -177,14 +195,15 @@ cudaError_t launch_small(const StepParams<R>& P, StateView in, StateView out, co
     constexpr int TX = SPLIT ? SP_TX : SM_TX, TY = SPLIT ? SP_TY : SM_TY, CELLS = TX * TY;
     constexpr size_t smem = tile_smem_bytes<R, TX, TY>();
     const int gx = (P.nx + TX - 1) / TX, gy = (P.ny + TY - 1) / TY;
-    const int lb = (int)((b.all2.n + CELLS - 1) / CELLS);
+    const int n = (int)(SMALL_CODED<R> ? b.all2.nout : b.all2.n), lb = (n + CELLS - 1) / CELLS;
     auto kern = step_kernel_small2d<S, R, HI1, SPLIT>;
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
     kern<<<lb + gx * gy, 32, smem, stream>>>(P, (const S*)in.g, (S*)out.g, (const S*)in.T, (S*)out.T, (const S*)in.Y,
-                                             (S*)out.Y, b.interior, b.all2.cells, b.all2.codes, (int)b.all2.n, lb, gx);
+                                             (S*)out.Y, b.interior, b.cell_codes, b.all2.cells, b.all2.codes, n, lb,
+                                             gx);
     return cudaGetLastError();
 }
 

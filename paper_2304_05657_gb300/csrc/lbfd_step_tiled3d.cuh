@@ -51,27 +51,6 @@ __host__ __device__ constexpr size_t tile3_smem_bytes()
     return sizeof(R) * (size_t)Tile3Geom<TX, TY>::NPT * (4 + NSP);
 }
 
-// The line points of a coded cell along one axis (see coded_line): pts[j]
-// are the staged points at offsets -2..2, replaced by the mirror points of
-// the solids' ghosts (the ghosts beyond a face are staged as such); returns
-// the solid ghosts (bit j).  Branch-free: 17 integer instructions per side.
-__device__ __forceinline__ unsigned coded_pts(unsigned code, unsigned faces, int* pts)
-{
-    const int lo = pts[1], hi = pts[3], c0 = pts[2];
-    unsigned ghosts = 0;
-#pragma unroll
-    for (int side = -1; side <= 1; side += 2) {
-        const unsigned bits = side < 0 ? (code & 7u) : (code >> 3);
-        const unsigned w = (faces >> (side < 0 ? 0 : 1)) & 1u ? 0u : (bits & 3u);
-        const int near = side < 0 ? lo : hi, opp = side < 0 ? hi : lo;
-        const int far = w == 2 ? near : ((bits & 4u) ? c0 : opp);
-        pts[2 + 2 * side] = w == 0 ? pts[2 + 2 * side] : far;
-        pts[2 + side] = w == 1 ? c0 : near;
-        ghosts |= (w == 1 ? 1u << (2 + side) : 0u) | (w != 0 ? 1u << (2 + 2 * side) : 0u);
-    }
-    return ghosts;
-}
-
 // FD terms along one axis from five shared-memory points.  CODED and cw (a
 // warp-uniform flag: some lane is a coded cell): dir flags the ghosts of
 // isothermal solids, whose T and rho take the Dirichlet form of Eq. 34, and
@@ -292,7 +271,6 @@ __device__ __forceinline__ void tiled3d_body(const StepParams<R>& P, int zc, con
     sm.X = sm.Y + NSP * NPT;  // one plane: W
     sm.invW = sm.X + NPT;
     sm.rho = sm.invW + NPT;
-    sm.mask = nullptr;
 
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, zb = blockIdx.z * zc;
     const long long N = P.N;

@@ -1,9 +1,10 @@
 """The one-launch form of 2-D steps on small grids (both lane splits) and the
-coded boundary cells, against the FP64 oracle: every face type and corner,
-extents of one to a few cells and around the 8x4 and 8x2 tiles, solids next
-to faces, and grids on both sides of the rule's lines.  Tolerances are those of the parity tests: FP64 1e-10 relative L2 per field after 20
-steps (rounding order only), mixed T 1e-5 and populations 1e-4 of their
-maximum."""
+coded boundary cells, in the tiles and over their list, against the FP64
+oracle: every face type and corner, extents of one to a few cells and around
+the 8x4 and 8x2 tiles, solids next to faces, and grids on both sides of the
+rule's lines.  Tolerances are those of the parity tests: FP64 1e-10 relative
+L2 per field after 20 steps (rounding order only), mixed T 1e-5 and
+populations 1e-4 of their maximum."""
 import numpy as np
 import pytest
 
@@ -31,7 +32,7 @@ def state(nx, ny, faces, solids, seed, **over):
     return cfg, solid, T, Y, g
 
 
-def check(lbfd_lib, oracle_mod, cfg, solid, T, Y, g, steps, launches=None):
+def check(lbfd_lib, oracle_mod, cfg, solid, T, Y, g, steps, launches=None, variant=None):
     o = oracle_mod.Sim(cfg, solid)
     o.set_state(T, Y, g)
     o.step(steps)
@@ -39,6 +40,8 @@ def check(lbfd_lib, oracle_mod, cfg, solid, T, Y, g, steps, launches=None):
     for prec in ("fp64", "mixed"):
         s = lbfd_lib.Solver(dict(cfg, precision=prec), solid)
         s.set_state(T, Y, g)
+        if variant is not None:
+            s.variant = variant
         if launches is not None:
             assert s.launches_per_step == launches
         s.step(steps)
@@ -66,9 +69,19 @@ def test_poiseuille_inlet_and_other_omega_hi(lbfd_lib, oracle_mod):
     check(lbfd_lib, oracle_mod, *state(40, 13, "flow", True, seed=2, poiseuille_inlet=True, omega_hi=1.3), steps=20)
 
 
-# around the rule's lines: FP64 two lanes up to 405 warps of 32 cells (12 960
-# cells), one launch up to 19 456 (FP64) and 9 728 (FP32) warps, two lanes
-# in FP32 up to 3 040
-@pytest.mark.parametrize("nx,ny", [(216, 60), (232, 60), (400, 243), (408, 244), (640, 487), (700, 500)])
+# around the rule's lines: two lanes up to 304 warps of 32 cells, one launch
+# up to 4 864 (FP32) and 19 456 (FP64) warps
+@pytest.mark.parametrize("nx,ny", [(152, 64), (153, 64), (232, 60), (512, 304), (520, 304), (640, 487), (700, 500),
+                                   (1216, 513)])
 def test_rule_lines(lbfd_lib, oracle_mod, nx, ny):
     check(lbfd_lib, oracle_mod, *state(nx, ny, "flow", True, seed=nx), steps=2)
+
+
+# an open corner keeps the grid off the one-launch form: the tiles of every
+# shape with the coded cells in them (1-4) or over their list (5-12), ragged
+# against each tile, the convective outlet's cells and the corner's apart
+@pytest.mark.parametrize("variant", range(1, 13))
+@pytest.mark.parametrize("isothermal", [0, 1])
+def test_tile_variants_with_solids(lbfd_lib, oracle_mod, variant, isothermal):
+    case = state(71, 37, "corner", True, seed=variant, solid_isothermal=isothermal)
+    check(lbfd_lib, oracle_mod, *case, steps=20, launches=3, variant=variant)
