@@ -331,12 +331,12 @@ int lbfd_gradient(lbfd_handle* h, int objective, double* value, double* grad);
  * values: by hand-derived local adjoints of every cell's step when
  * omega_hi = 1 and there is neither a convective outlet nor a cell with a
  * link through two open faces, else by recording every fluid cell's step on
- * a reverse-mode tape and sweeping it backwards.  The forward pass keeps a copy of the state
- * every `checkpoint_every` steps; the backward pass recomputes each segment
- * from its copy with the forward kernels (FP32 ones for LBFD_MIXED) and
- * evaluates every step's adjoint at that trajectory, the step differentiated
- * in FP64 (by a tape for LBFD_MIXED: FP32 values and partials), accumulating
- * lambda and the gradient in FP64.
+ * a reverse-mode tape and sweeping it backwards.  The forward pass keeps a
+ * copy of the state every `checkpoint_every` steps; the backward pass
+ * recomputes each segment from its copy with the forward kernels (FP32 ones
+ * for LBFD_MIXED) and evaluates every step's adjoint at that trajectory, the
+ * step differentiated in FP64 (by a tape for LBFD_MIXED: FP32 values and
+ * partials), accumulating lambda and the gradient in FP64.
  *
  * lbfd_adjoint_setup: the checkpoint interval of later calls (default 200).
  * lbfd_adjoint_record: advance the handle's state by `steps` steps, keeping
@@ -351,11 +351,12 @@ int lbfd_gradient(lbfd_handle* h, int objective, double* value, double* grad);
  * lbfd_adjoint_gradient: lbfd_adjoint_run with this checkpoint interval
  *   for the one call.
  * Device memory of a backward call: checkpoint_every + 2 state copies and
- *   two FP64 adjoint states, plus tapes of at most 12 GB: 20 B (12 B for
- *   LBFD_MIXED) x 2048 nodes per cell and recorded step, in two buffers of up to 4 steps each (one
- *   recorded while the other is swept) when they fit, else one step with
- *   its cells in chunks; and 8 B x 2048 nodes per cell for the sweep.  A
- *   step that needs more nodes is taken again with 4096.  Freed before
+ *   two FP64 adjoint states.  With tapes also at most 12 GB of them: 20 B
+ *   (12 B for LBFD_MIXED) x 2048 nodes per cell and recorded step, in two
+ *   buffers of up to 4 steps each (one recorded while the other is swept)
+ *   when they fit, else one step with its cells in chunks; and 8 B x 2048
+ *   nodes per cell for the sweep.  A step that needs more nodes is taken
+ *   again with 4096.  Freed before
  *   returning.  All synchronise.
  * Errors: LBFD_EINVAL (arguments, backward without a record), LBFD_ENOTSUP
  * (other precision, 3-D, curved walls, or a cell whose step needs more than
