@@ -749,7 +749,7 @@ def run_ours(args):
                      "frac": achieved / peak, "peak_kind": peak_kind, "traffic": traffic,
                      "traffic_unit": "DRAM bytes per step (ncu, all kernels of one step)",
                      "algorithmic_bytes_per_step": alg_bytes, "algorithmic_bytes_per_cell": bpc,
-                     "kernel": "one lbfd_step (the tile kernel with its boundary and wall kernels)",
+                     "kernel": "one lbfd_step (the tile kernel with the lists of the cells it leaves out)",
                      "mean_launch_ms": mean_s * 1e3, "issue": issue},
         "e2e": {"value": e2e_value, "unit": "MLUPS", "h2d_bytes_per_step": nbytes, "d2h_bytes_per_step": nbytes,
                 "steps": e2e_steps, "api": "lbfd_set_state_raw + lbfd_step + lbfd_get_state_raw (pinned)"},

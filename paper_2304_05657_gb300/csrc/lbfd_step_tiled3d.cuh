@@ -372,7 +372,8 @@ __device__ __forceinline__ void tiled3d_body(const StepParams<R>& P, int zc, con
             R Y0[NSP];
 #pragma unroll
             for (int k = 0; k < NSP; ++k) Y0[k] = sm.Y[k * NPT + p0];
-            const R Lam = update_scalars<S, R>(P, c, T0, Y0, rho0 * invW0 * par<R>(P.inv_rho_c), sm.X[p0], acc, T_out, Y_out);
+            const R Lam = update_scalars<S, R>(P, c, T0, Y0, rho0 * invW0 * par<R>(P.inv_rho_c), sm.X[p0], acc, T_out,
+                                               Y_out);
             if constexpr (SPLIT) {
                 aux[c] = Lam;
 #pragma unroll
@@ -409,7 +410,8 @@ __global__ void __launch_bounds__(TX * TY, MINB)
 // four 128-thread blocks per SM
 template <typename S, typename R, int TX, int TY>
 __global__ void __launch_bounds__(TX * TY, sizeof(R) == 4 ? 512 / (TX * TY) : 1)
-    step_kernel_fd3d(StepParams<R> P, int zc, const S* LBFD_RESTRICT g_in, const S* LBFD_RESTRICT T_in, S* LBFD_RESTRICT T_out,
+    step_kernel_fd3d(StepParams<R> P, int zc, const S* LBFD_RESTRICT g_in, const S* LBFD_RESTRICT T_in,
+                     S* LBFD_RESTRICT T_out,
                      const S* LBFD_RESTRICT Y_in, S* LBFD_RESTRICT Y_out,
                      const unsigned long long* LBFD_RESTRICT words, R* LBFD_RESTRICT aux)
 {

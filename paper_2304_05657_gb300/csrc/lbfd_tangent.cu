@@ -73,8 +73,9 @@ static cudaError_t step_tangent(int dim, const StepParams<TT>& P, StateView in, 
             const cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) return e;
         }
-        return small_warps(P.nx, P.ny) <= (sizeof(TT) == sizeof(Tan) ? 2 * PARTITIONS / 3 : 2 * PARTITIONS) ? launch_small<TT, TT, true, true>(P, in, out, b, stream)
-                                                             : launch_small<TT, TT, true, false>(P, in, out, b, stream);
+        const bool split = small_warps(P.nx, P.ny) <= (sizeof(TT) == sizeof(Tan) ? 2 * PARTITIONS / 3 : 2 * PARTITIONS);
+        return split ? launch_small<TT, TT, true, true>(P, in, out, b, stream)
+                     : launch_small<TT, TT, true, false>(P, in, out, b, stream);
     }
     const unsigned blocks = (unsigned)((P.ncell + 127) / 128);
     auto kern = val(P.omega_hi) == 1.0 ? step_kernel_tangent<2, TT, true> : step_kernel_tangent<2, TT, false>;
