@@ -197,6 +197,17 @@ __device__ __forceinline__ void eos_w(const StepParams<PR>& P, R T, R invW, R& r
     rho = par<R>(P.rho_c) * r;
     W = T * r;
 }
+// In forward mode W by its own reciprocal: where Y is uniform, W and its
+// derivatives (0) are then so exactly.  T r leaves the rounding of T there,
+// which the species equations integrate (mixed form, 512x64 channel with 0.3 K
+// of noise, 1000 steps: dJ/dT_wall 6.5e-5 off FP64, 1.7e-6 with this).
+template <typename PR, typename T, int N>
+__device__ __forceinline__ void eos_w(const StepParams<PR>& P, Dual<T, N> Tc, Dual<T, N> invW, Dual<T, N>& rho,
+                                      Dual<T, N>& W)
+{
+    rho = par<Dual<T, N>>(P.rho_c) * frcp(Tc * invW);
+    W = frcp(invW);
+}
 
 // Single-step rate per unit mass of fuel, per step.  The mixed form
 // evaluates it in FP64 where T > T_fp64.
