@@ -22,8 +22,11 @@
 namespace lbfd {
 
 // the value `off` bytes from a pointer that is uniform over the block: a
-// 32-bit offset keeps the 64-bit arithmetic out of the lanes (in-plane
-// offsets of every grid that fits the device are below 2^32 bytes)
+// 32-bit offset keeps the 64-bit arithmetic out of the lanes.  In-plane
+// offsets of a state array stay below 2^32 bytes on every grid that fits the
+// device: 2^30 FP32 cells of 297 bytes each (two states, the split variants'
+// planes, word, read-out value, mask) or 2^29 FP64 cells of 577 are 319 and
+// 310 GB.
 template <typename S>
 __device__ __forceinline__ const S* at_bytes(const S* base, unsigned off)
 {
@@ -33,6 +36,15 @@ template <typename S>
 __device__ __forceinline__ S* at_bytes(S* base, unsigned off)
 {
     return reinterpret_cast<S*>(reinterpret_cast<char*>(base) + off);
+}
+
+// the cell whose value lies `off` bytes into a plane of S that starts at cell
+// `base`: the words are indexed by it in 64 bits, 8 bytes a cell for either S
+// (as a 32-bit byte offset they would wrap from 2^29 cells a plane on)
+template <typename S>
+__host__ __device__ __forceinline__ long long cell_at(long long base, unsigned off)
+{
+    return base + off / (unsigned)sizeof(S);
 }
 
 template <int TX, int TY>
@@ -300,20 +312,19 @@ __device__ __forceinline__ void tiled3d_body(const StepParams<R>& P, int zc, con
 #pragma unroll
             for (int a = 0; a < 3; ++a) oxy[b][a] = (xs[a] + (unsigned)P.nx * ys[b]) * (unsigned)sizeof(S);
     }
-    constexpr unsigned WB = sizeof(unsigned long long) / sizeof(S);
     constexpr unsigned long long OTHER = ~0ull;  // solid, or another kernel's cell
-    unsigned long long next = inside ? *at_bytes(words + plane * zb, oxy[1][1] * WB) : OTHER;
+    unsigned long long next = inside ? words[cell_at<S>(plane * zb, oxy[1][1])] : OTHER;
     for (int z = zb; z < zend; ++z) {
         // what the cell is; the next plane's word is loaded meanwhile
         unsigned long long word = next;
         if (word != 0 && !(CODED && (coded_cells == 2 || (coded_cells == 1 && !(word >> 63))))) word = OTHER;
         const bool active = word != OTHER, coded = CODED && active && word != 0;
         const bool cw = CODED && __any_sync(0xffffffffu, coded);
-        if (z + 1 < zend && inside) next = *at_bytes(words + plane * (z + 1), oxy[1][1] * WB);
+        if (z + 1 < zend && inside) next = words[cell_at<S>(plane * (z + 1), oxy[1][1])];
         // a1 issued before the staging of plane z+2, so that the population
         // loads are in flight meanwhile
         const long long zo[3] = {plane * (z == 0 ? P.nz - 1 : z - 1), plane * z, plane * (z == P.nz - 1 ? 0 : z + 1)};
-        const long long c = zo[1] + oxy[1][1] / (unsigned)sizeof(S);
+        const long long c = cell_at<S>(zo[1], oxy[1][1]);
         R g[27];
 #pragma unroll
         for (int i = 0; i < 27; ++i)
