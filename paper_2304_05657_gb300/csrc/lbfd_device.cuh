@@ -327,7 +327,9 @@ __device__ __forceinline__ Dual<T, ND> conv_deriv(const Dual<T, ND>* v, bool neg
     const T t1 = (s - q) * i1, t0 = (q - p) * i0, w = t1 + t0, qe = q * eq;
     T rp = -(hB * i0) * (T(1) + T(8) * t0 * (p * ep));
     T rs = hB * i1 * (T(1) - T(2) * t1 * (s * es));
-    T rq = T(1) + T(2) * qe * w + hB * ((i0 - i1) - T(4) * qe * (t1 * i1 + t0 * i0));
+    // (i ~ 1 / eps^2 and t ~ eps^-3/2 where the field is nearly uniform: their
+    // product would leave the FP32 range from eps = 1e-11 down, hB i is of order 1)
+    T rq = T(1) + T(2) * qe * w + hB * (i0 - i1) - T(4) * qe * ((hB * i1) * t1 + (hB * i0) * t0);
     Dual<T, ND> r;
     r.v = q + hB * w;
     if (CENTRED && near) {
