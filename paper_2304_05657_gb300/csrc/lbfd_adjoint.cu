@@ -234,8 +234,10 @@ static StepParams<RevT<V>> rev_params(const StepParams<double>& D)
     P.T_solid = D.solid_isothermal ? Rv(D.T_solid, 2) : Rv(D.T_solid);
     P.solid_isothermal = D.solid_isothermal;
     P.poiseuille = D.poiseuille;
-    P.epsY = Rv(D.epsY);
-    P.epsT = Rv(D.epsT);
+    // (the FP32 tape takes the epsilons of the FP32 step that it records)
+    const double eps_lo = sizeof(V) == 4 ? WENO_EPS_LOW_FP32 : WENO_EPS_LOW_FP64;
+    P.epsY = Rv(D.epsY > eps_lo ? D.epsY : eps_lo);
+    P.epsT = Rv(D.epsT > eps_lo ? D.epsT : eps_lo);
     P.cs = Rv(D.cs);
     P.curved = 0;
     P.link_row = nullptr;

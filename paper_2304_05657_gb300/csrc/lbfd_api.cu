@@ -193,9 +193,7 @@ void fill_params(const lbfd_handle* h, StepParams<R>& P)
     P.rho_solid = (R)(p.T_in * invW_in / p.T_solid);  // (FP64 and mixed tiles)
     P.solid_isothermal = p.solid_isothermal;
     P.poiseuille = p.poiseuille_inlet;
-    // the WENO3 weights hold eps^2 (FP32) and eps^4 (FP64): kept in range (the
-    // limits lie far below the squared resolution of any field)
-    const double eps_lo = sizeof(R) % 8 ? 1e-18 : 1e-75;
+    const double eps_lo = sizeof(R) % 8 ? lbfd::WENO_EPS_LOW_FP32 : lbfd::WENO_EPS_LOW_FP64;
     P.epsY = (R)std::max(p.weno_eps, eps_lo);
     P.epsT = (R)std::max(p.weno_eps * p.T_in * p.T_in, eps_lo);
     P.cs = (R)sqrt(cs2);

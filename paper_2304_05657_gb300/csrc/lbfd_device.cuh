@@ -304,10 +304,18 @@ __device__ __forceinline__ R conv_deriv(const R* v, N neg, const_t<R> eps, bool 
     const R ep = eps + p * p, eq = eps + q * q, es = eps + s * s;
     const R A = ep * ep, B = eq * eq, C = es * es;
     const R d1 = B + K<R>(0.5) * C, d0 = B + K<R>(2) * A;
-    R w;
-    if constexpr (std::is_same<R, double>::value) w = fdiv((s - q) * d0 + (q - p) * d1, d1 * d0);
-    else w = R(s - q) * frcp(d1) + R(q - p) * frcp(d0);
-    const R r = q + R(K<R>(0.5) * B) * w;
+    const R hB = K<R>(0.5) * B;
+    R r;
+    if constexpr (std::is_same<R, double>::value) {
+        r = q + hB * fdiv((s - q) * d0 + (q - p) * d1, d1 * d0);
+    } else if constexpr (std::is_same<R, float>::value || std::is_same<R, F2>::value) {
+        r = q + hB * R(R(s - q) * frcp(d1) + R(q - p) * frcp(d0));
+    } else {
+        // reverse mode: B scales the numerators first, so that the partials of
+        // the divisions stay within 1 / eps^2 (of a reciprocal: 1 / eps^4, beyond
+        // the FP32 tape's range from eps = 1e-10 down)
+        r = q + fdiv(hB * R(s - q), d1) + fdiv(hB * R(q - p), d0);
+    }
     if constexpr (CENTRED) {
         if (any_near) return near ? R(K<R>(0.5) * R(d - b)) : r;
     }

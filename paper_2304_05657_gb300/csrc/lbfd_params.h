@@ -17,6 +17,10 @@ namespace lbfd {
 
 constexpr int NSP = 5;  // species count the kernels are built for
 
+// the least WENO3 epsilons: the weights hold eps^2 (FP32) and eps^4 (FP64),
+// kept in range (far below the squared resolution of any field)
+constexpr double WENO_EPS_LOW_FP32 = 1e-18, WENO_EPS_LOW_FP64 = 1e-75;
+
 template <typename R>
 struct StepParams {
     int dim, nx, ny, nz;
