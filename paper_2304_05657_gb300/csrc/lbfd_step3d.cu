@@ -1,4 +1,5 @@
 // lbfd_step3d.cu -- launchers of the 3-D (D3Q27) tile kernels.
+#include <algorithm>
 #include <cmath>
 
 #include "lbfd_internal.h"
@@ -30,7 +31,9 @@ static int planes_per_block(bool fp64, long long columns, int nz, int zmax)
     const double* us = fp64 ? us64 : us32;
     const int R = fp64 ? 2 : 4;
     const double steady = fp64 ? 109.0 : 8.4, sms = 152.0, fill = 4 * 0.2;
-    const int top = nz < zmax ? nz : zmax, low = top < 4 ? top : 4;  // (fewer than 4 measured slower)
+    // (fewer than 4 measured slower; and a grid has at most 65535 pieces)
+    const int top = nz < zmax ? nz : zmax, enough = (nz + 65534) / 65535;
+    const int low = std::min(top, std::max(4, enough));
     double cost[64], least = 1e300;
     for (int z = low; z <= top; ++z) {
         const double n = (double)columns * nz / z / sms;  // blocks per SM
