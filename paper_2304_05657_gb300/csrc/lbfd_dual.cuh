@@ -144,7 +144,11 @@ __host__ __device__ inline Dual<T, N> operator/(const Dual<T, N>& a, const Dual<
     Dual<T, N> r;
     const T inv = T(1) / b.v;
     r.v = a.v * inv;
-    Vec<T, N>::comb(r.d, inv, a.d, -r.v * inv, b.d);
+    // (a' - r b') / b: the terms cancel before the last rounding
+#pragma unroll
+    for (int k = 0; k < N; ++k) r.d[k] = a.d[k];
+    Vec<T, N>::axpy(r.d, -r.v, b.d);
+    Vec<T, N>::scale(r.d, inv, r.d);
     return r;
 }
 template <typename T, int N>
