@@ -164,20 +164,17 @@ cudaError_t launch_step(int dim, int precision, int variant, const StepParams<do
     return launch_general<3, float, float>(Pf, in, out, solid, stream);
 }
 
-void wall_codes(int nx, int ny, int nz, const int* bc, const uint8_t* solid, const std::vector<long long>& cells,
+void wall_codes(int nx, int ny, int nz, const int*, const uint8_t* solid, const std::vector<long long>& cells,
                 std::vector<unsigned long long>& out)
 {
     // every neighbour within reach of a listed cell is inside the domain up
     // to periodic wrap (the list leaves out the cells near other faces)
-    const int n[3] = {nx, ny, nz};
     auto at = [&](int x, int y, int z) {
         x = ((x % nx) + nx) % nx;
         y = ((y % ny) + ny) % ny;
         z = ((z % nz) + nz) % nz;
         return solid[(long long)x + (long long)nx * ((long long)y + (long long)ny * z)] != 0;
     };
-    (void)bc;
-    (void)n;
     out.resize(cells.size());
     for (size_t t = 0; t < cells.size(); ++t) {
         const long long c = cells[t];
