@@ -237,9 +237,11 @@ int lbfd_set_wait_limit(lbfd_handle* h, long long ns);
  * in-domain solids and for those near inlet and outlet faces of one axis.
  * The lists are made at create.  The general form takes the
  * others, and every listed cell when the walls are curved.  2-D grids too
- * small to fill the GPU with a variant's tiles (up to 155 648 cells in FP32,
- * 622 592 in FP64, staircase walls) run as one launch of small tiles and the
- * cells they leave out, whatever the variant (except 0).  With omega_hi = 1 the
+ * small to fill the GPU with a variant's tiles (staircase walls, no cell that
+ * needs the general form) run as one launch of small tiles and the cells they
+ * leave out: variant 1 up to 58 368 cells in FP32 and 252 928 in FP64 (as
+ * warps of 8x4 cells: 1 824 and 7 904), the others but 0 up to 19 456 (608
+ * warps).  With omega_hi = 1 the
  * collision uses the moments of orders 0-2 of the populations alone (the
  * relaxation sets the higher cumulants to equilibrium).  All variants
  * compute the same step up to rounding order.  Default: 1 (0 for
@@ -257,7 +259,8 @@ int lbfd_launches_per_step(const lbfd_handle* h);
 /* Autotuner: time every variant over `reps` launches on the current state
  * (the output buffer is overwritten, the state does not advance), select
  * the fastest and return it in *best; ms_per_variant (may be NULL) gets
- * lbfd_num_variants(h) mean launch times [ms].  Synchronises. */
+ * lbfd_num_variants(h) mean launch times [ms] (variants that launch the same
+ * kernels are timed once and share the time).  Synchronises. */
 int lbfd_autotune(lbfd_handle* h, int reps, double* ms_per_variant, int* best);
 
 /* Copy one field (LBFD_FIELD_*) of all N cells to host FP64 out[N].

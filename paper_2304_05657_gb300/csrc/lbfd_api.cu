@@ -364,7 +364,16 @@ lbfd::BoundaryLists lists(const lbfd_handle* h)
 bool runs_small(const lbfd_handle* h, int v, const lbfd::BoundaryLists& b)
 {
     return h->dim == 2 && v > 0 && !is_tangent(h->precision) && !h->Pd.curved &&
-           lbfd::small2d_applies(h->precision, h->grid.nx, h->grid.ny, b);
+           lbfd::small2d_applies(h->precision, v, h->grid.nx, h->grid.ny, b);
+}
+
+// The first variant that launches the same kernels as variant v: the 2-D ones
+// that the small form stands for, and 3-D variant 3, which differs from 1
+// only in FP32 with omega_hi != 1 (launch_3d_tiles)
+int same_as(const lbfd_handle* h, int v)
+{
+    if (h->dim == 2) return v > 1 && runs_small(h, v, lists(h)) ? 1 : v;
+    return v == 3 && (h->precision == LBFD_FP64 || h->Pf.omega_hi == 1.f) ? 1 : v;
 }
 
 // one FP64 or mixed step with kernel variant v
@@ -895,6 +904,11 @@ int lbfd_autotune(lbfd_handle* h, int reps, double* ms_per_variant, int* best)
     int arg = h->variant;
     float best_ms = 3.4e38f;
     for (int v = 0; v < nv; ++v) {
+        const int twin = same_as(h, v);
+        if (twin < v) {  // timed already
+            if (ms_per_variant) ms_per_variant[v] = ms_per_variant[twin];
+            continue;
+        }
         // the input buffer is never written: the state does not advance
         cudaError_t e = cudaSuccess;
         for (int r = 0; r < 2 && e == cudaSuccess; ++r)

@@ -92,9 +92,9 @@ cudaError_t launch_step(int dim, int precision, int variant, const StepParams<do
 int num_variants(int dim);
 
 // One launch for a whole 2-D step on a grid too small to fill the GPU with
-// the tiles of the variants (lbfd_step_small.cu): whether it applies (a rule
-// on the grid and the precision), and the launch.
-bool small2d_applies(int precision, int nx, int ny, const BoundaryLists& b);
+// the tiles of the variants (lbfd_step_small.cu): whether it stands for a
+// variant (a rule on the grid, the precision and the variant), and the launch.
+bool small2d_applies(int precision, int variant, int nx, int ny, const BoundaryLists& b);
 cudaError_t launch_step_small2d(int precision, const StepParams<double>& Pd, const StepParams<float>& Pf, StateView in,
                                 StateView out, const BoundaryLists& b, cudaStream_t stream);
 

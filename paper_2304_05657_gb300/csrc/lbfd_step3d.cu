@@ -149,7 +149,8 @@ static cudaError_t launch_3d_tiles(int variant, const StepParams<R>& P, StateVie
     switch (variant) {
     case 1: return launch_t3<HI1, S, R, MINB>(16, true, P, in, out, solid, b, side, stream);
     case 2: return launch_t3<HI1, S, R, MINB>(32, true, P, in, out, solid, b, side, stream);
-    // variant 3: as 1 with the registers capped for four blocks per SM (FP32)
+    // variant 3: FP32 with omega_hi != 1 at four blocks per SM (128 registers)
+    // instead of three; elsewhere the same as 1
     case 3: return launch_t3<HI1, S, R, sizeof(R) == 4 ? 4 : 2>(16, true, P, in, out, solid, b, side, stream);
     // variants 4, 5: as 1, 2 split into an FD tile kernel and a collision kernel
     case 4: return launch_t3<HI1, S, R, MINB, true>(16, false, P, in, out, solid, b, side, stream);

@@ -4,23 +4,32 @@
 
 namespace lbfd {
 
-// The rule, in warps of 32 cells against the 608 SM partitions of the GPU
-// (us per step of an isothermal channel in a graph; big = the best of the
-// variants' tiles):
-//   FP32 cells     8192  12288  32768  65536  98304 131072 196608 262144
-//     two lanes     4.8    5.0    6.1    9.2   11.2   13.8   18.7   23.6
-//     one lane      5.0    5.0    5.4    6.9    9.8   10.8   14.6   17.4
-//     big           6.7    7.1    7.2    9.6    9.4   11.5   12.4   15.9
-//   FP64 cells     4096   8192  12288  16384  32768  98304 262144
-//     two lanes    25.6   27.8   35.8   40.4   85.7    221    536
-//     one lane     35.8   35.5   35.7   38.0   58.6    183    415
-//     big          36.5   36.5   36.5   36.5   65.4    178    408
-// Two lanes per cell as long as that leaves the partitions at most one warp
-// each.  One lane per cell up to 8 warps (FP32; beyond, the larger tiles'
-// smaller halo and the packed pairs win) or 32 (FP64; beyond, the halo).
-bool small2d_applies(int precision, int nx, int ny, const BoundaryLists& b)
+// The rules, in warps of 32 cells against the 608 SM partitions of the GPU
+// (us per step of an isothermal channel in a graph).  Lanes per cell: two as
+// long as that leaves the partitions at most one warp each.
+//   FP32 cells     8192  12288  32768    FP64 cells     4096   8192  12288  16384
+//     two lanes     4.8    5.0    6.1      two lanes    25.6   27.8   35.8   40.4
+//     one lane      5.0    5.0    5.4      one lane     35.8   35.5   35.7   38.0
+// Against the tiles of variants 1 (32x8) and 2 (32x4):
+//   FP32 cells   8192 16384 32768 49152 57344 65536 73728 81920 98304 155648
+//     small       4.6   5.0   5.4   6.2   6.4   7.0   6.9   7.6   9.8   12.1
+//     variant 1   4.9   5.2   5.2   6.2   6.4   6.6   6.2   7.7   7.8    9.6
+//     variant 2   4.7   4.9   5.5   5.8   5.9   6.5   6.4   7.1   7.8    9.9
+//   FP64 cells  24576 32768 40960 49152 65536 73728 81920 98304 131072 163840 204800 245760 262144 409600
+//     small        52    59    76    87   126   151   154   184    213    272    330    389    417    649
+//     variant 1    65    65   122   122   127   122   180   179    236    297    350    407    410    635
+//     variant 2    64    67    92    95   127   124   151   180    210    268    326    384    413    638
+// Variant 1 (the default) is the small form up to 3 warps a partition in FP32
+// (from there on its own tiles are no slower) and 13 in FP64, where its
+// 256-thread blocks fill the last wave badly: the small form is up to 37 %
+// faster and, but for about 4 warps a partition, at most 3 % slower.  The
+// other variants are the small form only up to one warp a partition, where
+// their tiles leave partitions idle; beyond, each runs its own, so that the
+// autotuner has them and the small form (as variant 1) to choose from.
+bool small2d_applies(int precision, int variant, int nx, int ny, const BoundaryLists& b)
 {
-    return b.all2.nrest == 0 && small_warps(nx, ny) <= PARTITIONS * (precision == 0 ? 32 : 8);
+    const long long per_partition = variant > 1 ? 1 : (precision == 0 ? 13 : 3);
+    return b.all2.nrest == 0 && small_warps(nx, ny) <= PARTITIONS * per_partition;
 }
 
 cudaError_t launch_step_small2d(int precision, const StepParams<double>& Pd, const StepParams<float>& Pf, StateView in,
