@@ -367,13 +367,17 @@ bool runs_small(const lbfd_handle* h, int v, const lbfd::BoundaryLists& b)
            lbfd::small2d_applies(h->precision, v, h->grid.nx, h->grid.ny, b);
 }
 
-// The first variant that launches the same kernels as variant v: the 2-D ones
-// that the small form stands for, and 3-D variant 3, which differs from 1
+// The first variant that launches the same kernels as variant v: of the 2-D
+// ones that the small form stands for, and 3-D variant 3, which differs from 1
 // only in FP32 with omega_hi != 1 (launch_3d_tiles)
 int same_as(const lbfd_handle* h, int v)
 {
-    if (h->dim == 2) return v > 1 && runs_small(h, v, lists(h)) ? 1 : v;
-    return v == 3 && (h->precision == LBFD_FP64 || h->Pf.omega_hi == 1.f) ? 1 : v;
+    if (h->dim == 3) return v == 3 && (h->precision == LBFD_FP64 || h->Pf.omega_hi == 1.f) ? 1 : v;
+    const lbfd::BoundaryLists b = lists(h);
+    int first = v;
+    for (int w = v - 1; w > 0; --w)
+        if (runs_small(h, v, b) && runs_small(h, w, b)) first = w;
+    return first;
 }
 
 // one FP64 or mixed step with kernel variant v

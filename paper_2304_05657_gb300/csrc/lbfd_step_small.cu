@@ -22,14 +22,19 @@ namespace lbfd {
 // Variant 1 (the default) is the small form up to 3 warps a partition in FP32
 // (from there on its own tiles are no slower) and 13 in FP64, where its
 // 256-thread blocks fill the last wave badly: the small form is up to 37 %
-// faster and, but for about 4 warps a partition, at most 3 % slower.  The
-// other variants are the small form only up to one warp a partition, where
-// their tiles leave partitions idle; beyond, each runs its own, so that the
-// autotuner has them and the small form (as variant 1) to choose from.
+// faster and, but for about 4 warps a partition, at most 3 % slower.  Variants
+// 2-4 (coded tiles, one launch like it) run their own tiles beyond one warp a
+// partition, so that the autotuner has both to choose from.  Variants 5-12 (a
+// list beside the tiles) are slower than either up to 8 warps a partition in
+// FP32 (98304 cells 11.6-13.8 us, 155648 13.5-14.5) and mostly in FP64 (32768
+// cells 105-126, 131072 230-260, 196608 319-350, 262144 423), where they take
+// 60 or 115 us on 32768 cells by the order in which the two kernels' blocks are
+// placed: a few timed launches do not tell.  Up to 8 and 13 warps they are the
+// small form.
 bool small2d_applies(int precision, int variant, int nx, int ny, const BoundaryLists& b)
 {
-    const long long per_partition = variant > 1 ? 1 : (precision == 0 ? 13 : 3);
-    return b.all2.nrest == 0 && small_warps(nx, ny) <= PARTITIONS * per_partition;
+    const long long fp32 = variant == 1 ? 3 : (variant < 5 ? 1 : 8), fp64 = variant > 1 && variant < 5 ? 1 : 13;
+    return b.all2.nrest == 0 && small_warps(nx, ny) <= PARTITIONS * (precision == 0 ? fp64 : fp32);
 }
 
 cudaError_t launch_step_small2d(int precision, const StepParams<double>& Pd, const StepParams<float>& Pf, StateView in,
