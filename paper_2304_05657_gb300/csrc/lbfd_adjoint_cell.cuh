@@ -1,7 +1,8 @@
 // lbfd_adjoint_cell.cuh -- hand-derived local adjoints of the D2Q9 step in
 // FP64: the WENO3 derivative's weights and the transpose of the collision
-// with omega_hi = 1.  Plain arithmetic, for host and device (the CPU test
-// compares them with central differences of the forward forms).
+// with omega_hi = 1.  Plain arithmetic, for host and device: the CPU test
+// (tests/test_adjoint_cell_host.py) compares them with central differences of
+// the forward forms.
 #pragma once
 #include "lbfd_device.cuh"
 

@@ -23,7 +23,8 @@ namespace lbfd {
 // x (1 + e + e^2) with e = 1 - b x, whose remaining error e^3 is below the
 // rounding: within 1 ulp of 1/b (tests/test_gpu_reciprocal.py) for three
 // FP64 instructions, where an IEEE division takes about ten (and the pipe
-// issues one per 64 cycles and SM partition).
+// issues one per 64 cycles and SM partition).  A zero, subnormal or infinite
+// divisor gives NaN, where a division would give inf or 0.
 __device__ __forceinline__ float frcp(float b)
 {
     float r;
@@ -282,10 +283,10 @@ __device__ __forceinline__ R upwind_sel(bool neg, const R& a, const R& b)
 // the reconstruction with weights 1/3 : 2/3 over the smoothness, rearranged
 // so that no face value is formed and every weight enters once (17 FP32
 // instructions and two reciprocals, against 31 and two divisions for the
-// two faces).  Plain FP64 takes one division for both terms (its pipe issues
-// one warp instruction per 16 cycles and SM, a division is about nine);
-// there the product of two smoothness squares cannot leave the range, in
-// FP32 it can.  CENTRED: `near` selects the centred 2nd-order derivative
+// two faces).  Plain FP64 takes one reciprocal (three instructions) for both
+// terms, eight instructions where two take nine; there the product of two
+// smoothness squares cannot leave the range, in FP32 it can.  CENTRED: `near`
+// selects the centred 2nd-order derivative
 // (any_near: false, uniformly over the warp, when no lane does).
 template <bool CENTRED, typename R, typename N>
 __device__ __forceinline__ R conv_deriv(const R* v, N neg, const_t<R> eps, bool near, bool any_near)

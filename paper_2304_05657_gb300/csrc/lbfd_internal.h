@@ -98,7 +98,7 @@ bool small2d_applies(int precision, int variant, int nx, int ny, const BoundaryL
 cudaError_t launch_step_small2d(int precision, const StepParams<double>& Pd, const StepParams<float>& Pf, StateView in,
                                 StateView out, const BoundaryLists& b, cudaStream_t stream);
 
-// 3-D tile kernels (variants 1..2 in 3-D), lbfd_step3d.cu
+// 3-D tile kernels (variants 1..7 in 3-D), lbfd_step3d.cu
 cudaError_t launch_step3d_tiled(int precision, int variant, const StepParams<double>& Pd, const StepParams<float>& Pf,
                                 StateView in, StateView out, const uint8_t* solid, const BoundaryLists& b,
                                 const SideStream& side, cudaStream_t stream);
@@ -122,7 +122,8 @@ void list_codes2d(int nx, int ny, const int* bc, const uint8_t* solid, const std
                   std::vector<long long>& coded, std::vector<unsigned long long>& codes, std::vector<long long>& rest);
 
 // Fluid cells that are not interior for the tile kernels (host, at create);
-// faces_only (3-D): only cells whose stencil leaves the domain.
+// faces_only (3-D): only cells whose stencil leaves the domain.  (The last
+// argument, and the face types of wall_codes, are not used.)
 void boundary_cells(int dim, int nx, int ny, int nz, const int* bc, const uint8_t* solid, std::vector<long long>& out,
                     bool faces_only, const int* = nullptr);
 

@@ -21,10 +21,12 @@ struct Tile3Shape {
 // modelled from the measured us per plane of 1 .. R blocks sharing an SM (R
 // resident): blocks in rounds of R on the fullest SM, or, with many rounds,
 // the steady rate and half a round of tail.  Measured us per step over z:
-//   128x64x64 FP32:   4: 91   7: 85   8: 94  16: 140  32: 209  64: 405
-//   256x128x128 FP32: 4: 517  8: 504 11: 493 16: 531  32: 598  64: 694
-//   101x53x47 FP64:   4: 945  8: 939 16: 1049 32: 2085
-//   128x64x64 FP64:   5: 1686 7: 1647 8: 1861 16: 1989 32: 2099
+//   128x64x64 FP32:   4: 91   7: 85   8: 94   9: 100  16: 139   (picks 7)
+//   256x128x128 FP32: 4: 511  5: 496  7: 494  8: 500  11: 490  16: 527   (5)
+//   101x53x47 FP64:   4: 941  5: 1087 7: 1143 8: 941  9: 1057  16: 1049   (8)
+//   128x64x64 FP64:   4: 1714 5: 1680 7: 1646 8: 1859 9: 1978  16: 1985   (9)
+// The last pick is the model's error: three FP64 blocks on an SM that holds two
+// take about 194 us a plane, not 109 + 63.
 static int planes_per_block(bool fp64, long long columns, int nz, int zmax)
 {
     static const double us32[] = {0.0, 6.4, 7.9, 9.4, 10.9}, us64[] = {0.0, 63.0, 109.0};
@@ -65,6 +67,8 @@ static int planes_per_block(bool fp64, long long columns, int nz, int zmax)
 // Otherwise the tile kernel updates the coded cells too, next to in-domain
 // solids and (faces) near inlet and outlet faces; with curved walls both
 // go through the general form.
+// zmax: the most planes per block; the variants that differ only in it (16 or
+// 32) are one kernel where the rule stays below 16.
 // MINB: resident blocks per SM.  FP32: four (128 registers) when the
 // collision needs only the low moments, else three; FP64: two.
 template <bool HI1, typename S, typename R, int MINB, bool SPLIT = false>
