@@ -67,8 +67,9 @@ static int planes_per_block(bool fp64, long long columns, int nz, int zmax)
 // Otherwise the tile kernel updates the coded cells too, next to in-domain
 // solids and (faces) near inlet and outlet faces; with curved walls both
 // go through the general form.
-// zmax: the most planes per block; the variants that differ only in it (16 or
-// 32) are one kernel where the rule stays below 16.
+// zmax: the most planes per block; variants that differ only in it (16 or 32)
+// are one kernel with the same or, on large grids, a few more planes
+// (512x256x256 FP32: 10 and 11).
 // MINB: resident blocks per SM.  FP32: four (128 registers) when the
 // collision needs only the low moments, else three; FP64: two.
 template <bool HI1, typename S, typename R, int MINB, bool SPLIT = false>
