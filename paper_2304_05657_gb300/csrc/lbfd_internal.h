@@ -247,8 +247,9 @@ cudaError_t launch_step_persistent(int precision, const StepParams<double>& Pd, 
 
 // Number of words of the reduction scratch.
 constexpr int RED_WORDS = 16;
-// Blocks of the diagnostics reduction (eight 256-thread blocks per SM), and
+// Blocks of the diagnostics reduction (four 256-thread blocks per SM, all
+// resident: twice as many would take two rounds and twice the sums to join), and
 // the words of their sums.
-constexpr int DIAG_BLOCKS = 152 * 8, DIAG_WORDS = 8 * DIAG_BLOCKS;
+constexpr int DIAG_BLOCKS = 152 * 4, DIAG_WORDS = 8 * DIAG_BLOCKS;
 
 }  // namespace lbfd

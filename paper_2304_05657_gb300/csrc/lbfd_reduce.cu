@@ -99,7 +99,9 @@ __device__ void centreline(const StepParams<double>& P, const S* __restrict__ T,
 // stored there and the last block adds them in block order, so that the
 // result does not depend on the order in which blocks finish; without it
 // (the fixed scratch of the allocation-free form) they are added to `red`
-// atomically.  The last block also scans the centre line: one launch.
+// atomically.  Block 0 scans the centre line meanwhile (a serial chain of FP64
+// work on one SM: after the sums it would add 10 to 20 us where nx is 1024 and
+// more); the others take the sums: one launch.
 template <int DIM, typename S>
 __global__ void __launch_bounds__(256) diag_kernel(StepParams<double> P, const S* __restrict__ g,
                                                    const S* __restrict__ T, const S* __restrict__ Y,
@@ -107,12 +109,17 @@ __global__ void __launch_bounds__(256) diag_kernel(StepParams<double> P, const S
                                                    double* part)
 {
     constexpr int Q = DIM == 2 ? 9 : 27;
+    if (blockIdx.x == 0) {
+        centreline<DIM, S>(P, T, Y, solid, y0, y1, red);
+        return;
+    }
+    const unsigned nsum = gridDim.x - 1, self = blockIdx.x - 1;
     double s[4] = {0.0, 0.0, 0.0, 0.0};
     unsigned long long tkey = 0ull, nonf = 0ull, nfl = 0ull, sec = 0ull;
-    const long long stride = (long long)gridDim.x * blockDim.x;
+    const long long stride = (long long)nsum * blockDim.x;
     const int rows = y1 - y0;
     const long long ncount = (long long)P.nx * rows * P.nz;  // cells with y0 <= y < y1
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < ncount; t += stride) {
+    for (long long t = (long long)self * blockDim.x + threadIdx.x; t < ncount; t += stride) {
         const long long r = t / P.nx;
         const long long c = t % P.nx + (long long)P.nx * (y0 + r % rows + (long long)P.ny * (r / rows));
         if (solid[c]) continue;
@@ -176,7 +183,7 @@ __global__ void __launch_bounds__(256) diag_kernel(StepParams<double> P, const S
         }
         unsigned long long* ru = reinterpret_cast<unsigned long long*>(red);
         if (part) {
-            double* pb = part + 8 * (size_t)blockIdx.x;
+            double* pb = part + 8 * (size_t)self;
             unsigned long long* pu = reinterpret_cast<unsigned long long*>(pb);
             for (int j = 0; j < 4; ++j) pb[j] = s[j];
             pu[4] = tkey;
@@ -191,17 +198,17 @@ __global__ void __launch_bounds__(256) diag_kernel(StepParams<double> P, const S
             atomicAdd(&ru[7], sec);
         }
         __threadfence();  // this block's sums before its count
-        last = atomicInc(reinterpret_cast<unsigned*>(&red[10]), gridDim.x - 1) == gridDim.x - 1;
+        last = atomicInc(reinterpret_cast<unsigned*>(&red[10]), nsum - 1) == nsum - 1;
     }
     __syncthreads();
-    if (!last) return;
+    if (!last || !part) return;
     __threadfence();
-    if (part) {
+    {
         // word j = thread % 8 of a run of consecutive blocks per thread, the 32
         // runs then joined in order
         __shared__ unsigned long long run[32][8];
         const int j = threadIdx.x & 7, r = threadIdx.x >> 3;
-        const unsigned len = (gridDim.x + 31) / 32;
+        const unsigned len = (nsum + 31) / 32;
         const unsigned long long* pu = reinterpret_cast<const unsigned long long*>(part) + j;
         auto join = [&](double& d, unsigned long long& u, unsigned long long w) {
             if (j < 4) d += __longlong_as_double((long long)w);
@@ -210,10 +217,10 @@ __global__ void __launch_bounds__(256) diag_kernel(StepParams<double> P, const S
         };
         double d = 0.0;
         unsigned long long u = 0ull;
-#pragma unroll 8
+#pragma unroll 10
         for (unsigned k = 0; k < len; ++k) {
             const unsigned b = r * len + k;
-            if (b < gridDim.x) join(d, u, __ldcg(pu + 8 * (size_t)b));
+            if (b < nsum) join(d, u, __ldcg(pu + 8 * (size_t)b));
         }
         run[r][j] = j < 4 ? (unsigned long long)__double_as_longlong(d) : u;
         __syncthreads();
@@ -224,7 +231,6 @@ __global__ void __launch_bounds__(256) diag_kernel(StepParams<double> P, const S
             reinterpret_cast<unsigned long long*>(red)[j] = j < 4 ? (unsigned long long)__double_as_longlong(d) : u;
         }
     }
-    centreline<DIM, S>(P, T, Y, solid, y0, y1, red);
 }
 
 template <int DIM, typename S>
@@ -236,7 +242,7 @@ static cudaError_t diag_launch(const StepParams<double>& P, StateView st, const 
         if (e != cudaSuccess) return e;
     }
     const long long want = ((long long)P.nx * (y1 - y0) * P.nz + 255) / 256;
-    const unsigned blocks = (unsigned)(want < DIAG_BLOCKS ? want : DIAG_BLOCKS);
+    const unsigned blocks = (unsigned)(want < DIAG_BLOCKS ? want : DIAG_BLOCKS) + 1;  // and the centre line's
     diag_kernel<DIM, S><<<blocks, 256, 0, stream>>>(P, (const S*)st.g, (const S*)st.T, (const S*)st.Y, solid, y0, y1,
                                                     red, part);
     return cudaGetLastError();
