@@ -239,9 +239,9 @@ int lbfd_set_wait_limit(lbfd_handle* h, long long ns);
  * others, and every listed cell when the walls are curved.  2-D grids too
  * small to fill the GPU with a variant's tiles (staircase walls, no cell that
  * needs the general form) run as one launch of small tiles and the cells they
- * leave out: in FP32 variant 1 up to 58 368 cells (as 1 824 warps of 8x4 cells),
- * 2..4 up to 19 456 (608) and 5..12 up to 155 648 (4 864); in FP64 2..4 up to
- * 19 456 and the others up to 252 928 (7 904).  With omega_hi = 1 the
+ * leave out, up to 155 648 cells in FP32 (as 4 864 warps of 8x4 cells) and
+ * 622 592 in FP64 (19 456 warps); 2..4, where their tiles leave no cell to a
+ * list, up to 19 456 (608) only.  With omega_hi = 1 the
  * collision uses the moments of orders 0-2 of the populations alone (the
  * relaxation sets the higher cumulants to equilibrium).  All variants
  * compute the same step up to rounding order.  Default: 1 (0 for

@@ -19,22 +19,21 @@ namespace lbfd {
 //     small        52    59    76    87   126   151   154   184    213    272    330    389    417    649
 //     variant 1    65    65   122   122   127   122   180   179    236    297    350    407    410    635
 //     variant 2    64    67    92    95   127   124   151   180    210    268    326    384    413    638
-// Variant 1 (the default) is the small form up to 3 warps a partition in FP32
-// (from there on its own tiles are no slower) and 13 in FP64, where its
-// 256-thread blocks fill the last wave badly: the small form is up to 37 %
-// faster and, but for about 4 warps a partition, at most 3 % slower.  Variants
-// 2-4 (coded tiles, one launch like it) run their own tiles beyond one warp a
-// partition, so that the autotuner has both to choose from.  Variants 5-12 (a
-// list beside the tiles) are slower than either up to 8 warps a partition in
-// FP32 (98304 cells 11.6-13.8 us, 155648 13.5-14.5) and mostly in FP64 (32768
-// cells 105-126, 131072 230-260, 196608 319-350, 262144 423), where they take
-// 60 or 115 us on 32768 cells by the order in which the two kernels' blocks are
-// placed: a few timed launches do not tell.  Up to 8 and 13 warps they are the
-// small form.
+// and with many cells next to walls (us per pass): 86 271 cells of channels
+// between solid rows, FP32, 24 steps: small 268, variant 1 300; 522 880 cells of
+// a burner, FP64, 4 steps: 3 359, 3 646.  No one line is right for both kinds, so
+// variants 2-4 run their own tiles beyond one warp a partition where these are
+// one launch too (no cell for a list): with variant 1, the default, as the small
+// form the autotuner has both to choose from.  Variant 1 and 5-12 (a list beside
+// the tiles) are the small form up to 8 warps a partition in FP32 and 32 in FP64.
+// There 5-12 are slower in FP32 (98304 cells 11.6-13.8 us, 155648 13.5-14.5) and
+// mostly in FP64 (131072 cells 230-260, 196608 319-350, 262144 423), where they
+// take 60 or 115 us on 32768 cells by the order in which the two kernels' blocks
+// are placed: a few timed launches do not tell.
 bool small2d_applies(int precision, int variant, int nx, int ny, const BoundaryLists& b)
 {
-    const long long fp32 = variant == 1 ? 3 : (variant < 5 ? 1 : 8), fp64 = variant > 1 && variant < 5 ? 1 : 13;
-    return b.all2.nrest == 0 && small_warps(nx, ny) <= PARTITIONS * (precision == 0 ? fp64 : fp32);
+    const bool own = variant >= 2 && variant <= 4 && b.all2.nout == 0;
+    return b.all2.nrest == 0 && small_warps(nx, ny) <= PARTITIONS * (own ? 1 : (precision == 0 ? 32 : 8));
 }
 
 cudaError_t launch_step_small2d(int precision, const StepParams<double>& Pd, const StepParams<float>& Pf, StateView in,

@@ -1,6 +1,6 @@
 """Each 2-D variant's own kernels on grids beyond the small form's lines (in
-FP32 4 864 warps of 8x4 cells, FP64 608 for variants 2-4), where the variants are
-not one kernel: the packed pairs (9-12) with even nx over 1 000 steps and with odd
+FP32 4 864 warps of 8x4 cells, and 608 for variants 2-4 in both), where the variants
+are not one kernel: the packed pairs (9-12) with even nx over 1 000 steps and with odd
 nx over 200, every variant over 60, and the persistent step against the variant
 whose tiles it runs.  Bars of
 the parity tests: mixed T and Y 1e-5 relative L2, populations 1e-4 of their
