@@ -54,5 +54,6 @@ def test_autotune_times_each_kernel_once(lbfd_lib, nx, ny, shared):
     assert np.all(ms > 0) and ms[best] == ms.min() and s.variant == best
     assert len({ms[v] for v in shared}) <= 1
     # the others are timed by themselves (events resolve 32 ns: some tie)
-    assert len({ms[v] for v in range(13) if v not in shared}) > 1
+    others = [ms[v] for v in range(13) if v not in shared]
+    assert len(others) == 1 or len(set(others)) > 1
     check(s, "mixed", (T, Y, g), (0, 1, 2, 3, 4, 6, 9))
